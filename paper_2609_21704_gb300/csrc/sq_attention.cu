@@ -16,13 +16,9 @@
 // output rows [B*T, Hq D].  Token t of sequence b sits at position
 // pos0[b] + t.
 //
-// Attention is split over 32-key chunks of the cache (one CTA per
-// (sequence, key/value head, chunk)): all G * T queries of the group read
-// the chunk once from shared memory, then a combine kernel merges the
-// chunks' (max, sum, weighted value) partials.  Bound: the cache bytes
-// (2 * pos * Hkv * D * 2 per sequence) and, for long query groups, CUDA-core
-// arithmetic (G * T * 2 D flops per cached key).
 #include <math.h>
+
+#include <mutex>
 
 #include "sq_decoder.h"
 
@@ -31,9 +27,8 @@ namespace sq {
 __device__ unsigned int g_attn_status;
 
 constexpr int kHeadDim = 128;
-constexpr int kAttnChunk = 32;      // cache positions per CTA
-constexpr int kAttnThreads = 256;
-constexpr int kRowPad = kHeadDim + 4;  // fp32 row stride in shared memory (16-byte rows, fewer conflicts)
+constexpr int kAttnWarps = 4;
+constexpr int kAttnThreads = 32 * kAttnWarps;
 constexpr int kMaxT = 32;           // new tokens per sequence and call
 // Per-query partial record in the workspace: (max, sum, 2 unused, o[D]):
 // 132 floats = 528 bytes, so records and their o[] stay 16-byte aligned.
@@ -81,21 +76,27 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const __half* __restrict__
 }
 
 // ---- RoPE --------------------------------------------------------------------
-// Inverse frequencies theta^(-2d/D), d < D/2, computed on the host in fp64.
+// Inverse frequencies theta^(-2d/D), d < D/2, as turns per position in units
+// of 2^-64 of a turn: pos * f modulo 2^64 is the angle modulo 2 pi without
+// any fp64 arithmetic (two fp64 operations per clock and SM on this GPU: the
+// T positions' table cost 2 us per CTA at T = 28).  f comes from fp64, so
+// positions up to 2^17 keep the angle within 1e-10, as an fp64 reduction would.
 struct RopeFreq {
-  double f[kHeadDim / 2];
+  unsigned long long f[kHeadDim / 2];
 };
 
-// cos and sin of pos * f: the angle and its reduction modulo 2 pi in fp64
-// (positions up to 2^20 keep the reduced angle within ~1e-10), then fp32
-// sincosf of the reduced angle.
-__device__ __forceinline__ float2 rope_cs(int pos, double f) {
-  const double a = (double)pos * f;
-  const double k = rint(a * 0.15915494309189535);       // a / (2 pi)
-  double r = fma(-k, 6.283185307179586, a);              // 2 pi, head
-  r = fma(-k, 2.4492935982947064e-16, r);                 // 2 pi, tail
+// cos and sin of the angle at `pos`: the turn as a signed fraction a + b of
+// 2^64 (24 leading bits, and the rest), times 2 pi in fp32 (head and tail of
+// the constant, one rounding of the angle), then fp32 sincosf.
+__device__ __forceinline__ float2 rope_cs(int pos, unsigned long long f) {
+  const long long turn = (long long)((unsigned long long)(long long)pos * f);
+  const float a = __ll2float_rz(turn);
+  const float b = __ll2float_rn(turn - __float2ll_rz(a));
+  // 2 pi 2^-64 = head + tail
+  const float head = 0x1.921fb6p-62f, tail = -0x1.777a5cp-87f;
+  const float r = fmaf(a, head, fmaf(a, tail, b * head));
   float s, c;
-  sincosf((float)r, &s, &c);
+  sincosf(r, &s, &c);
   return make_float2(c, s);
 }
 
@@ -136,211 +137,504 @@ __global__ void __launch_bounds__(64) kv_append_kernel(const __half* __restrict_
 }
 
 // ---- attention ----------------------------------------------------------------
-__device__ __forceinline__ float h2f_lo(uint32_t w) { return __half2float(__ushort_as_half((uint16_t)(w & 0xffffu))); }
-__device__ __forceinline__ float h2f_hi(uint32_t w) { return __half2float(__ushort_as_half((uint16_t)(w >> 16))); }
-
 struct AttnArgs {
   const __half* qkv;
   const __half* kc;
   const __half* vc;
   __half* kcw;  // the same caches, written when append != 0
   __half* vcw;
-  int append;   // the new tokens' keys/values are appended by the chunk that holds them
+  int append;   // the new tokens' keys/values are appended by the CTAs that hold them
   const int32_t* pos0;
   __half* out;
-  float* part;  // [(B*Hkv) * nsplit * Q * kPartStride]: per query (m, l, -, -, o[D])
+  float* part;  // [(B*Hkv) * nsplit * Q * kPartStride]: per query (m, l, -, -, o[D]); unused by a cluster
   int B, T, Hq, Hkv, G, Q;
   int64_t max_ctx;
-  int nsplit;
+  int nsplit;   // CTAs sharing one (sequence, key/value head, query group)'s keys
+  int cluster;  // they form a cluster and merge through distributed shared memory
   float scale;  // 1 / sqrt(D)
   RopeFreq rf;
 };
 
-// Shared memory (fp32): cos/sin of the T positions [T][D/2], q [Q][kRowPad]
-// (rotated, scaled), k [C][kRowPad], v [C][kRowPad], scores [Q][C].
-// Queries q = g * T + t (head kvh * G + g, token t).
-__global__ void __launch_bounds__(kAttnThreads) attention_partial_kernel(const AttnArgs a) {
+constexpr int kBlockKeys = 64;                         // keys of one pipeline stage
+constexpr int kStageHalf = kBlockKeys * kHeadDim * 2;  // bytes of a stage's keys (its values follow)
+constexpr float kProbScale = 16384.0f;                 // probabilities enter the product times 2^14
+
+__device__ __forceinline__ void ldsm_x4(uint32_t r[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t r[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void attn_mma(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// 16-byte asynchronous copy; zeros when !in (src is then not read).
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0)
+               : "memory");
+}
+// Byte offset of 16-byte chunk c of row r in a tile of 256-byte rows: chunks
+// are permuted by the row, so the eight rows of a matrix load hit distinct banks.
+__device__ __forceinline__ uint32_t tile_off(int r, int c) { return (uint32_t)(r * 256 + ((c ^ (r & 7)) << 4)); }
+
+// (hi, lo): x = hi + lo to 22 bits and more (hi the nearest fp16; a
+// non-finite hi carries x alone).
+__device__ __forceinline__ void split_f16(float x, __half& hi, __half& lo) {
+  hi = __float2half_rn(x);
+  const float h = __half2float(hi);
+  lo = isfinite(h) ? __float2half_rn(x - h) : __ushort_as_half(0);
+}
+__device__ __forceinline__ uint32_t pack_h2(__half a, __half b) {
+  return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
+}
+
+__device__ __forceinline__ uint32_t attn_rank_addr(const float* local, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void attn_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Shapes of the kernel's instances: WM warps along the queries (the other
+// kAttnWarps / WM split every block of keys), NT tiles of eight queries a warp.
+template <int WM, int NT>
+struct AttnCfg {
+  static constexpr int kWK = kAttnWarps / WM;          // warps along the keys
+  static constexpr int kQT = 8 * WM * NT;              // queries a CTA holds
+  static constexpr int kKeysWarp = kBlockKeys / kWK;   // keys of a block a warp takes
+  static constexpr int kKeysStep = kKeysWarp < 32 ? kKeysWarp : 32;
+  static constexpr int kStages = WM > 1 ? 2 : 3;
+  static constexpr int kMaxTokens = kQT < kMaxT && WM < 4 ? kQT : kMaxT;  // new tokens a launch may have
+  static constexpr int kQBytes = WM * NT * 4096;       // packed query tiles
+  static constexpr int kOffFac = kQBytes;              // per query: factor of its scores
+  static constexpr int kOffStage = kOffFac + (kQT * 4 + 127) / 128 * 128;
+  static constexpr int kOffCs = kOffStage + kStages * 2 * kStageHalf;
+};
+constexpr int attn_smem(int off_cs, int T) { return off_cs + T * (kHeadDim / 2) * 8; }
+
+// One CTA: kQT queries (q = g * T + t: head kvh * G + g, token t) of one
+// (sequence, key/value head) against one contiguous share of its 64-key blocks.
+//
+// Products on mma.sync (fp16 inputs, fp32 sums; tcgen05 would want 128 query
+// rows, these groups have 1 to 200) without giving up fp32 operands: a query
+// (rotated in fp32) is split into two fp16 terms after scaling it by a power
+// of two (its largest value to [2^10, 2^11)), a probability into two fp16
+// terms after scaling by 2^14; keys and values are fp16 already.  An m16 tile
+// holds eight queries: rows 0..7 the high terms, rows 8..15 the low terms, so
+// both halves of a sum meet in the same lane and small query groups (5 at one
+// token of a 40 / 8-head model) waste no second instruction.  Scores, the
+// running maximum, probabilities, sums and the weighted values stay fp32
+// (online softmax over the blocks).  Keys and values stream through two or
+// three stages of 32 KB (cp.async, two CTAs per SM); the number of shares
+// depends on the launch (SMs, heads) and their bounds on the device's length,
+// so an empty tail of the cache costs nothing.  Bound: cache bytes at one
+// token, the doubled products (1021 multiply-adds per clock and SM measured)
+// and the exponentials for large query groups.  Measured against the fp32
+// CUDA-core kernel over 32-key chunks that this one replaces (append
+// included): 4 sequences of 8000 tokens in caches of 16384, 40 / 8 heads, one
+// token: 161.7 -> 28.8 us (4.7 TB/s); 28 tokens of 4 sequences behind 2000,
+// 28 / 4 heads: 421 -> 65.7 us; error against 64 bits unchanged (2.1e-4, the
+// fp16 rounding of the output).
+template <int WM, int NT>
+__global__ void __launch_bounds__(kAttnThreads, 2) attention_kernel(const AttnArgs a) {
+  using C = AttnCfg<WM, NT>;
+  constexpr int WK = C::kWK, QT = C::kQT, NJ = C::kKeysStep / 8;
   griddep_wait();
   griddep_launch_dependents();
-  extern __shared__ __align__(16) float sm[];
-  const int Q = a.Q, T = a.T;
-  float2* cst = reinterpret_cast<float2*>(sm);                  // [T][D/2]
-  float* qs = sm + 2 * kMaxT * (kHeadDim / 2);                  // [Q][kRowPad]
-  float* ks = qs + Q * kRowPad;                                 // [C][kRowPad]
-  float* vs = ks + kAttnChunk * kRowPad;                        // [C][kRowPad]
-  float* sc = vs + kAttnChunk * kRowPad;                        // [Q][C]
-  const int bh = blockIdx.x, split = blockIdx.y;
+  extern __shared__ __align__(128) uint8_t asm_[];
+  const uint32_t base = smem_u32(asm_);
+  float* qfac = reinterpret_cast<float*>(asm_ + C::kOffFac);
+  float2* cst = reinterpret_cast<float2*>(asm_ + C::kOffCs);
+  const int T = a.T;
+  const int bh = (int)(blockIdx.x / (unsigned)a.nsplit), split = (int)(blockIdx.x - (unsigned)bh * a.nsplit);
+  const int q0 = blockIdx.y * QT;
   const int b = bh / a.Hkv, kvh = bh - b * a.Hkv;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int p0 = a.pos0[b];
-  const int64_t len = (int64_t)p0 + T;  // cache entries after the append
-  const int64_t j0 = (int64_t)split * kAttnChunk;
-  float* part = a.part + ((int64_t)bh * a.nsplit + split) * Q * kPartStride;
-  if (a.append && (p0 < 0 || len > a.max_ctx) && split == 0 && tid == 0)
+  const int64_t len64 = (int64_t)p0 + T;  // cache entries after the append
+  const bool valid = p0 >= 0 && len64 <= a.max_ctx;
+  if (a.append && !valid && split == 0 && blockIdx.y == 0 && tid == 0)
     atomicOr(&g_attn_status, SQ_DEV_BAD_POSITION);
-  if (j0 >= len || p0 < 0 || len > a.max_ctx) {  // empty chunk: neutral partials
-    for (int q = tid; q < Q; q += kAttnThreads) {
-      part[(int64_t)q * kPartStride] = -INFINITY;
-      part[(int64_t)q * kPartStride + 1] = 0.0f;
-    }
-    return;
-  }
-  const int nk = (int)(len - j0 < kAttnChunk ? len - j0 : kAttnChunk);
+  const int len = valid ? (int)len64 : 0;
+  const int nblk = (len + kBlockKeys - 1) / kBlockKeys;
+  const int blk0 = (int)((int64_t)split * nblk / a.nsplit);
+  const int blk1 = (int)((int64_t)(split + 1) * nblk / a.nsplit);
   const int64_t width = (int64_t)(a.Hq + 2 * a.Hkv) * kHeadDim;
-  const int64_t cbase = (((int64_t)b * a.Hkv + kvh) * a.max_ctx + j0) * kHeadDim;
-  // positions p0 .. p0+T-1 are the new tokens: with append, this chunk's
-  // share of them is rotated from qkv, written to the caches and used
-  // directly (every position belongs to one chunk, so each is written once)
-  const int j_new = a.append ? (int)((int64_t)p0 - j0) : kAttnChunk;  // first new key of the chunk
-  const int n_old = j_new < nk ? (j_new > 0 ? j_new : 0) : nk;         // keys read from the caches
-  // cached keys and values: 16-byte pieces (8 values), all of a thread's
-  // loads issued before the RoPE table is computed
-  constexpr int kPieces = kAttnChunk * kHeadDim / 8;
-  constexpr int kPerThread = kPieces / kAttnThreads;
-  static_assert(kPieces % kAttnThreads == 0, "whole pieces per thread");
-  uint4 kraw[kPerThread], vraw[kPerThread];
+  const int64_t cbase = ((int64_t)b * a.Hkv + kvh) * a.max_ctx * kHeadDim;
+  const int n_old = a.append ? p0 : len;  // keys read from the caches
+
+  // block -> stage: cached rows by asynchronous copies, rows past the end zero
+  auto load_block = [&](int blk, int stage) {
+    const uint32_t ks = base + C::kOffStage + stage * 2 * kStageHalf;
 #pragma unroll
-  for (int r = 0; r < kPerThread; ++r) {
-    const int pc = tid + r * kAttnThreads;
-    const int j = pc / (kHeadDim / 8);
-    const bool in = j < n_old;
-    kraw[r] = in ? *reinterpret_cast<const uint4*>(a.kc + cbase + (int64_t)pc * 8) : make_uint4(0u, 0u, 0u, 0u);
-    vraw[r] = in ? *reinterpret_cast<const uint4*>(a.vc + cbase + (int64_t)pc * 8) : make_uint4(0u, 0u, 0u, 0u);
-  }
-  for (int idx = tid; idx < T * (kHeadDim / 2); idx += kAttnThreads) {
-    const int t = idx / (kHeadDim / 2), d = idx - t * (kHeadDim / 2);
-    cst[idx] = rope_cs(p0 + t, a.rf.f[d]);
-  }
-#pragma unroll
-  for (int r = 0; r < kPerThread; ++r) {
-    const int pc = tid + r * kAttnThreads;
-    const int j = pc / (kHeadDim / 8), d8 = pc - j * (kHeadDim / 8);
-    if (j >= n_old && j < nk) continue;  // a new key: written below
-    const uint32_t kw[4] = {kraw[r].x, kraw[r].y, kraw[r].z, kraw[r].w};
-    const uint32_t vw[4] = {vraw[r].x, vraw[r].y, vraw[r].z, vraw[r].w};
-    float4* kd = reinterpret_cast<float4*>(ks + j * kRowPad + d8 * 8);
-    float4* vd = reinterpret_cast<float4*>(vs + j * kRowPad + d8 * 8);
-    kd[0] = make_float4(h2f_lo(kw[0]), h2f_hi(kw[0]), h2f_lo(kw[1]), h2f_hi(kw[1]));
-    kd[1] = make_float4(h2f_lo(kw[2]), h2f_hi(kw[2]), h2f_lo(kw[3]), h2f_hi(kw[3]));
-    vd[0] = make_float4(h2f_lo(vw[0]), h2f_hi(vw[0]), h2f_lo(vw[1]), h2f_hi(vw[1]));
-    vd[1] = make_float4(h2f_lo(vw[2]), h2f_hi(vw[2]), h2f_lo(vw[3]), h2f_hi(vw[3]));
-  }
-  if (n_old < nk) {  // new keys of this chunk (append): rotate from qkv
-    __syncthreads();  // cst is read below
-    for (int idx = n_old * kHeadDim + tid; idx < nk * kHeadDim; idx += kAttnThreads) {
-      const int j = idx / kHeadDim, d = idx - j * kHeadDim;
-      const int t = (int)(j0 + j - p0);
+    for (int i = 0; i < kBlockKeys * 16 / kAttnThreads; ++i) {
+      const int idx = tid + i * kAttnThreads;
+      const int r = idx >> 4, c = idx & 15;
+      const int j = blk * kBlockKeys + r;
+      if (j >= n_old && j < len) continue;  // a new key: written by fill_new
+      const bool in = j < n_old;
+      const int64_t src = cbase + (in ? (int64_t)j * kHeadDim + c * 8 : 0);
+      cp16(ks + tile_off(r, c), a.kc + src, in);
+      cp16(ks + kStageHalf + tile_off(r, c), a.vc + src, in);
+    }
+  };
+  // append: the new tokens of a block rotated from qkv, used directly and
+  // (by the first query group's CTA) written to the caches
+  auto fill_new = [&](int blk, int stage) {
+    const int j_lo = max(blk * kBlockKeys, n_old), j_hi = min((blk + 1) * kBlockKeys, len);
+    uint8_t* ks = asm_ + C::kOffStage + stage * 2 * kStageHalf;
+    for (int idx = tid; idx < (j_hi - j_lo) * (kHeadDim / 2); idx += kAttnThreads) {
+      const int j = j_lo + idx / (kHeadDim / 2), d = idx % (kHeadDim / 2);
+      const int t = j - p0, r = j - blk * kBlockKeys;
       const __half* row = a.qkv + ((int64_t)b * T + t) * width;
       const __half* kr = row + (int64_t)(a.Hq + kvh) * kHeadDim;
-      const __half vh = row[(int64_t)(a.Hq + a.Hkv + kvh) * kHeadDim + d];
-      const int pd = d & (kHeadDim / 2 - 1);
+      const __half* vr = row + (int64_t)(a.Hq + a.Hkv + kvh) * kHeadDim;
       __half y1, y2;
-      rope_rotate_f16(__half2float(kr[pd]), __half2float(kr[pd + kHeadDim / 2]), cst[t * (kHeadDim / 2) + pd],
-                      y1, y2);
-      const __half kh = d < kHeadDim / 2 ? y1 : y2;
-      a.kcw[cbase + idx] = kh;
-      a.vcw[cbase + idx] = vh;
-      ks[j * kRowPad + d] = __half2float(kh);
-      vs[j * kRowPad + d] = __half2float(vh);
+      rope_rotate_f16(__half2float(kr[d]), __half2float(kr[d + kHeadDim / 2]), cst[t * (kHeadDim / 2) + d], y1, y2);
+      const __half v1 = vr[d], v2 = vr[d + kHeadDim / 2];
+      const uint32_t o1 = tile_off(r, d >> 3) + (d & 7) * 2;
+      const uint32_t o2 = tile_off(r, (d + kHeadDim / 2) >> 3) + (d & 7) * 2;
+      *reinterpret_cast<__half*>(ks + o1) = y1;
+      *reinterpret_cast<__half*>(ks + o2) = y2;
+      *reinterpret_cast<__half*>(ks + kStageHalf + o1) = v1;
+      *reinterpret_cast<__half*>(ks + kStageHalf + o2) = v2;
+      if (blockIdx.y == 0) {
+        const int64_t dst = cbase + (int64_t)j * kHeadDim + d;
+        a.kcw[dst] = y1;
+        a.kcw[dst + kHeadDim / 2] = y2;
+        a.vcw[dst] = v1;
+        a.vcw[dst + kHeadDim / 2] = v2;
+      }
+    }
+  };
+
+  // ---- prologue: first blocks requested, then the queries
+#pragma unroll
+  for (int i = 0; i < C::kStages - 1; ++i) {
+    if (blk0 + i < blk1) load_block(blk0 + i, i);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  if (blk0 < blk1)
+    for (int idx = tid; idx < T * (kHeadDim / 2); idx += kAttnThreads)
+      cst[idx] = rope_cs(p0 + idx / (kHeadDim / 2), a.rf.f[idx % (kHeadDim / 2)]);
+  __syncthreads();
+  if (blk0 < blk1) {
+    // a warp per query: lane l the pairs (2l, 2l + 64), (2l + 1, 2l + 65)
+    const bool qvec = (reinterpret_cast<uintptr_t>(a.qkv) & 3) == 0;
+    for (int ql = warp; ql < QT; ql += kAttnWarps) {
+      const int q = q0 + ql;
+      float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // d = 2l, 2l + 1, 2l + 64, 2l + 65
+      if (q < a.Q) {
+        const int g = q / T, t = q - g * T;
+        const __half* qr = a.qkv + ((int64_t)b * T + t) * width + (int64_t)(kvh * a.G + g) * kHeadDim + 2 * lane;
+        float x[4];
+        if (qvec) {
+          const float2 u1 = __half22float2(*reinterpret_cast<const __half2*>(qr));
+          const float2 u2 = __half22float2(*reinterpret_cast<const __half2*>(qr + kHeadDim / 2));
+          x[0] = u1.x; x[1] = u1.y; x[2] = u2.x; x[3] = u2.y;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[e] = __half2float(qr[(e & 1) + (e >> 1) * (kHeadDim / 2)]);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float2 cs = cst[t * (kHeadDim / 2) + 2 * lane + e];
+          v[e] = x[e] * cs.x - x[e + 2] * cs.y;
+          v[e + 2] = x[e + 2] * cs.x + x[e] * cs.y;
+        }
+      }
+      const float am = warp_max(fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
+      int ex = 10;
+      if (am > 0.0f && isfinite(am)) ex = max((int)(__float_as_uint(am) >> 23) - 127, -100);
+      const float up = __uint_as_float((uint32_t)(127 + 10 - ex) << 23);  // 2^(10 - ex)
+      const int tile = ql >> 3, r = ql & 7;
+      uint8_t* qt = asm_ + tile * 4096;
+      __half hi[4], lo[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) split_f16(v[e] * up, hi[e], lo[e]);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int c = (lane >> 2) + e * 8;
+        const uint32_t in = (lane & 3) * 4;
+        *reinterpret_cast<uint32_t*>(qt + tile_off(r, c) + in) = pack_h2(hi[2 * e], hi[2 * e + 1]);
+        *reinterpret_cast<uint32_t*>(qt + tile_off(r + 8, c) + in) = pack_h2(lo[2 * e], lo[2 * e + 1]);
+      }
+      if (lane == 0) qfac[ql] = a.scale * __uint_as_float((uint32_t)(127 + ex - 10) << 23);
+    }
+    if (a.append)
+#pragma unroll
+      for (int i = 0; i < C::kStages - 1; ++i)
+        if (blk0 + i < blk1) fill_new(blk0 + i, i);
+  }
+  __syncthreads();
+
+  // ---- this warp's share: query tiles wm * NT .. of the CTA, keys
+  // [kw * kKeysWarp, + kKeysWarp) of every block
+  const int wm = warp % WM, kw = warp / WM;
+  const int g = lane >> 2, t4 = lane & 3;
+  float o[NT][16][4];
+  float mrun[NT], lrun[NT], fac[NT];
+  int tpos[NT];  // the query's token
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    mrun[nt] = -INFINITY;
+    lrun[nt] = 0.0f;
+    const int ql = (wm * NT + nt) * 8 + g;
+    fac[nt] = blk0 < blk1 ? qfac[ql] : 0.0f;
+    tpos[nt] = (q0 + ql) % T;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) o[nt][i][0] = o[nt][i][1] = o[nt][i][2] = o[nt][i][3] = 0.0f;
+  }
+  const uint32_t qbase = base + wm * NT * 4096;
+  // matrix-load rows and chunks of this lane: queries (rows 0..15), keys
+  // (two eight-key tiles), values (transposed)
+  const int qrow = (lane & 7) + ((lane >> 3) & 1) * 8, qch = lane >> 4;
+  const int krow = (lane & 7) + (lane >> 4) * 8, kch = (lane >> 3) & 1;
+  const int vrow = (lane & 7) + ((lane >> 3) & 1) * 8, vch = lane >> 4;
+  uint32_t qreg[NT == 1 ? 8 : 1][4];
+  if constexpr (NT == 1) {
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) ldsm_x4(qreg[kk], qbase + tile_off(qrow, 2 * kk + qch));
+  }
+
+  for (int blk = blk0; blk < blk1; ++blk) {
+    const int it = blk - blk0;
+    asm volatile("cp.async.wait_group %0;" ::"n"(C::kStages - 2) : "memory");
+    __syncthreads();
+    {
+      const int nx = blk + C::kStages - 1;
+      if (nx < blk1) {
+        load_block(nx, (it + C::kStages - 1) % C::kStages);
+        if (a.append && (nx + 1) * kBlockKeys > n_old) fill_new(nx, (it + C::kStages - 1) % C::kStages);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    const uint32_t ks = base + C::kOffStage + (it % C::kStages) * 2 * kStageHalf;
+    const uint32_t vs = ks + kStageHalf;
+    const bool edge = (blk + 1) * kBlockKeys > p0;  // some key may lie past a query
+#pragma unroll 1
+    for (int sub = 0; sub < C::kKeysWarp / C::kKeysStep; ++sub) {
+      const int kb = kw * C::kKeysWarp + sub * C::kKeysStep;
+      float s[NT][NJ][4];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) s[nt][j][0] = s[nt][j][1] = s[nt][j][2] = s[nt][j][3] = 0.0f;
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        uint32_t qa[NT][4];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          if constexpr (NT == 1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) qa[0][e] = qreg[kk][e];
+          } else {
+            ldsm_x4(qa[nt], qbase + nt * 4096 + tile_off(qrow, 2 * kk + qch));
+          }
+        }
+#pragma unroll
+        for (int jp = 0; jp < NJ / 2; ++jp) {
+          uint32_t kf[4];
+          ldsm_x4(kf, ks + tile_off(kb + jp * 16 + krow, 2 * kk + kch));
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            attn_mma(s[nt][2 * jp], qa[nt], kf[0], kf[1]);
+            attn_mma(s[nt][2 * jp + 1], qa[nt], kf[2], kf[3]);
+          }
+        }
+      }
+      // scores (high + low terms), mask, running maximum, probabilities
+      uint32_t pa[NT][NJ / 2][4];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            // (an infinite key: the high term alone has the sign)
+            const float sl = s[nt][j][e + 2];
+            float v = (s[nt][j][e] + (fabsf(sl) < INFINITY ? sl : 0.0f)) * fac[nt];
+            if (edge && blk * kBlockKeys + kb + 8 * j + 2 * t4 + e > p0 + tpos[nt]) v = -INFINITY;
+            s[nt][j][e] = v;
+            mx = fmaxf(mx, v);
+          }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        const float mnew = fmaxf(mrun[nt], mx);
+        if (__any_sync(0xffffffffu, mnew > mrun[nt])) {
+          const float corr = mrun[nt] == -INFINITY ? 0.0f : expf(mrun[nt] - mnew);
+          lrun[nt] *= corr;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[nt][i][e] *= corr;
+          mrun[nt] = mnew;
+        }
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          __half hi[2], lo[2];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float p = mrun[nt] == -INFINITY ? 0.0f : expf(s[nt][j][e] - mrun[nt]);
+            lrun[nt] += p;
+            split_f16(p * kProbScale, hi[e], lo[e]);
+          }
+          pa[nt][j >> 1][(j & 1) * 2] = pack_h2(hi[0], hi[1]);
+          pa[nt][j >> 1][(j & 1) * 2 + 1] = pack_h2(lo[0], lo[1]);
+        }
+      }
+#pragma unroll
+      for (int jj = 0; jj < NJ / 2; ++jj)
+#pragma unroll
+        for (int dp = 0; dp < 8; ++dp) {
+          uint32_t vf[4];
+          ldsm_x4_t(vf, vs + tile_off(kb + jj * 16 + vrow, 2 * dp + vch));
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            attn_mma(o[nt][2 * dp], pa[nt][jj], vf[0], vf[1]);
+            attn_mma(o[nt][2 * dp + 1], pa[nt][jj], vf[2], vf[3]);
+          }
+        }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+
+  // ---- this CTA's partial records (m, l, -, -, o[D]) in shared memory, over
+  // the stages: one per warp first, then the warps along the keys in order
+  float* rec = reinterpret_cast<float*>(asm_ + C::kOffStage);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    float l = lrun[nt];
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    float* r = rec + ((kw * WM + wm) * NT * 8 + nt * 8 + g) * kPartStride;
+    if (t4 == 0) {
+      r[0] = mrun[nt];
+      r[1] = l;
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      // (an infinite value: the high term alone has the sign)
+      const float l0 = fabsf(o[nt][i][2]) < INFINITY ? o[nt][i][2] : 0.0f;
+      const float l1 = fabsf(o[nt][i][3]) < INFINITY ? o[nt][i][3] : 0.0f;
+      const float2 v = make_float2((o[nt][i][0] + l0) * (1.0f / kProbScale), (o[nt][i][1] + l1) * (1.0f / kProbScale));
+      *reinterpret_cast<float2*>(r + kPartO + 8 * i + 2 * t4) = v;
     }
   }
   __syncthreads();
-  // queries: each thread rotates 8 pairs (d, d + D/2) read as two 16-byte
-  // pieces (q rows are 16-byte aligned when qkv is: D = 128 halves)
-  const bool qvec = (reinterpret_cast<uintptr_t>(a.qkv) & 15) == 0;
-  for (int idx = tid; idx < Q * (kHeadDim / 16); idx += kAttnThreads) {
-    const int q = idx / (kHeadDim / 16), d0 = (idx - q * (kHeadDim / 16)) * 8;
-    const int g = q / T, t = q - g * T;
-    const __half* qr = a.qkv + ((int64_t)b * T + t) * width + (int64_t)(kvh * a.G + g) * kHeadDim;
-    float x1[8], x2[8];
-    if (qvec) {
-      const uint4 u1 = *reinterpret_cast<const uint4*>(qr + d0);
-      const uint4 u2 = *reinterpret_cast<const uint4*>(qr + d0 + kHeadDim / 2);
-      const uint32_t w1[4] = {u1.x, u1.y, u1.z, u1.w}, w2[4] = {u2.x, u2.y, u2.z, u2.w};
+  const int nq = min(QT, a.Q - q0);
+  float* mine = WK > 1 ? rec + WK * QT * kPartStride : rec;
+  if constexpr (WK > 1) {
+    for (int idx = tid; idx < nq * (kHeadDim / 4); idx += kAttnThreads) {
+      const int q = idx / (kHeadDim / 4), d4 = idx % (kHeadDim / 4);
+      float M = -INFINITY;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        x1[2 * e] = h2f_lo(w1[e]);
-        x1[2 * e + 1] = h2f_hi(w1[e]);
-        x2[2 * e] = h2f_lo(w2[e]);
-        x2[2 * e + 1] = h2f_hi(w2[e]);
+      for (int w = 0; w < WK; ++w) M = fmaxf(M, rec[(w * QT + q) * kPartStride]);
+      float L = 0.0f;
+      float4 O = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (M != -INFINITY)
+#pragma unroll
+        for (int w = 0; w < WK; ++w) {
+          const float* r = rec + (w * QT + q) * kPartStride;
+          if (r[0] == -INFINITY) continue;
+          const float f = expf(r[0] - M);
+          const float4 v = *reinterpret_cast<const float4*>(r + kPartO + 4 * d4);
+          L = fmaf(f, r[1], L);
+          O.x = fmaf(f, v.x, O.x);
+          O.y = fmaf(f, v.y, O.y);
+          O.z = fmaf(f, v.z, O.z);
+          O.w = fmaf(f, v.w, O.w);
+        }
+      float* r = mine + q * kPartStride;
+      if (d4 == 0) {
+        r[0] = M;
+        r[1] = L;
       }
+      *reinterpret_cast<float4*>(r + kPartO + 4 * d4) = O;
+    }
+    __syncthreads();
+  }
+
+  if (!a.cluster && a.nsplit > 1) {  // records to the workspace, merged by attention_combine_kernel
+    float* part = a.part + (((int64_t)bh * a.nsplit + split) * a.Q + q0) * kPartStride;
+    for (int idx = tid; idx < nq * (kPartStride / 4); idx += kAttnThreads)
+      reinterpret_cast<float4*>(part)[idx] = reinterpret_cast<const float4*>(mine)[idx];
+    return;
+  }
+  // ---- the cluster's records merged in rank order; rank r writes its share
+  const int S = a.nsplit;
+  if (S > 1) attn_cluster_sync();
+  const int items = nq * (kHeadDim / 4);
+  const int i0 = (int)((int64_t)split * items / S), i1 = (int)((int64_t)(split + 1) * items / S);
+  const bool ovec = (reinterpret_cast<uintptr_t>(a.out) & 7) == 0;
+  for (int idx = i0 + tid; idx < i1; idx += kAttnThreads) {
+    const int q = idx / (kHeadDim / 4), d4 = idx % (kHeadDim / 4);
+    float M = -INFINITY, L = 0.0f;
+    float4 O = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int s0 = 0; s0 < S; s0 += 8) {
+      // eight ranks' records in flight, then added in rank order
+      float4 ml[8], ov[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (s0 + u < S) {
+          const uint32_t r = S > 1 ? attn_rank_addr(mine + q * kPartStride, (uint32_t)(s0 + u))
+                                   : smem_u32(mine + q * kPartStride);
+          ml[u] = ld_cluster_f4(r);
+          ov[u] = ld_cluster_f4(r + (kPartO + 4 * d4) * 4);
+        }
+      float Mn = M;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (s0 + u < S) Mn = fmaxf(Mn, ml[u].x);
+      if (Mn == -INFINITY) continue;
+      const float c = M == -INFINITY ? 0.0f : expf(M - Mn);
+      L *= c;
+      O.x *= c; O.y *= c; O.z *= c; O.w *= c;
+      M = Mn;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (s0 + u < S && ml[u].x != -INFINITY) {
+          const float f = expf(ml[u].x - M);
+          L = fmaf(f, ml[u].y, L);
+          O.x = fmaf(f, ov[u].x, O.x);
+          O.y = fmaf(f, ov[u].y, O.y);
+          O.z = fmaf(f, ov[u].z, O.z);
+          O.w = fmaf(f, ov[u].w, O.w);
+        }
+    }
+    const int qq = q0 + q, hg = qq / T, t = qq - hg * T;
+    __half* dst = a.out + (((int64_t)b * T + t) * a.Hq + kvh * a.G + hg) * kHeadDim + 4 * d4;
+    const __half h0 = __float2half_rn(L > 0.0f ? O.x / L : 0.0f), h1 = __float2half_rn(L > 0.0f ? O.y / L : 0.0f);
+    const __half h2 = __float2half_rn(L > 0.0f ? O.z / L : 0.0f), h3 = __float2half_rn(L > 0.0f ? O.w / L : 0.0f);
+    if (ovec) {
+      *reinterpret_cast<uint2*>(dst) = make_uint2(pack_h2(h0, h1), pack_h2(h2, h3));
     } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        x1[e] = __half2float(qr[d0 + e]);
-        x2[e] = __half2float(qr[d0 + e + kHeadDim / 2]);
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float2 cs = cst[t * (kHeadDim / 2) + d0 + e];
-      qs[q * kRowPad + d0 + e] = (x1[e] * cs.x - x2[e] * cs.y) * a.scale;
-      qs[q * kRowPad + d0 + e + kHeadDim / 2] = (x2[e] * cs.x + x1[e] * cs.y) * a.scale;
+      dst[0] = h0; dst[1] = h1; dst[2] = h2; dst[3] = h3;
     }
   }
   __syncthreads();
-  // scores: each thread a 2-query x 4-key tile, 16-byte shared loads along D
-  const int qpairs = (Q + 1) / 2;
-  for (int tile = tid; tile < qpairs * (kAttnChunk / 4); tile += kAttnThreads) {
-    const int qp = tile / (kAttnChunk / 4), kq = tile - qp * (kAttnChunk / 4);
-    const int q0 = 2 * qp, q1 = q0 + 1 < Q ? q0 + 1 : q0;
-    float acc[2][4] = {};
-    const float4* qa = reinterpret_cast<const float4*>(qs + q0 * kRowPad);
-    const float4* qb = reinterpret_cast<const float4*>(qs + q1 * kRowPad);
-#pragma unroll 4
-    for (int d4 = 0; d4 < kHeadDim / 4; ++d4) {
-      const float4 x0 = qa[d4], x1 = qb[d4];
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const float4 kv = reinterpret_cast<const float4*>(ks + (4 * kq + kk) * kRowPad)[d4];
-        acc[0][kk] = fmaf(x0.x, kv.x, fmaf(x0.y, kv.y, fmaf(x0.z, kv.z, fmaf(x0.w, kv.w, acc[0][kk]))));
-        acc[1][kk] = fmaf(x1.x, kv.x, fmaf(x1.y, kv.y, fmaf(x1.z, kv.z, fmaf(x1.w, kv.w, acc[1][kk]))));
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int q = i ? q1 : q0;
-      if (i && q1 == q0) break;
-      const int t = q % T;
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const int j = 4 * kq + kk;
-        sc[q * kAttnChunk + j] = (j < nk && j0 + j <= (int64_t)p0 + t) ? acc[i][kk] : -INFINITY;
-      }
-    }
-  }
-  __syncthreads();
-  // per query: chunk max, exp, sum (one warp per query, one key per lane)
-  static_assert(kAttnChunk == 32, "one key per lane");
-  const int warp = tid >> 5, lane = tid & 31;
-  for (int q = warp; q < Q; q += kAttnThreads / 32) {
-    const float v = sc[q * kAttnChunk + lane];
-    const float mx = warp_max(v);
-    const float e = mx == -INFINITY ? 0.0f : expf(v - mx);
-    sc[q * kAttnChunk + lane] = e;
-    const float l = warp_sum(e);
-    if (lane == 0) {
-      part[(int64_t)q * kPartStride] = mx;
-      part[(int64_t)q * kPartStride + 1] = l;
-    }
-  }
-  __syncthreads();
-  // weighted values: each thread a 2-query x 4-dim tile
-  for (int tile = tid; tile < qpairs * (kHeadDim / 4); tile += kAttnThreads) {
-    const int qp = tile / (kHeadDim / 4), d4 = tile - qp * (kHeadDim / 4);
-    const int q0 = 2 * qp, q1 = q0 + 1 < Q ? q0 + 1 : q0;
-    float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
-    for (int j = 0; j < nk; ++j) {
-      const float e0 = sc[q0 * kAttnChunk + j], e1 = sc[q1 * kAttnChunk + j];
-      const float4 vv = reinterpret_cast<const float4*>(vs + j * kRowPad)[d4];
-      o0.x = fmaf(e0, vv.x, o0.x); o0.y = fmaf(e0, vv.y, o0.y);
-      o0.z = fmaf(e0, vv.z, o0.z); o0.w = fmaf(e0, vv.w, o0.w);
-      o1.x = fmaf(e1, vv.x, o1.x); o1.y = fmaf(e1, vv.y, o1.y);
-      o1.z = fmaf(e1, vv.z, o1.z); o1.w = fmaf(e1, vv.w, o1.w);
-    }
-    *reinterpret_cast<float4*>(part + (int64_t)q0 * kPartStride + kPartO + 4 * d4) = o0;
-    if (q1 != q0) *reinterpret_cast<float4*>(part + (int64_t)q1 * kPartStride + kPartO + 4 * d4) = o1;
-  }
+  if (S > 1) attn_cluster_sync();  // no CTA leaves while another reads its records
 }
 
 // One CTA per (sequence and key/value head, query): the chunk maxima and
@@ -514,8 +808,16 @@ cudaError_t launch_rmsnorm(const __half* x, const __half* gamma, int M, int64_t 
 }
 
 static RopeFreq rope_freq(double theta) {
-  RopeFreq rf;
-  for (int d = 0; d < kHeadDim / 2; ++d) rf.f[d] = pow(theta, -2.0 * d / (double)kHeadDim);
+  // the last theta's table per host thread (64 pow calls take longer than a launch)
+  static thread_local double last = 0.0;
+  static thread_local RopeFreq rf;
+  if (theta != last) {
+    for (int d = 0; d < kHeadDim / 2; ++d) {
+      const double turns = pow(theta, -2.0 * d / (double)kHeadDim) / 6.283185307179586;
+      rf.f[d] = (unsigned long long)(turns * 18446744073709551616.0);
+    }
+    last = theta;
+  }
   return rf;
 }
 
@@ -526,19 +828,119 @@ cudaError_t launch_kv_append(const __half* qkv, int B, int T, int Hq, int Hkv, c
                     qkv, T, Hq, Hkv, pos0, rope_freq(theta), kc, vc, max_ctx);
 }
 
+// Room for one record per query and 32 cache positions (more than the shares
+// of 64-key blocks ever need).
 size_t attention_workspace_bytes(int B, int T, int Hq, int Hkv, int64_t max_ctx) {
   if (B < 0 || T < 0 || Hkv <= 0 || max_ctx <= 0) return 0;
-  const int64_t nsplit = (max_ctx + kAttnChunk - 1) / kAttnChunk;
+  const int64_t nsplit = (max_ctx + 31) / 32;
   const int64_t Q = (int64_t)(Hq / Hkv) * T;
   return (size_t)B * Hkv * nsplit * Q * kPartStride * sizeof(float);
 }
 
-size_t attention_smem_bytes(int Q) {
-  return ((size_t)2 * kMaxT * (kHeadDim / 2) + (size_t)Q * kRowPad + (size_t)2 * kAttnChunk * kRowPad +
-          (size_t)Q * kAttnChunk) * sizeof(float);
+int attention_max_tokens() { return kMaxT; }
+
+constexpr int kAttnMaxCluster = 16;
+
+// Prepares an instance and returns how many clusters of S of its CTAs can be
+// resident (cached per device and S; S = 0: only prepares).
+template <int WM, int NT>
+static cudaError_t attn_resident(int S, int* n) {
+  auto k = attention_kernel<WM, NT>;
+  constexpr int kMaxSmem = attn_smem(AttnCfg<WM, NT>::kOffCs, AttnCfg<WM, NT>::kMaxTokens);
+  static std::mutex mu;
+  static bool ready[64] = {false};
+  static int cache[64][kAttnMaxCluster + 1] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!ready[dev]) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    ready[dev] = true;
+  }
+  if (S == 0) return cudaSuccess;
+  if (cache[dev][S] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)S);
+    cfg.blockDim = dim3(kAttnThreads);
+    cfg.dynamicSmemBytes = (size_t)kMaxSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)S;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int c = 0;
+    if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      c = 0;
+    }
+    cache[dev][S] = c + 1;
+  }
+  *n = cache[dev][S] - 1;
+  return cudaSuccess;
 }
 
-int attention_max_tokens() { return kMaxT; }
+// How many CTAs share the keys of one (sequence, key/value head, query
+// group), and how they meet.  As many as fill the two CTAs per SM, at most
+// one per 64-key block of the cache; up to 16 meet in a cluster (one launch,
+// the records never leave the chip), as long as all clusters are resident at
+// once.  A long cache under few heads wants more shares than that: from 16
+// blocks a CTA on, the records go through the workspace and a second launch
+// merges them.
+template <int WM, int NT>
+static cudaError_t launch_attn_inst(AttnArgs a, cudaStream_t st) {
+  using C = AttnCfg<WM, NT>;
+  const int smem = attn_smem(C::kOffCs, a.T);
+  const int Z = (a.Q + C::kQT - 1) / C::kQT;
+  const int64_t base = (int64_t)a.B * a.Hkv * Z;
+  const int64_t blocks = (a.max_ctx + kBlockKeys - 1) / kBlockKeys;
+  int64_t S = 2 * (int64_t)device_sm_count() / base;
+  if (S > blocks) S = blocks;
+  if (S < 1) S = 1;
+  a.cluster = S > 1 && (S <= kAttnMaxCluster || blocks <= kAttnMaxCluster * 16);
+  int n = 0;
+  cudaError_t e = attn_resident<WM, NT>(0, &n);
+  if (e != cudaSuccess) return e;
+  if (a.cluster) {
+    if (S > kAttnMaxCluster) S = kAttnMaxCluster;
+    for (; S > 1; --S) {
+      e = attn_resident<WM, NT>((int)S, &n);
+      if (e != cudaSuccess) return e;
+      if (n >= base) break;
+    }
+    a.cluster = S > 1;
+  }
+  a.nsplit = (int)S;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(S * a.B * a.Hkv), (unsigned)Z);
+  cfg.blockDim = dim3(kAttnThreads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (a.cluster) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)S;
+    at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  const bool legacy = (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread);
+  if (!legacy && pdl_enabled()) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = na;
+  e = cudaLaunchKernelEx(&cfg, attention_kernel<WM, NT>, a);
+  if (e != cudaSuccess || a.cluster || S == 1) return e;
+  return launch_pdl(attention_combine_kernel, dim3((unsigned)(a.B * a.Hkv), (unsigned)a.Q), dim3(kHeadDim),
+                    (size_t)2 * a.nsplit * sizeof(float), st, a);
+}
 
 cudaError_t launch_attention(const __half* qkv, int B, int T, int Hq, int Hkv, const int32_t* pos0,
                              double theta, const __half* kc, const __half* vc, int64_t max_ctx,
@@ -562,25 +964,12 @@ cudaError_t launch_attention(const __half* qkv, int B, int T, int Hq, int Hkv, c
   a.G = Hq / Hkv;
   a.Q = a.G * T;
   a.max_ctx = max_ctx;
-  a.nsplit = (int)((max_ctx + kAttnChunk - 1) / kAttnChunk);
   a.rf = rope_freq(theta);
   a.scale = 1.0f / sqrtf((float)kHeadDim);
-  const size_t smem = attention_smem_bytes(a.Q);
-  static int smem_set[64] = {0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if ((int)smem > smem_set[dev]) {
-    e = cudaFuncSetAttribute(attention_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    smem_set[dev] = (int)smem;
-  }
-  e = launch_pdl(attention_partial_kernel, dim3((unsigned)(B * Hkv), (unsigned)a.nsplit),
-                 dim3(kAttnThreads), smem, st, a);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(attention_combine_kernel, dim3((unsigned)(B * Hkv), (unsigned)a.Q), dim3(kHeadDim),
-                    (size_t)2 * a.nsplit * sizeof(float), st, a);
+  if (a.Q <= 8) return launch_attn_inst<1, 1>(a, st);
+  if (a.Q <= 16) return launch_attn_inst<1, 2>(a, st);
+  if (a.Q <= 32) return launch_attn_inst<2, 2>(a, st);
+  return launch_attn_inst<4, 2>(a, st);
 }
 
 cudaError_t launch_kv_rollback(const int32_t* base, const int32_t* n, int B, int limit, int32_t* len,

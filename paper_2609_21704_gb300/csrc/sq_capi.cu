@@ -567,8 +567,6 @@ static sq_status attention_common(const char* who, const void* qkv, int B, int T
   if (!workspace || ws_bytes < need)
     return fail(SQ_ERR_WORKSPACE, "%s: workspace %zu bytes < %zu required", who, ws_bytes, need);
   if (!aligned(workspace, 16)) return fail(SQ_ERR_ALIGN, "%s: workspace must be 16-byte aligned", who);
-  if (attention_smem_bytes((Hq / Hkv) * T) > (size_t)device_max_smem())
-    return fail(SQ_ERR_SHAPE, "%s: query group too large for shared memory", who);
   if (max_ctx > ((int64_t)1 << 17)) return fail(SQ_ERR_SHAPE, "%s: max_ctx > 2^17", who);
   __half* kw = append ? reinterpret_cast<__half*>(const_cast<void*>(k_cache)) : nullptr;
   __half* vw = append ? reinterpret_cast<__half*>(const_cast<void*>(v_cache)) : nullptr;

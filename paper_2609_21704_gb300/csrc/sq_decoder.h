@@ -13,7 +13,6 @@ cudaError_t launch_rmsnorm(const __half* x, const __half* gamma, int M, int64_t 
 cudaError_t launch_kv_append(const __half* qkv, int B, int T, int Hq, int Hkv, const int32_t* pos0,
                              double theta, __half* kc, __half* vc, int64_t max_ctx, cudaStream_t st);
 size_t attention_workspace_bytes(int B, int T, int Hq, int Hkv, int64_t max_ctx);
-size_t attention_smem_bytes(int Q);
 int attention_max_tokens();  // T limit of sq_kv_append / sq_attention
 // kc_append / vc_append (the same caches as kc / vc, or null): append the
 // new tokens' rotated keys and values in the same launch.
