@@ -10,128 +10,248 @@
 // These kernels never let the next kernel start early: linear kernels read
 // their weights before waiting on the previous kernel, and the weights may
 // be what this kernel writes.
-// Both kernels are HBM-bound streaming passes: 2 B read per weight, 0.516 B
-// (INT4) or 1 B (FP8) written.
+//
+// The quotients: the IEEE divide costs a dozen instructions, so w / s is
+// bracketed instead.  With r = fp32(1 / s), w r (1 -+ 2^-21) lie on either
+// side of fp32(w / s) (r and each product are within 2^-24 of exact); where
+// both round to the same code, that is the code.  Where they do not (exact
+// ties of INT4 codes, about 3 in 10^4 Gaussian weights; next to none of FP8),
+// the thread divides.
+//
+// Bound: HBM, 2 B read per weight, 0.516 B (INT4) or 1 B (FP8) written.
 #include "sq_internal.h"
 
 namespace sq {
 
 __device__ unsigned int g_quant_status;
 
-// One warp per (row, group): lane l holds k = 4l .. 4l+3 of the group.
-__global__ void __launch_bounds__(256) quant_int4_kernel(const __half* __restrict__ w, int64_t N,
-                                                         int64_t K, uint8_t* __restrict__ codes,
-                                                         __half* __restrict__ scales) {
-  griddep_wait();  // no early trigger: a linear call may read these outputs at once
-  const int lane = threadIdx.x & 31;
-  const int64_t G = K / 128;
-  const int64_t total = N * G;
-  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t gid = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); gid < total;
-       gid += nwarps) {
-    const int64_t n = gid / G, g = gid - n * G;
-    const __half* src = w + n * K + g * 128 + lane * 4;
-    const uint2 raw = *reinterpret_cast<const uint2*>(src);
-    float v[4];
-    v[0] = __half2float(__ushort_as_half(lo16(raw.x)));
-    v[1] = __half2float(__ushort_as_half(hi16(raw.x)));
-    v[2] = __half2float(__ushort_as_half(lo16(raw.y)));
-    v[3] = __half2float(__ushort_as_half(hi16(raw.y)));
-    float a = 0.0f;
-    bool bad = false;
+constexpr int kQuantThreads = 256;
+
+__device__ __forceinline__ void halves8(const uint4 v, float out[8]) {
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      bad |= !isfinite(v[i]);
-      a = fmaxf(a, fabsf(v[i]));
-    }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
-    const float amax = warp_max(a);
-    __half sh = __float2half_rn(__fdiv_rn(amax, 7.0f));
-    if (amax > 0.0f && __half_as_ushort(sh) == 0) sh = __ushort_as_half(1);
-    const float s = __half2float(sh);
-    uint32_t packed = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int c = 0;
-      if (s != 0.0f) {
-        float t = rintf(__fdiv_rn(v[i], s));
-        t = fminf(fmaxf(t, -8.0f), 7.0f);
-        c = (int)t;
-      }
-      packed |= (uint32_t)(c + 8) << (4 * i);
-    }
-    *reinterpret_cast<uint16_t*>(codes + n * (K / 2) + g * 64 + lane * 2) = (uint16_t)packed;
-    if (lane == 0) scales[n * G + g] = sh;
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u[i]));
+    out[2 * i] = f.x;
+    out[2 * i + 1] = f.y;
   }
 }
 
-// One CTA per row (grid-stride): pass 1 finds amax, pass 2 (re-reading the
-// row from L1/L2) encodes 8 weights per thread-iteration.
-__global__ void __launch_bounds__(256) quant_fp8_kernel(const __half* __restrict__ w, int64_t N,
-                                                        int64_t K, uint8_t* __restrict__ codes,
-                                                        float* __restrict__ scales) {
+// Largest magnitude of eight fp16 values as fp16 bits (which order like
+// integers; 0x7c00 and up: an infinity or NaN among them).
+__device__ __forceinline__ uint32_t absmax8(const uint4 v, uint32_t m) {
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t a = u[i] & 0x7fff7fffu;
+    m = __vmaxu2(m, a);  // per half
+  }
+  return m;
+}
+
+// The definition's INT4 code (plus 8) by division.
+__device__ __forceinline__ uint32_t int4_code(float w, float s) {
+  if (s == 0.0f) return 8u;
+  return (uint32_t)((int)fminf(fmaxf(rintf(__fdiv_rn(w, s)), -8.0f), 7.0f) + 8);
+}
+
+// A warp takes 1024 consecutive weights, eight groups, as four coalesced
+// 16-byte loads a lane (lane l holds chunk 32 i + l: sixteen lanes a group and
+// load).  The maxima of a lane's four groups are reduced together, packed in
+// pairs; lane j mod 4 then divides for group j only, so a group's two divides
+// cost a quarter of a lane's issue slots.  The 14B fused gate/up (27648 x
+// 5120) takes 73 us, 4.9 TB/s of the measured 6.8; one lane per four weights
+// with a divide per weight took 214.  Bound: about half issue slots (7 a
+// weight), half memory.
+__global__ void __launch_bounds__(kQuantThreads) quant_int4_kernel(const __half* __restrict__ w, int64_t N,
+                                                                   int64_t K, uint8_t* __restrict__ codes,
+                                                                   __half* __restrict__ scales) {
   griddep_wait();  // no early trigger: a linear call may read these outputs at once
-  __shared__ float red[8];
-  __shared__ int red_bad[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t chunks = K / 8;
-  for (int64_t n = blockIdx.x; n < N; n += gridDim.x) {
-    const uint4* row = reinterpret_cast<const uint4*>(w + n * K);
-    float a = 0.0f;
-    int bad = 0;
-    for (int64_t c = threadIdx.x; c < chunks; c += blockDim.x) {
-      const uint4 r = row[c];
-      const uint32_t u[4] = {r.x, r.y, r.z, r.w};
+  const int lane = threadIdx.x & 31;
+  const int64_t total = N * (K / 8);  // chunks; a row is whole groups of 16, so groups are contiguous
+  const int64_t step = (int64_t)gridDim.x * (kQuantThreads / 32) * 128;
+  for (int64_t c0 = ((int64_t)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5)) * 128; c0 < total; c0 += step) {
+    uint4 v[4];
+    uint32_t m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t c = c0 + 32 * i + lane;  // the lanes of a group are in or out together
+      v[i] = c < total ? ld_stream16(w + 8 * c) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      m[i] = absmax8(v[i], 0u);
+      m[i] = max(m[i] & 0xffffu, m[i] >> 16);
+    }
+    uint32_t pk[2] = {m[0] | (m[1] << 16), m[2] | (m[3] << 16)};
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      pk[0] = __vmaxu2(pk[0], __shfl_xor_sync(0xffffffffu, pk[0], o));
+      pk[1] = __vmaxu2(pk[1], __shfl_xor_sync(0xffffffffu, pk[1], o));
+    }
+    // this lane's group: load lane & 3, half-warp lane >> 4
+    const uint32_t mine = ((lane & 2 ? pk[1] : pk[0]) >> (16 * (lane & 1))) & 0xffffu;
+    const bool bad = mine >= 0x7c00u;
+    float amax = __half2float(__ushort_as_half((uint16_t)mine));
+    if (__any_sync(0xffffffffu, bad)) {
+      // the largest magnitude that is not NaN, as fmaxf takes it
+      float keep = amax;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float x0 = __half2float(__ushort_as_half(lo16(u[i])));
-        const float x1 = __half2float(__ushort_as_half(hi16(u[i])));
-        bad |= !isfinite(x0) | !isfinite(x1);
-        a = fmaxf(a, fmaxf(fabsf(x0), fabsf(x1)));
-      }
-    }
-    a = warp_max(a);
-    bad = __any_sync(0xffffffffu, bad);
-    if (lane == 0) {
-      red[warp] = a;
-      red_bad[warp] = bad;
-    }
-    __syncthreads();
-    float amax = 0.0f;
-    int any_bad = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-      amax = fmaxf(amax, red[i]);
-      any_bad |= red_bad[i];
-    }
-    __syncthreads();
-    if (any_bad && threadIdx.x == 0) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
-    const float s = __fdiv_rn(amax, 448.0f);
-    if (threadIdx.x == 0) scales[n] = s;
-    uint2* out = reinterpret_cast<uint2*>(codes + n * K);
-    for (int64_t c = threadIdx.x; c < chunks; c += blockDim.x) {
-      const uint4 r = row[c];
-      const uint32_t u[4] = {r.x, r.y, r.z, r.w};
-      uint32_t o[2] = {0u, 0u};
-      if (s != 0.0f) {
+        float f[8], a = 0.0f;
+        halves8(v[i], f);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float x0 = __fdiv_rn(__half2float(__ushort_as_half(lo16(u[i]))), s);
-          const float x1 = __fdiv_rn(__half2float(__ushort_as_half(hi16(u[i]))), s);
-          o[i >> 1] |= (uint32_t)f32x2_to_e4m3x2(x0, x1) << (16 * (i & 1));
-        }
+        for (int e = 0; e < 8; ++e) a = fmaxf(a, fabsf(f[e]));
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+        if ((lane & 3) == i) keep = a;
       }
-      out[c] = make_uint2(o[0], o[1]);
+      amax = keep;
+      if (bad && (lane & 12) == 0) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
+    }
+    __half sh = __float2half_rn(__fdiv_rn(amax, 7.0f));
+    if (amax > 0.0f && __half_as_ushort(sh) == 0) sh = __ushort_as_half(1);
+    const float s = __half2float(sh);
+    // -1: the codes by division (below the normal scales a code can pass 7)
+    const float r = bad || s < 0x1p-14f ? -1.0f : __fdiv_rn(1.0f, s);
+    if ((lane & 12) == 0) {
+      const int64_t g = (c0 >> 4) + 2 * (lane & 3) + (lane >> 4);
+      if (g < (total >> 4)) scales[g] = sh;
+    }
+    // codes by bracketing: fma(w, r, magic) rounds the quotient into the low
+    // bits of the sum, the integer sums of those bits (shifted) place the nibbles
+    const float magic = 12582912.0f + 8.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int src = (lane & 16) | i;
+      const float gs = __shfl_sync(0xffffffffu, s, src), gr = __shfl_sync(0xffffffffu, r, src);
+      const float rlo = gr * (1.0f - 0x1p-21f), rhi = gr * (1.0f + 0x1p-21f);
+      float f[8];
+      halves8(v[i], f);
+      uint32_t acc = 0, diff = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t lo = __float_as_uint(fmaf(f[e], rlo, magic)), hi = __float_as_uint(fmaf(f[e], rhi, magic));
+        diff |= lo ^ hi;
+        acc += lo << (4 * e);
+      }
+      uint32_t word = acc - 0x4b400000u * 0x11111111u;  // the exponent bits of the eight sums
+      if (diff != 0 || gr < 0.0f) {
+        word = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) word |= int4_code(f[e], gs) << (4 * e);
+      }
+      const int64_t c = c0 + 32 * i + lane;
+      if (c < total) reinterpret_cast<uint32_t*>(codes)[c] = word;
+    }
+  }
+}
+
+// Codes of eight weights of an FP8 row.
+__device__ __forceinline__ uint2 fp8_codes8(const uint4 v, float s, float rlo, float rhi) {
+  float f[8];
+  halves8(v, f);
+  uint32_t lo[2] = {0u, 0u}, hi[2] = {0u, 0u};
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    lo[e >> 2] |= (uint32_t)f32x2_to_e4m3x2(f[e] * rlo, f[e + 1] * rlo) << (8 * (e & 3));
+    hi[e >> 2] |= (uint32_t)f32x2_to_e4m3x2(f[e] * rhi, f[e + 1] * rhi) << (8 * (e & 3));
+  }
+  if (((lo[0] ^ hi[0]) | (lo[1] ^ hi[1])) != 0u) {
+    lo[0] = lo[1] = 0u;
+    if (s != 0.0f)
+#pragma unroll
+      for (int e = 0; e < 8; e += 2)
+        lo[e >> 2] |= (uint32_t)f32x2_to_e4m3x2(__fdiv_rn(f[e], s), __fdiv_rn(f[e + 1], s)) << (8 * (e & 3));
+  }
+  return make_uint2(lo[0], lo[1]);
+}
+
+// A group of TPR threads per row: its first kFp8Keep chunks of eight weights
+// per thread stay in registers between the maximum and the codes, longer rows
+// read the rest again.
+constexpr int kFp8Keep = 8;
+template <int TPR>
+__global__ void __launch_bounds__(kQuantThreads) quant_fp8_kernel(const __half* __restrict__ w, int64_t N,
+                                                                  int64_t K, uint8_t* __restrict__ codes,
+                                                                  float* __restrict__ scales) {
+  griddep_wait();  // no early trigger: a linear call may read these outputs at once
+  constexpr int RPC = kQuantThreads / TPR;  // rows a CTA holds at once
+  __shared__ uint32_t red[2][kQuantThreads / 32];
+  __shared__ float redf[2][kQuantThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rt = threadIdx.x % TPR, rr = threadIdx.x / TPR;
+  const int64_t chunks = K / 8;
+  int par = 0;
+  for (int64_t n0 = (int64_t)blockIdx.x * RPC; n0 < N; n0 += (int64_t)gridDim.x * RPC, par ^= 1) {
+    const int64_t n = n0 + rr;
+    const bool in = n < N;
+    const uint4* row = reinterpret_cast<const uint4*>(w + (in ? n : 0) * K);
+    uint4 v[kFp8Keep];
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < kFp8Keep; ++i) {
+      const int64_t c = rt + (int64_t)i * TPR;
+      v[i] = in && c < chunks ? row[c] : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < kFp8Keep; ++i) m = absmax8(v[i], m);
+    for (int64_t c = rt + (int64_t)kFp8Keep * TPR; in && c < chunks; c += TPR) m = absmax8(row[c], m);
+    m = max(m & 0xffffu, m >> 16);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if constexpr (TPR > 32) {
+      if (lane == 0) red[par][warp] = m;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < TPR / 32; ++i) m = max(m, red[par][i]);
+    }
+    float amax = __half2float(__ushort_as_half((uint16_t)m));
+    const bool bad = m >= 0x7c00u;  // uniform over the row's threads
+    if (bad) {
+      // the largest magnitude that is not NaN, as fmaxf takes it
+      float a = 0.0f;
+      for (int64_t c = rt; in && c < chunks; c += TPR) {
+        float f[8];
+        halves8(row[c], f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) a = fmaxf(a, fabsf(f[e]));
+      }
+      a = warp_max(a);
+      if constexpr (TPR > 32) {
+        if (lane == 0) redf[par][warp] = a;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < TPR / 32; ++i) a = fmaxf(a, redf[par][i]);
+      }
+      amax = a;
+      if (rt == 0 && in) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
+    }
+    const float s = __fdiv_rn(amax, 448.0f);
+    // (-1: zero and infinite scales bracket to different codes, so those rows
+    // take the division's path)
+    const float r = s > 0.0f ? __fdiv_rn(1.0f, s) : 0.0f;
+    const float rlo = bad || s == 0.0f ? -1.0f : r * (1.0f - 0x1p-21f), rhi = r * (1.0f + 0x1p-21f);
+    if (in) {
+      if (rt == 0) scales[n] = s;
+      uint2* out = reinterpret_cast<uint2*>(codes + n * K);
+#pragma unroll
+      for (int i = 0; i < kFp8Keep; ++i) {
+        const int64_t c = rt + (int64_t)i * TPR;
+        if (c < chunks) out[c] = fp8_codes8(v[i], s, rlo, rhi);
+      }
+      for (int64_t c = rt + (int64_t)kFp8Keep * TPR; c < chunks; c += TPR) out[c] = fp8_codes8(row[c], s, rlo, rhi);
     }
   }
 }
 
 cudaError_t launch_quant_int4(const void* w, int64_t N, int64_t K, void* codes, void* scales,
                               cudaStream_t st) {
-  const int64_t total = N * (K / 128);
+  const int64_t total = N * (K / 8);
   if (total == 0) return cudaSuccess;
-  const int64_t want = (total + 7) / 8;
-  const int grid = (int)(want < 152 * 16 ? want : 152 * 16);
-  return launch_pdl(quant_int4_kernel, dim3(grid), dim3(256), 0, st,
+  const int64_t want = (total + 4 * kQuantThreads - 1) / (4 * kQuantThreads);
+  const int64_t cap = (int64_t)device_sm_count() * 16;
+  return launch_pdl(quant_int4_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kQuantThreads), 0, st,
                     reinterpret_cast<const __half*>(w), N, K, reinterpret_cast<uint8_t*>(codes),
                     reinterpret_cast<__half*>(scales));
 }
@@ -139,9 +259,13 @@ cudaError_t launch_quant_int4(const void* w, int64_t N, int64_t K, void* codes, 
 cudaError_t launch_quant_fp8(const void* w, int64_t N, int64_t K, void* codes, void* scales,
                              cudaStream_t st) {
   if (N == 0) return cudaSuccess;
-  const int grid = (int)(N < 152 * 8 ? N : 152 * 8);
-  return launch_pdl(quant_fp8_kernel, dim3(grid), dim3(256), 0, st,
-                    reinterpret_cast<const __half*>(w), N, K, reinterpret_cast<uint8_t*>(codes),
+  // a warp per row while its registers hold the row, else a CTA
+  const bool one_warp = K <= 32 * 8 * kFp8Keep;
+  const int rpc = one_warp ? kQuantThreads / 32 : 1;
+  const int64_t want = (N + rpc - 1) / rpc, cap = (int64_t)device_sm_count() * 8;
+  const dim3 grid((unsigned)(want < cap ? want : cap));
+  return launch_pdl(one_warp ? quant_fp8_kernel<32> : quant_fp8_kernel<kQuantThreads>, grid, dim3(kQuantThreads),
+                    0, st, reinterpret_cast<const __half*>(w), N, K, reinterpret_cast<uint8_t*>(codes),
                     reinterpret_cast<float*>(scales));
 }
 
