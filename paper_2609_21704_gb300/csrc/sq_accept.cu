@@ -71,6 +71,45 @@ __device__ __forceinline__ float exp_neg(float x) {
   return __fmul_rn(__fmul_rn(p, __uint_as_float((uint32_t)(ni + 127 + 64) << 23)), 0x1p-64f);
 }
 
+// exp_neg for the sums over a row: x is clamped at -80 (rintf as the sum with
+// 1.5 2^23, the same nearest-even integer).  A probability below e^-80 counts
+// for nothing: it adds no 2^-44, and changes no difference p - q that does.
+__device__ __forceinline__ float exp_neg_sum(float x) {
+  x = fmaxf(x, -80.0f);
+  const float magic = 12582912.0f;
+  const float tn = __fadd_rn(__fmul_rn(x, 0x1.715476p+0f), magic);
+  const float n = tn - magic;
+  float r = __fmaf_rn(-n, 0x1.62e4p-1f, x);
+  r = __fmaf_rn(-n, 0x1.7f7d1cp-20f, r);
+  float p = 0x1.a01a02p-13f;
+  p = __fmaf_rn(p, r, 0x1.6c16c2p-10f);
+  p = __fmaf_rn(p, r, 0x1.111112p-7f);
+  p = __fmaf_rn(p, r, 0x1.555556p-5f);
+  p = __fmaf_rn(p, r, 0x1.555556p-3f);
+  p = __fmaf_rn(p, r, 0.5f);
+  p = __fmaf_rn(p, r, 1.0f);
+  p = __fmaf_rn(p, r, 1.0f);
+  return __uint_as_float(__float_as_uint(p) + (__float_as_uint(tn) << 23));  // p 2^n, exact
+}
+__device__ __forceinline__ float logit_prob_sum(__half z, float m, float invT, float s) {
+  return __fdiv_rn(exp_neg_sum(__fmul_rn(__fsub_rn(__half2float(z), m), invT)), s);
+}
+
+// Partial sums of floor(r 2^44), r in [0, 1], as two 22-bit parts: hi is the
+// floor of r 2^22, lo that of the (exact) rest times 2^22; the sums carry the
+// bias 2^23 of every addition (kFix44Bias, as fp32 bits), up to 64 of them fit.
+constexpr uint32_t kFix44Bias = 0x4b000000u;
+__device__ __forceinline__ void add_fix44(float r, uint32_t& hi, uint32_t& lo) {
+  const float e22 = __fmul_rn(r, 4194304.0f);
+  const float th = __fadd_rz(e22, 8388608.0f);
+  hi += __float_as_uint(th);
+  const float rem = __fsub_rn(e22, __fsub_rn(th, 8388608.0f));
+  lo += __float_as_uint(__fadd_rz(__fmul_rn(rem, 4194304.0f), 8388608.0f));
+}
+__device__ __forceinline__ unsigned long long fix44_total(uint32_t hi, uint32_t lo, uint32_t count) {
+  return ((unsigned long long)(hi - count * kFix44Bias) << 22) + (lo - count * kFix44Bias);
+}
+
 // p_v = e_v / s with e_v = exp_neg((z_v - m) * invT) (fp32 subtract, multiply,
 // divide, each rounded to nearest).
 __device__ __forceinline__ float logit_prob(__half z, float m, float invT, float s) {
@@ -97,6 +136,7 @@ struct ProbRow {
   }
 };
 struct ProbSrc {
+  static constexpr bool kUnit = false;  // the caller's numbers, summed as they come
   const float* p;  // [B, K+1, V]
   const float* q;  // [B, K, V] or null
   int K;
@@ -128,6 +168,26 @@ struct LogitRow {
       for (int j = 0; j < 8; ++j) out[j] = v + j < vend ? logit_prob(z[v + j], m, invT, s) : 0.0f;
     }
   }
+  // the same in two steps, for sums: the bits of the entries, then their probabilities
+  __device__ __forceinline__ uint4 raw8(int64_t v, int64_t vend) const {
+    if (v + 8 <= vend && ((reinterpret_cast<uintptr_t>(z + v) & 15u) == 0)) return *reinterpret_cast<const uint4*>(z + v);
+    uint32_t h[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) h[j] = v + j < vend ? __half_as_ushort(z[v + j]) : 0u;
+    return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+  }
+  __device__ __forceinline__ void sum8(const uint4 w, int64_t v, int64_t vend, float out[8]) const {
+    const uint32_t h[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      out[2 * j] = logit_prob_sum(__ushort_as_half(lo16(h[j])), m, invT, s);
+      out[2 * j + 1] = logit_prob_sum(__ushort_as_half(hi16(h[j])), m, invT, s);
+    }
+    if (v + 8 > vend)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (v + j >= vend) out[j] = 0.0f;
+  }
 };
 
 // The 8 fp16 values [v, v + 8) of a row as fp32; entries at or past vend are
@@ -152,6 +212,7 @@ __device__ __forceinline__ void load8_half(const __half* z, int64_t v, int64_t v
   }
 }
 struct LogitSrc {
+  static constexpr bool kUnit = true;  // entries are e / s with e <= 1 <= s
   const __half* zp;  // [B, K+1, V]
   const __half* zq;  // [K, B, V]
   const float* m;    // row maxima: target rows b (K+1) + i, then draft rows B (K+1) + i B + b
@@ -265,6 +326,7 @@ __device__ __forceinline__ unsigned long long block_excl_scan_u64(unsigned long 
 }
 
 constexpr int kAcceptThreads = 256;
+constexpr int kAcceptMaxCpc = 4;  // chunks of one CTA at most
 static_assert(kAcceptChunk == 8 * kAcceptThreads, "a thread owns 8 consecutive entries of a chunk");
 static_assert(kSoftmaxChunk == 8 * kAcceptThreads, "a thread owns 8 consecutive entries of a chunk");
 
@@ -280,15 +342,15 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   __shared__ int s_chunk, s_use_p, s_token;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t bc = blockIdx.x;
-  const int b = (int)(bc / a.C), c = (int)(bc - (int64_t)b * a.C);
+  // this CTA: chunks [cb, ce) of sequence b
+  const int ctas = (a.C + a.cpc - 1) / a.cpc;
+  const int b = (int)(blockIdx.x / (unsigned)ctas);
+  const int cb = (int)(blockIdx.x - (unsigned)b * ctas) * a.cpc;
+  const int ce = cb + a.cpc < a.C ? cb + a.cpc : a.C;
   const int K = a.K;
   const int64_t V = a.V;
   const int32_t* xb = a.draft + (int64_t)b * K;
   const float* ub = a.u + (int64_t)b * (K + 1);
-  const int64_t v0 = (int64_t)c * a.chunk;
-  const int64_t v1 = v0 + a.chunk < V ? v0 + a.chunk : V;
-  unsigned long long* part = a.part + ((int64_t)b * a.C + c) * a.slots;
 
   // ---- validity and (sampling) the accept tests, evaluated by warp 0
   if (warp == 0) {
@@ -310,75 +372,122 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
     if (lane == 0) {
       s_valid = (bad_mask == 0u) && !bad_u && !rows_mask;
       s_n = rej_mask ? (__ffs(rej_mask) - 1) : K;
-      if (c == 0 && bad_mask) atomicOr(&g_accept_status, SQ_DEV_BAD_DRAFT_TOKEN);
-      if (c == 0 && bad_u) atomicOr(&g_accept_status, SQ_DEV_BAD_UNIFORM);
+      if (cb == 0 && bad_mask) atomicOr(&g_accept_status, SQ_DEV_BAD_DRAFT_TOKEN);
+      if (cb == 0 && bad_u) atomicOr(&g_accept_status, SQ_DEV_BAD_UNIFORM);
     }
   }
   __syncthreads();
   const int n = s_n;
 
   // ---- chunk partials
-  if (a.mode == SQ_ACCEPT_SAMPLE) {
-    const auto pn = src.prow(b, n);
-    const bool use_q = n < K;
-    const auto qn = src.qrow(b, use_q ? n : 0);
-    unsigned long long sr = 0, sp = 0;
-    // thread t: the 8 entries [v0 + 8t, v0 + 8t + 8) of the chunk
-    for (int64_t vb = v0 + 8 * (int64_t)tid; vb < v1; vb += 8 * kAcceptThreads) {
-      float pv[8], qv[8];
-      pn.load8(vb, v1, pv);
-      if (use_q) qn.load8(vb, v1, qv);
+  if constexpr (Src::kUnit) {
+    if (a.mode == SQ_ACCEPT_SAMPLE) {
+      // all of the CTA's chunks at once: their loads, their sums, one barrier.
+      // (The row's own mass, for a residual without any, is summed only if it
+      // turns out to be wanted.)
+      const auto pn = src.prow(b, n);
+      const bool use_q = n < K;
+      const auto qn = src.qrow(b, use_q ? n : 0);
+      uint4 pr[kAcceptMaxCpc], qr[kAcceptMaxCpc];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (use_q) {
-          const float d = pv[j] - qv[j];
-          sr += fix44(d > 0.0f ? d : 0.0f);
-          sp += fix44(pv[j]);
-        } else {
-          sr += fix44(pv[j]);
+      for (int i = 0; i < kAcceptMaxCpc; ++i) {
+        const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
+        if (cb + i < ce && v < V) {
+          pr[i] = pn.raw8(v, V);
+          if (use_q) qr[i] = qn.raw8(v, V);
         }
       }
-    }
-    sr = warp_sum_u64(sr);
-    sp = warp_sum_u64(sp);
-    if (lane == 0) {
-      red[warp][0] = sr;
-      red[warp][1] = sp;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      unsigned long long tr = 0, tp = 0;
-      for (int w = 0; w < kAcceptThreads / 32; ++w) {
-        tr += red[w][0];
-        tp += red[w][1];
+#pragma unroll
+      for (int i = 0; i < kAcceptMaxCpc; ++i) {
+        const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
+        unsigned long long sr = 0;
+        if (cb + i < ce && v < V) {
+          uint32_t hi = 0, lo = 0;
+          float pv[8], qv[8];
+          pn.sum8(pr[i], v, V, pv);
+          if (use_q) qn.sum8(qr[i], v, V, qv);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) add_fix44(use_q ? fmaxf(pv[j] - qv[j], 0.0f) : pv[j], hi, lo);
+          sr = fix44_total(hi, lo, 8);
+        }
+        sr = warp_sum_u64(sr);
+        if (lane == 0) red[warp][i] = sr;
       }
-      part[0] = tr;
-      part[1] = tp;
+      __syncthreads();
+      if (tid < ce - cb) {
+        unsigned long long tr = 0;
+        for (int w = 0; w < kAcceptThreads / 32; ++w) tr += red[w][tid];
+        a.part[((int64_t)b * a.C + cb + tid) * a.slots] = tr;
+      }
     }
-  } else {
-    // greedy: per position i, the maximum key over the chunk
-    for (int i = 0; i <= K; ++i) {
-      const auto pi = src.prow(b, i);
-      unsigned long long best = 0;
-      for (int64_t vb = v0 + 8 * (int64_t)tid; vb < v1; vb += 8 * kAcceptThreads) {
-        float pv[8];
-        pi.load8(vb, v1, pv);
+  }
+  for (int c = cb; c < ce && !(Src::kUnit && a.mode == SQ_ACCEPT_SAMPLE); ++c) {
+    const int64_t v0 = (int64_t)c * a.chunk;
+    const int64_t v1 = v0 + a.chunk < V ? v0 + a.chunk : V;
+    const int64_t vb = v0 + 8 * (int64_t)tid;  // thread t: the 8 entries [v0 + 8t, v0 + 8t + 8)
+    unsigned long long* part = a.part + ((int64_t)b * a.C + c) * a.slots;
+    if (a.mode == SQ_ACCEPT_SAMPLE) {
+      const auto pn = src.prow(b, n);
+      const bool use_q = n < K;
+      const auto qn = src.qrow(b, use_q ? n : 0);
+      unsigned long long sr = 0, sp = 0;
+      if (vb < v1) {
+        float pv[8], qv[8];
+        pn.load8(vb, v1, pv);
+        if (use_q) qn.load8(vb, v1, qv);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          if (vb + j >= v1) break;
-          const unsigned long long k = argmax_key(pv[j], vb + j);
-          best = k > best ? k : best;
+          if (use_q) {
+            const float d = pv[j] - qv[j];
+            sr += fix44(d > 0.0f ? d : 0.0f);
+            sp += fix44(pv[j]);
+          } else {
+            sr += fix44(pv[j]);
+          }
         }
       }
-      best = warp_max_u64(best);
-      if (lane == 0) red[warp][i] = best;
+      sr = warp_sum_u64(sr);
+      sp = warp_sum_u64(sp);
+      if (lane == 0) {
+        red[warp][0] = sr;
+        red[warp][1] = sp;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        unsigned long long tr = 0, tp = 0;
+        for (int w = 0; w < kAcceptThreads / 32; ++w) {
+          tr += red[w][0];
+          tp += red[w][1];
+        }
+        part[0] = tr;
+        part[1] = tp;
+      }
+    } else {
+      // greedy: per position i, the maximum key over the chunk
+      for (int i = 0; i <= K; ++i) {
+        const auto pi = src.prow(b, i);
+        unsigned long long best = 0;
+        if (vb < v1) {
+          float pv[8];
+          pi.load8(vb, v1, pv);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            if (vb + j >= v1) break;
+            const unsigned long long k = argmax_key(pv[j], vb + j);
+            best = k > best ? k : best;
+          }
+        }
+        best = warp_max_u64(best);
+        if (lane == 0) red[warp][i] = best;
+      }
+      __syncthreads();
+      if (tid <= K) {
+        unsigned long long best = 0;
+        for (int w = 0; w < kAcceptThreads / 32; ++w) best = red[w][tid] > best ? red[w][tid] : best;
+        part[tid] = best;
+      }
     }
-    __syncthreads();
-    if (tid <= K) {
-      unsigned long long best = 0;
-      for (int w = 0; w < kAcceptThreads / 32; ++w) best = red[w][tid] > best ? red[w][tid] : best;
-      part[tid] = best;
-    }
+    __syncthreads();  // red is written again
   }
 
   // ---- ticket: the last CTA of the sequence finishes it
@@ -386,7 +495,7 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   if (tid == 0) {
     __threadfence();
     const unsigned ticket = atomicAdd(&a.counter[b], 1u);
-    s_last = (ticket == (unsigned)(a.C - 1));
+    s_last = (ticket == (unsigned)(ctas - 1));
   }
   __syncthreads();
   if (!s_last) return;
@@ -433,8 +542,29 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   const int use_p = (S == 0 && n < K) ? 1 : 0;  // block-uniform
   unsigned long long m0 = r0, m1 = r1;
   if (use_p) {
-    m0 = partial(c0, 1);
-    m1 = partial(c1, 1);
+    if constexpr (Src::kUnit) {
+      // no mass in the residual (rare): the row's own, chunk by chunk
+      const auto pn = src.prow(b, n);
+      m0 = m1 = 0;
+      for (int c = 0; c < a.C; ++c) {
+        const int64_t v0 = (int64_t)c * a.chunk;
+        const int64_t v1 = v0 + a.chunk < V ? v0 + a.chunk : V;
+        const int64_t vb = v0 + 8 * (int64_t)tid;
+        unsigned long long sum = 0;
+        if (vb < v1) {
+          float pv[8];
+          pn.load8(vb, v1, pv);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) sum += fix44(pv[j]);
+        }
+        sum = block_sum_u64<kAcceptThreads>(sum, blk);
+        if (c == c0) m0 = sum;
+        if (c == c1) m1 = sum;
+      }
+    } else {
+      m0 = partial(c0, 1);
+      m1 = partial(c1, 1);
+    }
     S = block_sum_u64<kAcceptThreads>(m0 + m1, blk);
   }
   const int ok = s_valid && S != 0;
@@ -530,159 +660,248 @@ size_t accept_workspace_bytes(int B, int K, int64_t V) {
   return ctr + part + 16u;
 }
 
+// Chunks of one CTA: several (so that fewer CTAs repeat the accept tests and
+// the ticket) once that still leaves two CTAs per SM.
+static int accept_chunks_per_cta(const AcceptArgs& a) {
+  const int64_t per = (int64_t)a.B * a.C / (2 * (int64_t)device_sm_count());
+  return (int)(per < 1 ? 1 : per > kAcceptMaxCpc ? kAcceptMaxCpc : per);
+}
+
 cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t st) {
   if (a.B == 0) return cudaSuccess;
-  const int64_t blocks = (int64_t)a.B * a.C;
+  AcceptArgs b = a;
+  b.cpc = accept_chunks_per_cta(a);
   ProbSrc src{a.p, a.q, a.K, a.V};
-  return launch_pdl(accept_kernel<ProbSrc>, dim3((unsigned)blocks), dim3(kAcceptThreads), 0, st, a,
-                    src);
+  return launch_pdl(accept_kernel<ProbSrc>, dim3((unsigned)(a.B * ((a.C + b.cpc - 1) / b.cpc))),
+                    dim3(kAcceptThreads), 0, st, b, src);
 }
 
 // ---- softmax statistics of logit rows --------------------------------------
-// One CTA per (row, chunk of kSoftmaxChunk entries).  Pass 1: the row
-// maximum (a NaN marks a row holding a non-finite logit); pass 2: the
-// fixed-point normaliser S = sum_v floor(e_v 2^40) and s = float(S 2^-40).
-// The last CTA of a row (atomic ticket, counter left at zero) combines the
-// chunk partials; max and integer sums do not depend on their order.
+// A cluster of CTAs per row reads it once into registers: the row maximum
+// (NaN for a row holding a non-finite logit), the CTAs' maxima exchanged
+// through distributed shared memory, then the fixed-point normaliser S =
+// sum_v floor(e_v 2^40) and s = float(S 2^-40) from the same registers; max
+// and integer sums do not depend on the order.
 __device__ __forceinline__ const __half* softmax_row_ptr(const SoftmaxArgs& a, int64_t r) {
   return r < a.rp ? a.zp + r * a.V : a.zq + (r - a.rp) * a.V;
 }
 
-__global__ void __launch_bounds__(kAcceptThreads) softmax_max_kernel(SoftmaxArgs a) {
-  griddep_wait();
-  griddep_launch_dependents();
-  __shared__ float red[kAcceptThreads / 32];
-  __shared__ int red_bad[kAcceptThreads / 32];
-  __shared__ int s_last;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t r = blockIdx.x / a.C;
-  const int c = (int)(blockIdx.x - r * a.C);
-  const __half* z = softmax_row_ptr(a, r);
-  const int64_t v0 = (int64_t)c * kSoftmaxChunk;
-  const int64_t v1 = v0 + kSoftmaxChunk < a.V ? v0 + kSoftmaxChunk : a.V;
-  float mx = -INFINITY;
-  int bad = 0;
-  {
-    float f[8];
-    bool ok[8];
-    load8_half(z, v0 + 8 * (int64_t)tid, v1, f, ok);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (ok[j]) {
-        bad |= !isfinite(f[j]);
-        mx = fmaxf(mx, f[j]);
-      }
-  }
-  mx = warp_max(mx);
-  bad = __any_sync(0xffffffffu, bad);
-  if (lane == 0) {
-    red[warp] = mx;
-    red_bad[warp] = bad;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    float m = -INFINITY;
-    int any_bad = 0;
-    for (int w = 0; w < kAcceptThreads / 32; ++w) {
-      m = fmaxf(m, red[w]);
-      any_bad |= red_bad[w];
-    }
-    a.pmax[r * a.C + c] = any_bad ? __int_as_float(0x7fc00000) : m;
-    __threadfence();
-    s_last = atomicAdd(&a.counter[r], 1u) == (unsigned)(a.C - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  // the last CTA of the row: every thread takes chunks t and t + 256
-  float m = -INFINITY;
-  int nan = 0;
-  for (int cc = tid; cc < a.C; cc += kAcceptThreads) {
-    const float pm = __ldcg(a.pmax + r * a.C + cc);
-    nan |= isnan(pm);
-    m = fmaxf(m, pm);
-  }
-  m = warp_max(m);
-  nan = __any_sync(0xffffffffu, nan);
-  __syncthreads();
-  if (lane == 0) {
-    red[warp] = m;
-    red_bad[warp] = nan;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    float mm = -INFINITY;
-    int any_nan = 0;
-    for (int w = 0; w < kAcceptThreads / 32; ++w) {
-      mm = fmaxf(mm, red[w]);
-      any_nan |= red_bad[w];
-    }
-    if (any_nan) {
-      mm = __int_as_float(0x7fc00000);
-      atomicOr(&g_accept_status, SQ_DEV_NONFINITE_LOGIT);
-    }
-    a.m[r] = mm;
-    a.counter[r] = 0u;
-  }
+// floor(e 2^40) of e = exp_neg(x) as (hi, lo) 20-bit parts, added to the two
+// sums with the bias kFixBias each.  The steps of exp_neg down to the scaling,
+// with rintf as the sum with 1.5 2^23 (the same nearest-even integer, whose
+// low bits then hold n + 20); below x = -28 the term is zero, so the clamp
+// keeps every scale in the normal range.  p 2^(n + 20) is exact, and so are
+// the differences, so the parts are those of the definition.
+constexpr uint32_t kFixBias = 0x4b000000u;  // 2^23 as fp32 bits
+__device__ __forceinline__ void add_fix40(float x, uint32_t& hi, uint32_t& lo) {
+  x = fmaxf(x, -29.0f);
+  const float magic = 12582912.0f + 20.0f;
+  const float tn = __fadd_rn(__fmul_rn(x, 0x1.715476p+0f), magic);
+  const float n = tn - magic;
+  float r = __fmaf_rn(-n, 0x1.62e4p-1f, x);
+  r = __fmaf_rn(-n, 0x1.7f7d1cp-20f, r);
+  float p = 0x1.a01a02p-13f;
+  p = __fmaf_rn(p, r, 0x1.6c16c2p-10f);
+  p = __fmaf_rn(p, r, 0x1.111112p-7f);
+  p = __fmaf_rn(p, r, 0x1.555556p-5f);
+  p = __fmaf_rn(p, r, 0x1.555556p-3f);
+  p = __fmaf_rn(p, r, 0.5f);
+  p = __fmaf_rn(p, r, 1.0f);
+  p = __fmaf_rn(p, r, 1.0f);
+  const float e20 = __uint_as_float(__float_as_uint(p) + (__float_as_uint(tn) << 23));  // e 2^20
+  const float th = __fadd_rz(e20, 8388608.0f);
+  hi += __float_as_uint(th);
+  const float rem = __fsub_rn(e20, __fsub_rn(th, 8388608.0f));
+  lo += __float_as_uint(__fadd_rz(__fmul_rn(rem, 1048576.0f), 8388608.0f));
 }
 
-__global__ void __launch_bounds__(kAcceptThreads) softmax_sum_kernel(SoftmaxArgs a) {
+__device__ __forceinline__ void stats_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned long long stats_ld_rank(const unsigned long long* local, uint32_t rank) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
+  unsigned long long v;
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(remote) : "memory");
+  return v;
+}
+
+constexpr int kStatsKeep = 10;  // 16-byte pieces of the row a thread keeps
+constexpr int kStatsMaxCluster = 16;
+
+// One cluster of CL CTAs per row.  Against two launches of one CTA per 2048
+// entries (38 + 83 us for 272 rows of 152064 entries) the row is read once and
+// there is one launch and no ticket: 53 us.  Bound: issue slots, 32
+// instructions an entry at 70 % of the issue rate; memory time is 12 us.
+__global__ void __launch_bounds__(kAcceptThreads) softmax_stats_kernel(SoftmaxArgs a, int CL) {
   griddep_wait();
   griddep_launch_dependents();
-  __shared__ unsigned long long red[kAcceptThreads / 32];
-  __shared__ int s_last;
+  __shared__ float redm[kAcceptThreads / 32];
+  __shared__ int redb[kAcceptThreads / 32];
+  __shared__ unsigned long long blk[kAcceptThreads / 32];
+  __shared__ unsigned long long s_max, s_sum;  // read by the cluster's other CTAs
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t r = blockIdx.x / a.C;
-  const int c = (int)(blockIdx.x - r * a.C);
+  const int64_t r = blockIdx.x / CL;
+  const int rank = (int)(blockIdx.x - r * CL);
   const __half* z = softmax_row_ptr(a, r);
-  const int64_t v0 = (int64_t)c * kSoftmaxChunk;
-  const int64_t v1 = v0 + kSoftmaxChunk < a.V ? v0 + kSoftmaxChunk : a.V;
-  const float m = a.m[r];
-  unsigned long long acc = 0;
-  if (isfinite(m)) {
-    float f[8];
-    bool ok[8];
-    load8_half(z, v0 + 8 * (int64_t)tid, v1, f, ok);
+  const int V = (int)a.V;
+  const int npc = (V + 7) / 8;  // pieces of 8 entries; this thread's: i (CL 256) + rank 256 + tid
+  const int first = rank * kAcceptThreads + tid, stride = CL * kAcceptThreads;
+  const bool vec = (reinterpret_cast<uintptr_t>(z) & 15u) == 0;
+  // a piece's entries as fp16 bits; entries past the row repeat `pad`
+  auto piece = [&](int p, uint32_t pad) -> uint4 {
+    if (vec && 8 * p + 8 <= V) return *reinterpret_cast<const uint4*>(z + 8 * p);
+    uint32_t h[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (ok[j]) acc += fixq<40>(exp_neg(__fmul_rn(__fsub_rn(f[j], m), a.invT)));
+    for (int j = 0; j < 8; ++j) h[j] = 8 * p + j < V ? __half_as_ushort(z[8 * p + j]) : pad;
+    return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+  };
+  uint4 keep[kStatsKeep];
+#pragma unroll
+  for (int i = 0; i < kStatsKeep; ++i)
+    if (first + i * stride < npc) keep[i] = piece(first + i * stride, 0xfbffu);  // pad: the lowest finite value
+  __half2 mx = __half2half2(__ushort_as_half(0xfbffu));
+  uint32_t ab = 0;
+  auto fold = [&](const uint4 v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      mx = __hmax2(mx, *reinterpret_cast<const __half2*>(&w[j]));
+      ab = __vmaxu2(ab, w[j] & 0x7fff7fffu);
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < kStatsKeep; ++i)
+    if (first + i * stride < npc) fold(keep[i]);
+  for (int p = first + kStatsKeep * stride; p < npc; p += stride) fold(piece(p, 0xfbffu));
+  float m = warp_max(fmaxf(__low2float(mx), __high2float(mx)));
+  int bad = __any_sync(0xffffffffu, max(ab & 0xffffu, ab >> 16) >= 0x7c00u);
+  if (lane == 0) {
+    redm[warp] = m;
+    redb[warp] = bad;
   }
-  acc = warp_sum_u64(acc);
-  if (lane == 0) red[warp] = acc;
   __syncthreads();
-  if (tid == 0) {
-    unsigned long long t = 0;
-    for (int w = 0; w < kAcceptThreads / 32; ++w) t += red[w];
-    a.psum[r * a.C + c] = t;
-    __threadfence();
-    s_last = atomicAdd(&a.counter[r], 1u) == (unsigned)(a.C - 1);
+  m = redm[0];
+  bad = redb[0];
+#pragma unroll
+  for (int w = 1; w < kAcceptThreads / 32; ++w) {
+    m = fmaxf(m, redm[w]);
+    bad |= redb[w];
+  }
+  if (CL > 1) {
+    if (tid == 0) s_max = (unsigned long long)__float_as_uint(m) | ((unsigned long long)bad << 32);
+    stats_cluster_sync();
+    for (int q = 0; q < CL; ++q) {
+      const unsigned long long v = stats_ld_rank(&s_max, (uint32_t)q);
+      m = fmaxf(m, __uint_as_float((uint32_t)v));
+      bad |= (int)(v >> 32);
+    }
+  }
+  unsigned long long acc = 0;
+  if (!bad) {
+    auto sum = [&](const uint4 v, int p, uint32_t& hi, uint32_t& lo) {
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      float x[8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
+        x[2 * j] = __fmul_rn(__fsub_rn(f.x, m), a.invT);
+        x[2 * j + 1] = __fmul_rn(__fsub_rn(f.y, m), a.invT);
+      }
+      if (8 * p + 8 > V)  // the ragged last piece: x = -29 adds zero
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (8 * p + j >= V) x[j] = -29.0f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) add_fix40(x[j], hi, lo);
+    };
+    uint32_t hi = 0, lo = 0, cnt = 0;
+#pragma unroll
+    for (int i = 0; i < kStatsKeep; ++i)
+      if (first + i * stride < npc) {
+        sum(keep[i], first + i * stride, hi, lo);
+        cnt += 8;
+      }
+    // hi < 80 (2^20 + 1), lo < 80 2^20: no carry out of 32 bits
+    acc = ((unsigned long long)(hi - cnt * kFixBias) << 20) + (lo - cnt * kFixBias);
+    for (int p = first + kStatsKeep * stride; p < npc; p += stride) {
+      hi = lo = 0;
+      sum(piece(p, 0u), p, hi, lo);
+      acc += ((unsigned long long)(hi - 8 * kFixBias) << 20) + (lo - 8 * kFixBias);
+    }
+  }
+  unsigned long long S = block_sum_u64<kAcceptThreads>(acc, blk);
+  if (CL > 1) {
+    if (tid == 0) s_sum = S;
+    stats_cluster_sync();
+    if (rank == 0 && tid == 0)
+      for (int q = 1; q < CL; ++q) S += stats_ld_rank(&s_sum, (uint32_t)q);
+  }
+  if (rank == 0 && tid == 0) {
+    const float nan = __int_as_float(0x7fc00000);
+    if (bad) atomicOr(&g_accept_status, SQ_DEV_NONFINITE_LOGIT);
+    a.m[r] = bad ? nan : m;
+    a.s[r] = bad ? nan : __double2float_rn(__ull2double_rn(S) * 0x1p-40);
   }
   __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  unsigned long long part = 0;
-  for (int cc = tid; cc < a.C; cc += kAcceptThreads) part += __ldcg(a.psum + r * a.C + cc);
-  const unsigned long long S = block_sum_u64<kAcceptThreads>(part, red);
-  if (tid == 0) {
-    a.s[r] = isfinite(m) ? __double2float_rn(__ull2double_rn(S) * 0x1p-40)
-                         : __int_as_float(0x7fc00000);
-    a.counter[r] = 0u;
+  if (CL > 1) stats_cluster_sync();  // no CTA leaves while rank 0 reads its sum
+}
+
+static cudaError_t launch_stats(const SoftmaxArgs& sa, cudaStream_t st) {
+  // CTAs per row: one per 2048 entries, up to 8 (16 for few rows, where a row
+  // per 8 CTAs would leave most of the GPU idle)
+  const int64_t want = (sa.V + 8 * kAcceptThreads - 1) / (8 * kAcceptThreads);
+  const int most = sa.rows * kStatsMaxCluster <= 4 * device_sm_count() ? kStatsMaxCluster : 8;
+  const int CL = (int)(want < most ? want : most);
+  static std::mutex mu;
+  static bool ready[64] = {false};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!ready[dev]) {
+      e = cudaFuncSetAttribute(softmax_stats_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+      ready[dev] = true;
+    }
   }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(sa.rows * CL));
+  cfg.blockDim = dim3(kAcceptThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (CL > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)CL;
+    at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  const bool legacy = (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread);
+  if (!legacy && pdl_enabled()) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, softmax_stats_kernel, sa, CL);
 }
 
 cudaError_t launch_accept_logits(const AcceptArgs& a, const SoftmaxArgs& sa, cudaStream_t st) {
   if (a.B == 0) return cudaSuccess;
-  const int64_t sblocks = sa.rows * sa.C;
-  cudaError_t e = launch_pdl(softmax_max_kernel, dim3((unsigned)sblocks), dim3(kAcceptThreads), 0, st, sa);
-  if (e != cudaSuccess) return e;
-  e = launch_pdl(softmax_sum_kernel, dim3((unsigned)sblocks), dim3(kAcceptThreads), 0, st, sa);
+  cudaError_t e = launch_stats(sa, st);
   if (e != cudaSuccess) return e;
   LogitSrc src{sa.zp, sa.zq, sa.m, sa.s, sa.invT, a.B, a.K, a.V};
-  const int64_t blocks = (int64_t)a.B * a.C;
-  return launch_pdl(accept_kernel<LogitSrc>, dim3((unsigned)blocks), dim3(kAcceptThreads), 0, st, a,
-                    src);
+  AcceptArgs b = a;
+  b.cpc = accept_chunks_per_cta(a);
+  return launch_pdl(accept_kernel<LogitSrc>, dim3((unsigned)(a.B * ((a.C + b.cpc - 1) / b.cpc))),
+                    dim3(kAcceptThreads), 0, st, b, src);
 }
 
+// (room for the statistics; the rest of the documented size is not used)
 size_t softmax_rows_workspace_bytes(int64_t rows, int64_t V) {
   if (rows < 0 || V <= 0) return 0;
   const int64_t C = (V + kSoftmaxChunk - 1) / kSoftmaxChunk;
@@ -701,11 +920,8 @@ void softmax_layout(SoftmaxArgs& sa, void* ws) {
   char* sw = reinterpret_cast<char*>(ws);
   sa.C = (int)((sa.V + kSoftmaxChunk - 1) / kSoftmaxChunk);
   const size_t rows4 = up16((size_t)sa.rows * 4u);
-  sa.counter = reinterpret_cast<unsigned int*>(sw);
   sa.m = reinterpret_cast<float*>(sw + rows4);
   sa.s = reinterpret_cast<float*>(sw + 2 * rows4);
-  sa.pmax = reinterpret_cast<float*>(sw + 3 * rows4);
-  sa.psum = reinterpret_cast<unsigned long long*>(sw + 3 * rows4 + up16((size_t)sa.rows * sa.C * 4u));
 }
 
 // p[r, v] from the row statistics (the same expression the accept kernel
@@ -735,9 +951,7 @@ __global__ void __launch_bounds__(kAcceptThreads) softmax_write_kernel(SoftmaxAr
 cudaError_t launch_softmax(const SoftmaxArgs& sa, float* p, cudaStream_t st) {
   if (sa.rows == 0) return cudaSuccess;
   const int64_t sblocks = sa.rows * sa.C;
-  cudaError_t e = launch_pdl(softmax_max_kernel, dim3((unsigned)sblocks), dim3(kAcceptThreads), 0, st, sa);
-  if (e != cudaSuccess) return e;
-  e = launch_pdl(softmax_sum_kernel, dim3((unsigned)sblocks), dim3(kAcceptThreads), 0, st, sa);
+  cudaError_t e = launch_stats(sa, st);
   if (e != cudaSuccess) return e;
   return launch_pdl(softmax_write_kernel, dim3((unsigned)sblocks), dim3(kAcceptThreads), 0, st, sa, p);
 }

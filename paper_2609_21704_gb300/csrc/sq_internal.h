@@ -129,6 +129,7 @@ struct AcceptArgs {
   unsigned int* counter;     // [B]
   int C;                     // chunks per sequence
   int chunk;                 // vocabulary entries per chunk
+  int cpc;                   // chunks of one CTA
   int slots;                 // partial slots per chunk
 };
 constexpr int kAcceptChunk = 2048;
@@ -151,13 +152,10 @@ struct SoftmaxArgs {
   int C;                     // chunks per row
   float* m;                  // [rows] row maxima
   float* s;                  // [rows] normalisers
-  float* pmax;               // [rows * C]
-  unsigned long long* psum;  // [rows * C]
-  unsigned int* counter;     // [rows], zero on entry, left zero
 };
 size_t softmax_rows_workspace_bytes(int64_t rows, int64_t V);
 size_t softmax_workspace_bytes(int B, int K, int64_t V);
-// Points sa's counter / m / s / partial arrays into ws (sa.rows, sa.V set).
+// Points sa's m / s arrays into ws (sa.rows, sa.V set).
 void softmax_layout(SoftmaxArgs& sa, void* ws);
 cudaError_t launch_accept_logits(const AcceptArgs& a, const SoftmaxArgs& sa, cudaStream_t st);
 cudaError_t launch_softmax(const SoftmaxArgs& sa, float* p, cudaStream_t st);
