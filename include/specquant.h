@@ -125,12 +125,14 @@ SQ_API sq_status sq_quantize(const void* w16, int64_t N, int64_t K, sq_qkind kin
  * nearest fp16 once.  1 <= M <= 256; N >= 1; K as for sq_quantize (INT4:
  * K % 128 == 0, FP8: K % 16 == 0, FP16: K % 8 == 0).  x, codes, w16 and y
  * must be 16-byte aligned.  Each call runs on one of these engines, chosen
- * from (format, M, N, K, epilogue) alone (sq_linear_path reports which):
+ * from (format, M, N, K, epilogue) alone (sq_linear_path reports the class):
  * the CUDA-core GEMV family for few rows (for one INT4 row over many output
  * rows, with its products on the tensor cores' register-operand path), the
- * shared-memory ring engine for one to eight rows of large or quantised
- * weights, and the tcgen05 tensor-core tile path from 16 rows on and, below
- * that, for the formats and shapes where it is faster.  All give the same
+ * shared-memory ring engine for one row of large weights, the streaming
+ * engine for most calls of two to sixteen rows (weights through a ring of
+ * asynchronous copies, register-operand tensor cores), and the tcgen05
+ * tensor-core tile path from 16 rows on and, below that, for the formats and
+ * shapes where it is faster.  All give the same
  * fp32-accumulated result up to summation order.
  * y must not overlap x, the weights or the scales.
  * ---------------------------------------------------------------------- */
@@ -174,13 +176,15 @@ SQ_API sq_status sq_linear_norm(sq_wkind wkind, const void* x, const void* gamma
                                 const void* w, const void* scales, const void* bias, const void* residual,
                                 sq_epilogue epi, void* y, int M, int64_t N, int64_t K, sq_stream_t stream);
 
-/* Engine sq_linear_ex would use for these sizes: 1 = tcgen05 tensor cores,
- * 0 = CUDA-core GEMV, 2 = one INT4 activation row over at least 192 16-row
- * output tiles with the products on the tensor cores' register-operand path
- * (mma.sync), 3 = one to eight activation rows streamed through a
- * shared-memory ring of asynchronous copies, products on the same
- * register-operand path,
- * -1 = sizes or kinds sq_linear_ex rejects (pointers are not examined;
+/* Class of engine for these sizes: 1 = tensor-core tiles (tcgen05), 0 = few
+ * rows of a small matrix (CUDA-core GEMV), 2 = one INT4 activation row over at
+ * least 192 16-row output tiles with the products on the tensor cores'
+ * register-operand path (mma.sync), 3 = one to eight activation rows streamed
+ * through a shared-memory ring of asynchronous copies, products on the same
+ * register-operand path.  Inside a class a call may run on the streaming
+ * engine instead (a ring of asynchronous copies and the register-operand path
+ * too): most calls of two to sixteen rows, and the largest INT4 lm_heads at
+ * one row.  -1 = sizes or kinds sq_linear_ex rejects (pointers are not examined;
  * nothing runs on the device).  The paper has no counterpart: this is
  * introspection for tests and tuning. */
 SQ_API int sq_linear_path(sq_wkind wkind, int M, int64_t N, int64_t K, sq_epilogue epi);

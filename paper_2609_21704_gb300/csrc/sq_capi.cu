@@ -193,6 +193,11 @@ static sq_status run_linear(const sq_linear_op& op, cudaStream_t stream, const _
   cudaError_t e;
   // the ring engine where the planner sends it, else the tcgen05 tile path,
   // else the GEMV family (sq_plan.cu)
+  if (use_stream(op.wkind, op.M, op.N, op.K, op.epi)) {
+    e = launch_stream(op.wkind, a, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "sq_linear: launch");
+    return SQ_OK;
+  }
   const bool ring = use_ring(op.wkind, op.M, op.N, op.K, op.epi);
   const bool tc = !ring && use_tensor_cores(op.wkind, op.M, op.N, op.K, op.epi) &&
                   tc_supported(op.M, op.K, op.epi);

@@ -102,6 +102,13 @@ cudaError_t launch_tc(int wkind, const __half* x, const void* w, const void* sca
                       cudaStream_t st);
 cudaError_t take_tc_status(uint32_t* bits);
 
+// sq_stream.cu: up to sixteen activation rows, weights streamed once, products
+// on the register-operand tensor path.  gamma: x is normalised while staged.
+// use_stream (sq_plan.cu): where it runs instead of the engines below.
+bool stream_supported(int wkind, int M, int64_t N, int64_t K, int epi);
+bool use_stream(int wkind, int M, int64_t N, int64_t K, int epi);
+cudaError_t launch_stream(int wkind, const GemvArgs& a, cudaStream_t st);
+
 // sq_ring.cu: one to eight activation rows streamed through a shared-memory
 // ring, products on the register-operand tensor path (mma.sync).
 bool ring_supported(int wkind, int M, int64_t K);

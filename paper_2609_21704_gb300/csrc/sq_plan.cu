@@ -186,4 +186,49 @@ bool use_ring(int wkind, int M, int64_t N, int64_t K, int epi) {
   return false;
 }
 
+// The streaming engine (sq_stream.cu) where it measured faster than whatever
+// ran before (us a launch, weights cold, PDL graph of the same call; 1.5B, 7B
+// and 14B projections at 1 .. 5, 8, 9, 12 and 16 rows):
+//   INT4, one row: the lm_head of >= 400 Mi weights (14B 80.5 -> 72.0); smaller
+//     matrices stay on the GEMV family, whose lanes need no partial sums (1.5B
+//     q/k/v 2.4 against 3.3), and the fused gate/up on the ring (alone it gains,
+//     22.4 -> 17.6, but between launches of the GEMV family the four 14B layers
+//     take 253 us instead of 196);
+//   INT4 and FP8, 2 .. 8 rows: everything (14B q/k/v INT4 at 2 rows 10.6 -> 8.5,
+//     down FP8 at 8 rows 36.8 -> 17.2) but the FP8 lm_head of >= 200 Mi, which
+//     the ring streams as fast as memory gives (14B 131 against 137, 1.5B 49
+//     against 51);
+//   INT4 and FP8, 9 .. 16 rows: everything (14B lm_head INT4 at 16 rows 192 ->
+//     138, down FP8 at 16 38.4 -> 21.1) but long rows of small matrices (0.5B
+//     down FP8 5.7 against 7.2) and, from 13 rows on, long rows of FP8 (7B down
+//     21.6 against 25.0), narrow mid-sized FP8 (7B q/k/v 9.1 against 10.0) and
+//     the smallest INT4 matrices (1.5B o 4.6 against 6.1);
+//   FP16, 2 .. 8 rows: at two rows the fused gate/up and the lm_head (14B lm_head
+//     384 -> 253); from three rows on matrices of 8 Mi weights and more with K <
+//     8192 (14B o at five rows 16.3 -> 12.0; from 32 Mi up to five rows: 14B
+//     q/k/v at eight 15.2 against 16.2), the 14B down shape (36.9 -> 27.4),
+//     and, where the tile path's 128-row tiles are few, fused gate/up below 64 Mi
+//     (1.5B at five 12.5 -> 11.2) and lm_heads below 400 Mi (1.5B 96.6 -> 80.4);
+//     small matrices from six rows on (1.5B q/k/v at eight 5.5 -> 3.8).
+bool use_stream(int wkind, int M, int64_t N, int64_t K, int epi) {
+  if (!stream_supported(wkind, M, N, K, epi)) return false;
+  const bool silu = epi == SQ_EPI_SILU_GATE;
+  const int64_t Mi = (int64_t)1 << 20;
+  const int64_t weights = (silu ? 2 * N : N) * K;
+  const bool head = !silu && N >= 65536;
+  if (M == 1) return wkind == SQ_W_INT4 && head && weights >= 400 * Mi;
+  if (wkind == SQ_W_FP16) {
+    if (M > 8) return false;
+    if (silu) return weights < 64 * Mi ? weights >= 16 * Mi || M >= 6 : M == 2;
+    if (head) return weights < 400 * Mi ? M >= 3 : M == 2;
+    if (K >= 8192) return M >= 3 && N >= 4096 && K < 16384;
+    if (K >= 4096 && weights < 8 * Mi) return false;
+    return M >= (weights >= 8 * Mi ? 3 : 6) && !(M >= 6 && weights >= 32 * Mi);
+  }
+  if (M <= 8) return !(wkind == SQ_W_FP8 && head && weights >= 200 * Mi);
+  if (K >= 4096 && weights < 8 * Mi) return false;
+  if (M >= 13) return wkind == SQ_W_FP8 ? K < 16384 && (K < 3072 || N > 6144 || weights < 14 * Mi) : weights >= 3 * Mi;
+  return true;
+}
+
 }  // namespace sq
