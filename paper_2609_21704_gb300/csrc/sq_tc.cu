@@ -11,12 +11,12 @@
 // Both operands are K-major fp16 tiles of 64 k (128 bytes per row) loaded by
 // 2-D TMA with 128-byte swizzle into a ring of shared-memory stages; warp 0
 // lane 0 issues the TMA copies, warp 1 lane 0 issues tcgen05.mma (4 x K16
-// per stage) and commits each stage back to the producer; warps 2..5 read
-// the accumulator with tcgen05.ld (each warp its 32-lane TMEM sub-partition)
-// and run the epilogue.  With the fused SiLU gate the CTA also loads the up
+// per stage) and commits each stage back to the producer; warps 2..9 read
+// the accumulator with tcgen05.ld (each warp half the columns of its 32-lane
+// TMEM sub-partition) and run the epilogue.  With the fused SiLU gate the CTA also loads the up
 // rows' tile and accumulates a second NB-column block of TMEM.
 //
-// FP8 and INT4 weights: TMA brings the code tiles instead, and the four
+// FP8 and INT4 weights: TMA brings the code tiles instead, and the eight
 // epilogue warps (idle until the accumulator is final) dequantise each stage
 // into the swizzled fp16 A tile (generic stores, fence.proxy.async, then an
 // mbarrier arrive that releases the stage to the MMA thread).  FP8: exact
@@ -51,13 +51,18 @@ static __device__ unsigned int g_tc_status;
 
 constexpr int kTcBM = 128;      // weight rows per tile (MMA M)
 constexpr int kTcBK = 64;       // k per stage: 64 fp16 = one 128-byte swizzle row
-// Warp roles: warp 0 TMA, warp 1 MMA + TMEM, warps 2..5 epilogue (one TMEM
-// sub-partition each).  Quantised weights add converter warps: warps 2..
-// 2 + warps - 1 dequantise each stage (two per SM sub-partition, so that
-// one's dependent chain hides behind the other's).
+// Warp roles: warp 0 TMA, warp 1 MMA + TMEM, warps 2..9 the epilogue (two per
+// TMEM sub-partition, half of the columns each) and, for quantised weights,
+// the conversion of every stage before it (two per SM sub-partition, so that
+// one's dependent chain hides behind the other's).  What follows the last MMA
+// is latency bound (TMEM loads, the gate's exponential and quotient, cluster
+// loads of the partials), so warps hide it: FP16 weights, four such warps ->
+// eight, four layers (28 at 1.5B) per pass: 14B at 256 rows 817 -> 682 us, at
+// 80 rows (and lm_head) 794 -> 759; 7B at 256 1182 -> 963; 1.5B at 256
+// 3576 -> 2529; 14B at 16 rows 734 -> 730.
 template <int WK>
 struct TcConv {
-  static constexpr int warps = WK == 0 ? 4 : 8;
+  static constexpr int warps = 8;
   static constexpr int threads = 64 + 32 * warps;
 };
 constexpr int kTcStageA = kTcBM * kTcBK * 2;  // 16 KB
@@ -414,7 +419,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       }
     }
   }
-  if (warp >= 2 && warp < 6) {
+  if (warp >= 2) {
     // --------------------------------------------------------- epilogue
     if (!mbar_wait_bounded(accf, 0u)) {
       timed_out = true;
@@ -425,8 +430,12 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     const int row = q * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
     const int64_t n = tile * kTcBM + row;
+    // this warp's columns: the first or second half, in whole 16s
+    const int cols = S == 1 ? a.NB : a.NB * (SILU ? 2 : 1);
+    const int cmid = (cols / 16 + 1) / 2 * 16;
+    const int cb = warp < 6 ? 0 : cmid, ce = warp < 6 ? cmid : cols;
     if (S == 1) {
-      for (int c0 = 0; c0 < a.NB; c0 += 16) {
+      for (int c0 = cb; c0 < ce; c0 += 16) {
         float g[16], u[16];
         tc_ld16(taddr + (uint32_t)c0, g);
         if (SILU) tc_ld16(taddr + (uint32_t)(a.NB + c0), u);
@@ -453,8 +462,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       // partial tile -> this CTA's shared memory, [column][row] (stages are
       // free: every MMA has completed)
       float* part = reinterpret_cast<float*>(stages);
-      const int cols = a.NB * (SILU ? 2 : 1);
-      for (int c0 = 0; c0 < cols; c0 += 16) {
+      for (int c0 = cb; c0 < ce; c0 += 16) {
         float v[16];
         tc_ld16(taddr + (uint32_t)c0, v);
 #pragma unroll
