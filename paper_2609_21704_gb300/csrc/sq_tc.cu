@@ -145,23 +145,15 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
-__device__ __forceinline__ float ld_dsmem_f32(const float* local, uint32_t rank) {
+// Stores to the shared memory of CTA `rank` of the cluster at the place where
+// `addr` (a shared address) lies in this CTA's.
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-  return v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+  return remote;
 }
-// Four consecutive floats (16-byte aligned) of CTA `rank`'s shared memory.
-__device__ __forceinline__ float4 ld_dsmem_f32x4(const float* local, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(remote)
-               : "memory");
-  return v;
+__device__ __forceinline__ void st_dsmem_f32(uint32_t remote, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
 }
 
 // ---------------------------------------------------------------- kernel
@@ -182,7 +174,6 @@ struct TcArgs {
   int b_off;        // offset of B inside a stage
   int c_off;        // offset of the code tiles inside a stage (FP8 / INT4)
   int c_bytes;      // bytes of one code tile
-  int part_stride;  // floats between columns of the partial tile
   int sc_off;       // INT4: byte offset of the CTA's group-scale block
   int sc_ng;        // INT4: groups per row held in the block (>= any CTA's need)
   int max_split;    // largest split-K factor whose partial tile fits in the stages
@@ -426,6 +417,14 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       if (lane == 0) atomicOr(&g_tc_status, SQ_DEV_TIMEOUT);
     }
     tc_fence_after();
+  }
+  if (S > 1) {
+    // every CTA's MMAs are done: the stages of all of them are free
+    __syncwarp();
+    cluster_sync();
+  }
+  const int cper = (a.M + S - 1) / S;  // columns of the output each rank finishes
+  if (warp >= 2) {
     const int q = warp & 3;  // TMEM sub-partition this warp may read
     const int row = q * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
@@ -459,112 +458,91 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
         }
       }
     } else {
-      // partial tile -> this CTA's shared memory, [column][row] (stages are
-      // free: every MMA has completed)
-      float* part = reinterpret_cast<float*>(stages);
+      // Column m of the partial tile goes straight from TMEM to the rank that
+      // finishes it, m / cper, at [this rank][m % cper][row]: a warp's store
+      // is 32 consecutive rows, 128 bytes of one column, and nothing waits
+      // for it before the barrier.  SiLU: up columns behind the gate ones.
       for (int c0 = cb; c0 < ce; c0 += 16) {
         float v[16];
         tc_ld16(taddr + (uint32_t)c0, v);
+        const int up = SILU && c0 >= a.NB ? 1 : 0;
+        const int m0 = c0 - up * a.NB;
+        int owner = m0 / cper, mc = m0 - owner * cper;
+        const uint32_t base =
+            smem_u32(stages) + (uint32_t)((((int)rank * (SILU ? 2 : 1) + up) * cper * kTcBM + row) * 4);
+        uint32_t remote = map_rank(base, (uint32_t)min(owner, S - 1));
 #pragma unroll
-        for (int j = 0; j < 16; ++j) part[(size_t)(c0 + j) * a.part_stride + row] = v[j];
+        for (int j = 0; j < 16; ++j) {
+          if (m0 + j < a.M) st_dsmem_f32(remote + (uint32_t)(mc * kTcBM * 4), v[j]);
+          if (++mc == cper) {
+            mc = 0;
+            ++owner;
+            remote = map_rank(base, (uint32_t)min(owner, S - 1));
+          }
+        }
       }
     }
   }
 
   tc_fence_before();
   if (S > 1) {
-    cluster_sync();  // every partial tile is written
+    __syncwarp();
+    cluster_sync();  // every partial column has arrived
     if (warp >= 2) {
-      const int et = tid - 64;  // 0 .. blockDim.x - 65
-      // this rank's rows [r0, r0 + nr).  Small splits over many columns:
-      // four consecutive rows per 16-byte load of each partial and four such
-      // items in flight per thread, the shares rounded up to four rows so
-      // that every rank starts on a 16-byte boundary (14B FP16 at 144 rows,
-      // S = 2-3: qkv 42 -> 30 us, down 65 -> 53 us; the element loop there
-      // waited one cluster-load latency per element).  Otherwise one element
-      // per thread, with all S loads of an element in flight, and shares as
-      // even as possible (7B FP16 at 48 rows, S = 7-10: the four-row form,
-      // which waits one latency per rank, measured 1123 us against 1045 us
-      // per pass; INT4 at 16 rows, S = 8).  The decision depends only on S,
-      // M and the block, so every rank takes the same.  The partials are
-      // added in rank order either way.
-      const int nthr = (int)blockDim.x - 64;
-      const int rows1 = (kTcBM + S - 1) / S;
-      const int rows4 = (rows1 + 3) & ~3;
-      const bool vec = S <= 4 && (rows4 >> 2) * a.M >= nthr;
-      const int rows = vec ? rows4 : rows1;
-      const int r0 = (int)rank * rows;
-      const int nr = max(0, min(rows, kTcBM - r0));
+      // This rank's columns, one element per thread and four such in flight;
+      // a warp takes 32 consecutive rows.  The partials are added in rank
+      // order.  Columns rather than rows per rank, and pushed rather than
+      // fetched after the barrier: fetching a few rows of every column came
+      // in 64-byte pieces with their latency exposed (1.5B FP16 qkv, S = 6,
+      // 80 / 256 rows: 9.5 -> 6.8 / 19.8 -> 12.5 us; 7B pass at 256 rows
+      // 963 -> 896; 1.5B FP8 pass at 40 rows 1320 -> 1174).
       const float* part = reinterpret_cast<const float*>(stages);
-      // output (column m, row) from the summed partials g (and u, the up row's)
-      auto emit = [&](int m, int row, float g, float u) {
-        const int64_t n = tile * kTcBM + row;
-        if (n >= a.N) return;
-        float v = g;
-        if constexpr (WK == 2) v *= reinterpret_cast<const float*>(a.scales)[n];
-        if (a.bias) v += __half2float(a.bias[n]);
-        if (SILU) {
-          if constexpr (WK == 2) u *= reinterpret_cast<const float*>(a.scales)[a.N + n];
-          if (a.bias) u += __half2float(a.bias[a.N + n]);
-          v = v / (1.0f + expf(-v)) * u;
+      const int nthr = 32 * TcConv<WK>::warps;
+      const int m_lo = min((int)rank * cper, a.M);
+      const int items = (min(m_lo + cper, a.M) - m_lo) * kTcBM;
+      const int pstep = (SILU ? 2 : 1) * cper * kTcBM;  // floats from rank to rank
+      constexpr int kIt = 4;
+      for (int i0 = tid - 64; i0 < items; i0 += kIt * nthr) {
+        float g[kIt], u[kIt], res[kIt];
+        bool live[kIt];
+#pragma unroll
+        for (int j = 0; j < kIt; ++j) {
+          const int i = i0 + j * nthr;
+          const int64_t n = tile * kTcBM + i % kTcBM;
+          live[j] = i < items && n < a.N;
+          g[j] = u[j] = res[j] = 0.0f;
+          if (live[j] && a.residual)
+            res[j] = __half2float(a.residual[(int64_t)(m_lo + i / kTcBM) * a.N + n]);
         }
-        if (a.residual) v += __half2float(a.residual[(int64_t)m * a.N + n]);
-        a.y[(int64_t)m * a.N + n] = __float2half_rn(v);
-      };
-      if (vec) {
-        constexpr int kIt = 4;
-        const int nq = nr >> 2;
-        const int items = nq * a.M;
-        for (int i0 = et; i0 < items; i0 += kIt * nthr) {
-          float4 g[kIt], u[kIt];
-#pragma unroll
-          for (int j = 0; j < kIt; ++j) g[j] = u[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          for (int qq = 0; qq < S; ++qq) {
-#pragma unroll
-            for (int j = 0; j < kIt; ++j) {
-              const int i = i0 + j * nthr;
-              if (i < items) {
-                const int m = i / nq, r = r0 + 4 * (i - m * nq);
-                const float4 v = ld_dsmem_f32x4(part + (size_t)m * a.part_stride + r, (uint32_t)qq);
-                g[j].x += v.x;
-                g[j].y += v.y;
-                g[j].z += v.z;
-                g[j].w += v.w;
-                if (SILU) {
-                  const float4 w = ld_dsmem_f32x4(part + (size_t)(a.NB + m) * a.part_stride + r, (uint32_t)qq);
-                  u[j].x += w.x;
-                  u[j].y += w.y;
-                  u[j].z += w.z;
-                  u[j].w += w.w;
-                }
-              }
-            }
-          }
+        for (int qq = 0; qq < S; ++qq) {
 #pragma unroll
           for (int j = 0; j < kIt; ++j) {
             const int i = i0 + j * nthr;
-            if (i < items) {
-              const int m = i / nq, r = r0 + 4 * (i - m * nq);
-              emit(m, r, g[j].x, u[j].x);
-              emit(m, r + 1, g[j].y, u[j].y);
-              emit(m, r + 2, g[j].z, u[j].z);
-              emit(m, r + 3, g[j].w, u[j].w);
+            if (live[j]) {
+              g[j] += part[qq * pstep + i];
+              if (SILU) u[j] += part[qq * pstep + cper * kTcBM + i];
             }
           }
         }
-      } else {
-        for (int idx = et; idx < nr * a.M; idx += nthr) {
-          const int m = idx / nr, row = r0 + (idx - m * nr);
-          float g = 0.0f, u = 0.0f;
-          for (int qq = 0; qq < S; ++qq) {
-            g += ld_dsmem_f32(part + (size_t)m * a.part_stride + row, (uint32_t)qq);
-            if (SILU) u += ld_dsmem_f32(part + (size_t)(a.NB + m) * a.part_stride + row, (uint32_t)qq);
+#pragma unroll
+        for (int j = 0; j < kIt; ++j) {
+          if (!live[j]) continue;
+          const int i = i0 + j * nthr;
+          const int64_t n = tile * kTcBM + i % kTcBM;
+          float v = g[j];
+          if constexpr (WK == 2) v *= reinterpret_cast<const float*>(a.scales)[n];
+          if (a.bias) v += __half2float(a.bias[n]);
+          if (SILU) {
+            float uu = u[j];
+            if constexpr (WK == 2) uu *= reinterpret_cast<const float*>(a.scales)[a.N + n];
+            if (a.bias) uu += __half2float(a.bias[a.N + n]);
+            v = v / (1.0f + expf(-v)) * uu;
           }
-          emit(m, row, g, u);
+          if (a.residual) v += res[j];
+          a.y[(int64_t)(m_lo + i / kTcBM) * a.N + n] = __float2half_rn(v);
         }
       }
     }
-    cluster_sync();  // no CTA leaves while another still reads its partial
   }
   __syncthreads();
   if (warp == 1) {
@@ -818,8 +796,6 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   a.stage_bytes = a.c_off + (c_bytes * S2 + 1023) / 1024 * 1024;
   // the split of K over a cluster is chosen per kernel instance (occupancy)
   const int64_t tiles = (N + kTcBM - 1) / kTcBM;
-  a.part_stride = kTcBM + 4;
-  const size_t part_bytes = (size_t)cols * a.part_stride * 4;
   // INT4: room for a CTA's group scales, sized for an unsplit K range
   // (a range of n stages touches at most (n - 1) / 2 + 2 groups)
   a.sc_ng = 0;
@@ -849,9 +825,14 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   if (ns > 8) ns = 8;
   if (ns < 2) ns = 2;
   a.nstages = ns;
-  // split-K keeps its fp32 partial tile in the (then idle) stage memory;
-  // where that does not fit (very large M), K is not split
-  a.max_split = (size_t)ns * a.stage_bytes >= part_bytes ? kTcMaxSplit : 1;
+  // split-K: a rank gathers the fp32 partials of its ceil(M / S) columns from
+  // all S ranks in the (then idle) stage memory; the split stays where they fit
+  a.max_split = 1;
+  while (a.max_split < kTcMaxSplit) {
+    const int s1 = a.max_split + 1;
+    if ((size_t)s1 * ((M + s1 - 1) / s1) * S2 * kTcBM * 4 > (size_t)ns * a.stage_bytes) break;
+    ++a.max_split;
+  }
   const size_t fixed = (size_t)ns * a.stage_bytes + (3 * (size_t)ns + 2) * 8 + 16;
   a.sc_off = (int)((fixed + 15) / 16 * 16);
   const size_t smem = 1024 + (size_t)a.sc_off + sc_bytes;
