@@ -685,8 +685,15 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
     if (two_per_sm) {
       // two CTAs per SM: the largest S (up to 16, a cluster on 8 SMs) that
       // still fits one wave (1.5B down projection, M = 5: 10.4 -> 8.7 us
-      // from S = 8 to 16)
-      while (S < max_split && tiles * (S + 1) <= 2 * sms && ksteps >= 4 * (S + 1)) ++S;
+      // from S = 8 to 16).  Clusters of more than five CTAs leave places of
+      // a GPC unused, so they may claim 5/6 of the places (FP16, 12 / 40 / 64
+      // rows: 14B down S = 7 of 280 CTAs 37.8 / 39.7 / 41.7 us, S = 6 26.9 /
+      // 27.8 / 29.2; 7B qkv S = 8 of 288 9.7 / 11.1 / 12.3, S = 7 8.9 / 9.6 /
+      // 10.8); up to five, all of them (14B qkv S = 5 of 280: 14.9 / 15.6 /
+      // 16.7, S = 4 15.4 / 17.0 / 17.6).
+      while (S < max_split && ksteps >= 4 * (S + 1) &&
+             tiles * (S + 1) * (S < 5 ? 1 : 6) <= (S < 5 ? 2 : 10) * (int64_t)sms)
+        ++S;
       return S;
     }
     // one CTA per SM: clusters of at most the portable 8 SMs
