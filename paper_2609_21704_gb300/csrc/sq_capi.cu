@@ -191,8 +191,8 @@ static sq_status run_linear(const sq_linear_op& op, cudaStream_t stream, const _
   a.pieces = (int)(op.K / weights_per_piece(op.wkind));
   a.ppad = (a.pieces + 31) / 32 * 32;
   cudaError_t e;
-  // the ring engine where the planner sends it, else the tcgen05 tile path,
-  // else the GEMV family (sq_plan.cu)
+  // the streaming engine where the planner sends it, else the ring, else the
+  // tcgen05 tile path, else the GEMV family (sq_plan.cu)
   if (use_stream(op.wkind, op.M, op.N, op.K, op.epi)) {
     e = launch_stream(op.wkind, a, stream);
     if (e != cudaSuccess) return cuda_fail(e, "sq_linear: launch");
@@ -210,7 +210,7 @@ static sq_status run_linear(const sq_linear_op& op, cudaStream_t stream, const _
     a.gamma = nullptr;
   }
   if (ring) {
-    // one to eight rows through the shared-memory ring, register-operand tensor cores
+    // shared-memory ring, register-operand tensor cores
     e = launch_ring(op.wkind, a.x, op.w, op.scales, a.bias, a.residual, a.y, op.M, op.N, op.K, op.epi,
                     stream);
     if (e != cudaSuccess) return cuda_fail(e, "sq_linear: ring launch");

@@ -1,8 +1,9 @@
 // sq_plan.cu -- how a linear call runs: device properties, the choice of
-// engine (CUDA-core GEMV or tcgen05 tensor cores) and, for the GEMV, the
-// activation-row chunking and the rows-per-group / lanes-per-row
-// configuration.  Host code only; the kernels live in sq_gemv*.cu and
-// sq_tc.cu, argument checking in sq_capi.cu.
+// engine (streaming, ring, tcgen05 tiles or CUDA-core GEMV, asked in this order)
+// and, for the GEMV, the activation-row chunking and the rows-per-group /
+// lanes-per-row configuration.  Host code only; the kernels live in
+// sq_stream.cu, sq_ring.cu, sq_tc.cu and sq_gemv*.cu, argument checking in
+// sq_capi.cu.
 #include <stdlib.h>
 
 #include "sq_internal.h"
@@ -77,9 +78,11 @@ int gemv_cap_mr(int wk, int64_t K) {
   return best;
 }
 
-// Tensor cores or CUDA cores.  From 16 rows on a CUDA-core GEMV is issue
-// bound (16 fused multiply-adds per weight); below that the choice follows
-// timings of both paths on the 1.5B/7B/14B projection shapes:
+// Tensor cores or CUDA cores, for the calls that neither the streaming engine
+// nor the ring takes (the class of the others, for sq_linear_path).  From 16 rows
+// on a CUDA-core GEMV is issue bound (16 fused multiply-adds per weight); below
+// that the choice follows timings of both paths on the 1.5B/7B/14B projection
+// shapes:
 //   * 8..15 rows: tensor cores for FP16 and FP8 weights (1.5-3x faster on
 //     every shape), and for INT4 weights from 8 Mi weights on (the INT4
 //     GEMV keeps small matrices, where its 8 x dequant reuse still pays);
@@ -169,11 +172,9 @@ cudaError_t launch_gemv(int wk, const GemvArgs& a0, cudaStream_t st) {
 // 2-3 tiles per SM the ring's whole-tile work split leaves SMs idle.
 bool use_ring(int wkind, int M, int64_t N, int64_t K, int epi) {
   if (!ring_supported(wkind, M, K)) return false;
-  // two to eight rows cost the products of one on the ring: INT4 and FP8
-  // take it there, ahead of the tcgen05 tiles too (14B 8-layer passes, us:
-  // INT4 at 4 rows 1197 -> 655, at 8 rows 1099 -> 880; FP8 at 4 rows
-  // 1067 -> 872, at 8 rows 1271 -> 946); FP16 stays on the GEMV and the
-  // tiles (ring 1228 -> 1264 at 4 rows, 1229 -> 1283 at 8)
+  // two to eight INT4 / FP8 rows cost the products of one and form one class
+  // with this engine; of these calls only the FP8 lm_head of >= 200 Mi weights
+  // reaches it, the streaming engine is asked first (use_stream)
   if (M > 1) return wkind != SQ_W_FP16;
   const bool silu = epi == SQ_EPI_SILU_GATE;
   const int64_t weights = (silu ? 2 * N : N) * K;

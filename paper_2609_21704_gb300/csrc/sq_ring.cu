@@ -1,10 +1,11 @@
-// sq_ring.cu -- linear layer for one to eight activation rows (the draft
-// pass at small batch, Sec. III-D.2; the verify pass of one sequence, Sec.
-// III-D.3) streamed through a shared-memory ring, products on the tensor
-// cores' register-operand path.
+// sq_ring.cu -- linear layer for one activation row of the large matrices
+// (direct decoding and the draft pass at batch 1, Sec. III-D.2), and for one to
+// eight rows of large FP8 lm_heads, streamed through a shared-memory ring,
+// products on the tensor cores' register-operand path.
 //
-// Used for the large single-row matrices (fused gate/up, lm_head) where it
-// measured faster than the GEMV family; the engine rule is in sq_plan.cu.
+// Used for the fused gate/up (INT4, FP16) and the lm_head (FP16, FP8) where it
+// measured faster than the GEMV family and the streaming engine; the rules
+// are in sq_plan.cu.
 //
 // Design:
 //   * one CTA per SM (12 or 16 warps for INT4, 8 for FP16 / FP8) takes a
@@ -42,11 +43,7 @@ namespace {
 
 // Warps per CTA: 8 for FP16 / FP8 (memory-bound); for INT4 (bound by the
 // nibble conversion: many warps hide its latency; 8 warps measured 1.3x
-// slower at one row) 16 at one or two activation rows and 12 from three rows
-// on, unless the staged activations leave no room for them.  Measured on the
-// 14B draft pass: 12 warps (up to 168 registers a thread instead of 128)
-// take 4 rows in 599 us against 654 us with 16 and 8 rows in 753 us against
-// 864 us, but cost 2-10 us at one and two rows; 10 or 14 warps are no better.
+// slower) 16, or the next smaller count that leaves room for long rows.
 constexpr int kWarpsHalf = 8;
 constexpr int kWarpsMid = 12;
 constexpr int kWarpsFull = 16;
@@ -159,8 +156,8 @@ __device__ __forceinline__ void cur_next(const RingArgs& a, int64_t ta, int64_t 
 // 16 rows x 256 B (lane l copies piece l & 15 of rows 2i + l / 16) or, for
 // the fused gate/up, 32 rows x 128 B (piece l & 7 of rows 4i + l / 8, gate
 // rows first); one warp instruction moves 512 contiguous bytes.  INT4: every
-// lane also copies 4 bytes of group scales (16 rows x 2 copies, or 32 rows
-// x 1) into the scale slot.  Then every lane arms the slot's mbarrier to
+// lane also copies 4 bytes of group scales (32 rows x 2 groups) into the scale
+// slot.  Then every lane arms the slot's mbarrier to
 // arrive when its copies have landed.  Rows past N are not copied.
 template <int WK, bool SILU>
 __device__ __forceinline__ void issue_stage(const RingArgs& a, const Cur& c, uint32_t slot, uint32_t sslot,
@@ -188,13 +185,12 @@ __device__ __forceinline__ void issue_stage(const RingArgs& a, const Cur& c, uin
     }
   }
   if constexpr (WK == SQ_W_INT4) {
-    const int r = SILU ? lane : lane >> 1;
-    const int cpy = SILU ? 0 : lane & 1;
-    const int64_t n = n0 + (r & 15);
-    if (2 * cpy < nu && n < a.N) {
-      const int64_t row = (SILU && r >= 16 ? a.N : 0) + n;
-      const uint8_t* src = reinterpret_cast<const uint8_t*>(a.scales) + (row * a.U + c.u + 2 * cpy) * 2;
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sslot + r * (UPS * 2) + cpy * 4), "l"(src)
+    static_assert(SILU, "INT4: the fused gate/up only");
+    const int64_t n = n0 + (lane & 15);
+    if (n < a.N) {
+      const int64_t row = (lane >= 16 ? a.N : 0) + n;
+      const uint8_t* src = reinterpret_cast<const uint8_t*>(a.scales) + (row * a.U + c.u) * 2;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sslot + lane * (UPS * 2)), "l"(src)
                    : "memory");
     }
   }
@@ -213,24 +209,20 @@ __device__ __forceinline__ uint32_t chunk_addr(uint32_t slot, int h, int u, int 
   return slot + slot_off(h * 16 + r, u * 4 + t, RB);
 }
 
-template <int WR, bool FULL>
+template <bool FULL>
 __device__ __forceinline__ void stage_int4(uint32_t slot, uint32_t sslot, int nu, int ug, uint32_t xs, int pr,
                                            int t, float (&acc)[2][2][4]) {
-  constexpr int UPS = WR == 2 ? kUps32 : kUps16;
-  // this lane's scales: rows pr and pr + 8 of each tile h, units
-  // 0 .. UPS - 1, as fp16 pairs (units 2j, 2j + 1) per 32-bit word
-  uint32_t sw[WR][2][UPS / 2];
+  constexpr int WR = 2, UPS = kUps32;
+  // this lane's scales: rows pr and pr + 8 of each tile h, both units as an
+  // fp16 pair
+  uint32_t sw[WR][2];
 #pragma unroll
   for (int h = 0; h < WR; ++h)
 #pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      const uint32_t at = sslot + (uint32_t)((h * 16 + pr + 8 * rr) * (UPS * 2));
-      if constexpr (UPS == 4) {
-        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(sw[h][rr][0]), "=r"(sw[h][rr][1]) : "r"(at));
-      } else {
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sw[h][rr][0]) : "r"(at));
-      }
-    }
+    for (int rr = 0; rr < 2; ++rr)
+      asm volatile("ld.shared.u32 %0, [%1];"
+                   : "=r"(sw[h][rr])
+                   : "r"(sslot + (uint32_t)((h * 16 + pr + 8 * rr) * (UPS * 2))));
 #pragma unroll
   for (int u = 0; u < UPS; ++u) {
     if (FULL || u < nu) {
@@ -239,7 +231,7 @@ __device__ __forceinline__ void stage_int4(uint32_t slot, uint32_t sslot, int nu
       for (int h = 0; h < WR; ++h)
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) wv[h][rr] = lds16(chunk_addr<WR>(slot, h, u, pr + 8 * rr, t));
-      constexpr int NC = WR == 2 ? 2 : 4;  // independent accumulator chains
+      constexpr int NC = 2;  // independent accumulator chains
       float d[WR][NC][4];
 #pragma unroll
       for (int h = 0; h < WR; ++h)
@@ -261,12 +253,11 @@ __device__ __forceinline__ void stage_int4(uint32_t slot, uint32_t sslot, int nu
 #pragma unroll
       for (int h = 0; h < WR; ++h) {
         // (row pr, row pr + 8) scales of unit u
-        const uint32_t spair = __byte_perm(sw[h][0][u >> 1], sw[h][1][u >> 1], (u & 1) ? 0x7632 : 0x5410);
+        const uint32_t spair = __byte_perm(sw[h][0], sw[h][1], u ? 0x7632 : 0x5410);
         const float2 s = __half22float2(*reinterpret_cast<const __half2*>(&spair));
 #pragma unroll
         for (int e = 0; e < 4; ++e) {  // (row pr | pr + 8) x (column 2t | 2t + 1)
-          float r = d[h][0][e] + d[h][1][e];
-          if constexpr (NC == 4) r += d[h][2][e] + d[h][3][e];
+          const float r = d[h][0][e] + d[h][1][e];
           acc[h][0][e] = fmaf(e < 2 ? s.x : s.y, r, acc[h][0][e]);
         }
       }
@@ -444,11 +435,11 @@ __global__ void __launch_bounds__(NW * 32, NW > 8 ? 1 : 2) ring_linear_kernel(co
         const uint32_t sa = slot_addr + k * kStageBytes, ss = sslot_addr + k * kScaleBytes;
         constexpr int WR = SILU ? 2 : 1;
         if (nu == UPS) {  // full stage: no per-unit predicate
-          if constexpr (WK == SQ_W_INT4) stage_int4<WR, true>(sa, ss, UPS, cc.u, xs_addr, pr, t, acc);
+          if constexpr (WK == SQ_W_INT4) stage_int4<true>(sa, ss, UPS, cc.u, xs_addr, pr, t, acc);
           else if constexpr (WK == SQ_W_FP8) stage_fp8<WR, true>(sa, UPS, cc.u, xs_addr, pr, t, acc);
           else stage_fp16<WR, true>(sa, UPS, cc.u, xs_addr, pr, t, acc);
         } else {
-          if constexpr (WK == SQ_W_INT4) stage_int4<WR, false>(sa, ss, nu, cc.u, xs_addr, pr, t, acc);
+          if constexpr (WK == SQ_W_INT4) stage_int4<false>(sa, ss, nu, cc.u, xs_addr, pr, t, acc);
           else if constexpr (WK == SQ_W_FP8) stage_fp8<WR, false>(sa, nu, cc.u, xs_addr, pr, t, acc);
           else stage_fp16<WR, false>(sa, nu, cc.u, xs_addr, pr, t, acc);
         }
@@ -566,19 +557,20 @@ cudaError_t launch_inst(const RingArgs& a, size_t smem, int grid, cudaStream_t s
   return launch_pdl(k, dim3(grid), dim3(NW * 32), smem, st, a);
 }
 
-template <int WK>
-cudaError_t launch_wk(const RingArgs& a, int nw, size_t smem, int grid, cudaStream_t st) {
+// The instances that the rules reach: INT4 for the fused gate/up, FP8 for plain
+// outputs, FP16 for both.
+cudaError_t launch_any(int wkind, const RingArgs& a, int nw, size_t smem, int grid, cudaStream_t st) {
   const bool silu = a.silu != 0;
-  if constexpr (WK == SQ_W_INT4) {
-    if (nw == kWarpsFull)
-      return silu ? launch_inst<WK, true, kWarpsFull>(a, smem, grid, st)
-                  : launch_inst<WK, false, kWarpsFull>(a, smem, grid, st);
-    if (nw == kWarpsMid)
-      return silu ? launch_inst<WK, true, kWarpsMid>(a, smem, grid, st)
-                  : launch_inst<WK, false, kWarpsMid>(a, smem, grid, st);
+  if (wkind == SQ_W_INT4 && silu) {
+    if (nw == kWarpsFull) return launch_inst<SQ_W_INT4, true, kWarpsFull>(a, smem, grid, st);
+    if (nw == kWarpsMid) return launch_inst<SQ_W_INT4, true, kWarpsMid>(a, smem, grid, st);
+    return launch_inst<SQ_W_INT4, true, kWarpsHalf>(a, smem, grid, st);
   }
-  return silu ? launch_inst<WK, true, kWarpsHalf>(a, smem, grid, st)
-              : launch_inst<WK, false, kWarpsHalf>(a, smem, grid, st);
+  if (wkind == SQ_W_FP8 && !silu) return launch_inst<SQ_W_FP8, false, kWarpsHalf>(a, smem, grid, st);
+  if (wkind == SQ_W_FP16)
+    return silu ? launch_inst<SQ_W_FP16, true, kWarpsHalf>(a, smem, grid, st)
+                : launch_inst<SQ_W_FP16, false, kWarpsHalf>(a, smem, grid, st);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -648,11 +640,7 @@ cudaError_t launch_ring(int wkind, const __half* x, const void* w, const void* s
   while (ns > 2 && ring_smem(nw, a.x_bytes, ns, red_floats, ncnt) > (size_t)kSmemFull) --ns;
   a.ns = ns;
   const size_t smem = ring_smem(nw, a.x_bytes, ns, red_floats, ncnt);
-  switch (wkind) {
-    case SQ_W_INT4: return launch_wk<SQ_W_INT4>(a, nw, smem, grid, st);
-    case SQ_W_FP8: return launch_wk<SQ_W_FP8>(a, nw, smem, grid, st);
-    default: return launch_wk<SQ_W_FP16>(a, nw, smem, grid, st);
-  }
+  return launch_any(wkind, a, nw, smem, grid, st);
 }
 
 // Failure-path self-test of the ring's timed wait: one thread waits on an
