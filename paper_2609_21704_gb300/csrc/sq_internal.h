@@ -109,8 +109,9 @@ bool stream_supported(int wkind, int M, int64_t N, int64_t K, int epi);
 bool use_stream(int wkind, int M, int64_t N, int64_t K, int epi);
 cudaError_t launch_stream(int wkind, const GemvArgs& a, cudaStream_t st);
 
-// sq_ring.cu: one to eight activation rows streamed through a shared-memory
-// ring, products on the register-operand tensor path (mma.sync).
+// sq_ring.cu: one activation row (one to eight of large FP8 lm_heads) streamed
+// through a shared-memory ring, products on the register-operand tensor path
+// (mma.sync).
 bool ring_supported(int wkind, int M, int64_t K);
 bool use_ring(int wkind, int M, int64_t N, int64_t K, int epi);
 cudaError_t launch_ring(int wkind, const __half* x, const void* w, const void* scales, const __half* bias,

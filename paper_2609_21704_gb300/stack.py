@@ -264,9 +264,10 @@ def decoder_pass(stack: LinearStack, variant: str, st: DecoderState, stream=None
     B, T = st.B, st.T
     pos = st.pos0 if pos0 is None else pos0
     fuse_norm = fused if fuse_norm is None else fuse_norm
-    # the fused append measured faster in passes of one new token per
-    # sequence but slower from two on (the kernels launched after it lose
-    # overlap; 10 us per layer at five tokens), so it is the default at T = 1
+    # the fused append measured faster in passes of one new token per sequence;
+    # above that it varies (us a pass, separate -> fused: 1.5B FP16 at five
+    # tokens 1446 -> 1437, 7B FP16 at 4 x 5 1335 -> 1178, but 14B INT4 at 2 x 3
+    # behind 6000 858 -> 998), so it is the default at T = 1
     fuse_append = (fused and T == 1) if fuse_append is None else fuse_append
 
     def normed(x, gamma, h, w, s, epi, y):
