@@ -813,8 +813,8 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
     a.sc_ng = (int)(need < G ? need : G);
     sc_bytes = (size_t)S2 * kTcBM * (size_t)a.sc_ng * 2;
   }
-  // Few activation rows (NB <= 64) and few row tiles: stages for two CTAs
-  // per SM (100 KB each) and a deeper split, so every SM streams and one
+  // Few activation rows (NB <= 64) and few row tiles: stages for two CTAs per
+  // SM (100 KB each) and a deeper split, so every SM streams and one
   // CTA's prologue and epilogue overlap the other's loads (measured 8-28 %
   // faster on the 1.5B/7B down, qkv and o shapes); otherwise one CTA per SM
   // with 200 KB of stages.
@@ -826,7 +826,15 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   const int sms = device_sm_count();
   const double wbytes = (double)wrows * (double)(K / 2) + (double)wrows * (double)(K / 128) * 2.0;
   a.int4_large = (wk == SQ_W_INT4 && nb <= 64 && wbytes >= 20e6) ? 1 : 0;
-  a.two_per_sm = (a.int4_large || (nb <= 64 && tiles * 2 <= sms)) ? 1 : 0;
+  // FP16 without the gate and from 24 tiles on: also up to 96 rows, and up to
+  // 128 from 40 tiles on (one CTA per SM -> two: 14B q/k/v, o, down at 80 rows
+  // 21.7, 16.8, 34.1 -> 17.2, 14.5, 29.8 us, at 112 rows 22.9, 17.6, 35.1 ->
+  // 19.1, 16.4, 32.1; four 7B layers at 80 rows 456 -> 389, but its 28 and 36
+  // tiles at 112 rows 12.9, 11.9 against 13.5, 12.2; 1.5B, 12 and 16 tiles, 28
+  // layers at 80 rows 1153 against 1184; 14B FP8 at 80 rows 518 against 535).
+  const bool more_rows =
+      wk == SQ_W_FP16 && !silu && tiles >= 24 && (nb <= 96 || (nb <= 128 && tiles >= 40));
+  a.two_per_sm = (a.int4_large || (tiles * 2 <= sms && (nb <= 64 || more_rows))) ? 1 : 0;
   const int budget = (a.two_per_sm ? 100 : 200) * 1024;
   int ns = (int)((budget - (int64_t)sc_bytes) / a.stage_bytes);
   if (ns > 8) ns = 8;

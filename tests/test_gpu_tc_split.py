@@ -46,3 +46,17 @@ def test_column_shares_match_oracle(kind, epi, M):
     full = oracle.linear(x.astype(np.float64), w64, b.astype(np.float64))
     ref = oracle.silu_gate(full[:, :N], full[:, N:]) if silu else full + r.astype(np.float64)
     assert_close(dev_to_f64(y), ref, f"{kind} M={M} epi={epi}")
+
+
+# two CTAs per SM above 64 rows: both sides of its row and tile limits
+@pytest.mark.parametrize("M,N", [(65, 3000), (96, 3072), (97, 3072), (80, 5000), (128, 5120), (129, 5120), (80, 9800)])
+def test_two_per_sm_limits_match_oracle(M, N):
+    K = 1032
+    w = synth.weights_fp16(M + N, N, K)
+    x = synth.activations_fp16(M + 2 * N, M, K)
+    b = synth.fp16_normal(M + 5, (N,), 0.5)
+    y = torch.full((M, N), 9.0, dtype=torch.float16, device=dev())
+    sq.sq_linear_ex(sq.SQ_W_FP16, f16_to_dev(x), f16_to_dev(w), None, f16_to_dev(b), None, sq.SQ_EPI_NONE, y)
+    assert sq.sq_check() == 0
+    ref = oracle.linear(x.astype(np.float64), w.astype(np.float64), b.astype(np.float64))
+    assert_close(dev_to_f64(y), ref, f"M={M} N={N}")
