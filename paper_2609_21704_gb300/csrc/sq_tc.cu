@@ -161,7 +161,8 @@ __device__ __forceinline__ void st_dsmem_f32(uint32_t remote, float v) {
 struct TcArgs {
   const void* scales;  // FP8: fp32 [rows]; INT4: fp16 [rows, K/128]; FP16: unused
   int M;            // activation rows present
-  int NB;           // MMA N: M rounded up to 16
+  int NB;           // MMA N: a CTA's activation rows rounded up to 16
+  int colblocks;    // CTAs (grid z) that share a weight tile, NB activation rows each
   int64_t N;        // output columns (weight rows, or gate rows with SILU)
   int64_t K;
   int epi;
@@ -185,7 +186,9 @@ struct TcArgs {
 };
 
 // WK: 0 fp16 weights, 1 INT4 codes, 2 FP8 codes (the GEMV family's numbering).
-template <int WK, bool SILU>
+// CB: column blocks (instances of their own: the offsets cost the others up to
+// 1.8 %).
+template <int WK, bool SILU, bool CB>
 __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     tc_linear_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tx,
                      const TcArgs a) {
@@ -209,6 +212,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
   const int S = a.splits;
   const uint32_t rank = S > 1 ? cluster_rank() : 0u;
   const int64_t tile = blockIdx.y;
+  const int m0 = CB ? (int)blockIdx.z * a.NB : 0;  // this CTA's first activation row
   const int k_begin = (int)(((int64_t)rank * a.ksteps) / S);
   const int k_end = (int)(((int64_t)(rank + 1) * a.ksteps) / S);
   const int nk = k_end - k_begin;
@@ -257,7 +261,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       }
       griddep_wait();
       for (int it = 0; it < pre; ++it)
-        tma_load_2d(stages + (size_t)it * a.stage_bytes + a.b_off, &tx, (k_begin + it) * kTcBK, 0,
+        tma_load_2d(stages + (size_t)it * a.stage_bytes + a.b_off, &tx, (k_begin + it) * kTcBK, m0,
                     &full[it]);
       int issued = pre;  // iterations whose copies were requested
       for (int it = pre; it < nk; ++it) {
@@ -274,7 +278,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
         mbar_arrive_expect_tx(&full[s], bytes);
         tma_load_2d(st + wdst, &tw, wx(k0), (int)(tile * kTcBM), &full[s]);
         if (SILU) tma_load_2d(st + wdst_up, &tw, wx(k0), (int)(a.N + tile * kTcBM), &full[s]);
-        tma_load_2d(st + a.b_off, &tx, k0, 0, &full[s]);
+        tma_load_2d(st + a.b_off, &tx, k0, m0, &full[s]);
         issued = it + 1;
       }
       if (timed_out) {
@@ -423,7 +427,10 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     __syncwarp();
     cluster_sync();
   }
-  const int cper = (a.M + S - 1) / S;  // columns of the output each rank finishes
+  const int M = CB ? min(a.NB, a.M - m0) : a.M;
+  const __half* resid = CB && a.residual ? a.residual + (int64_t)m0 * a.N : a.residual;
+  __half* out = CB ? a.y + (int64_t)m0 * a.N : a.y;
+  const int cper = (M + S - 1) / S;  // columns of the output each rank finishes
   if (warp >= 2) {
     const int q = warp & 3;  // TMEM sub-partition this warp may read
     const int row = q * 32 + lane;
@@ -442,7 +449,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int m = c0 + j;
-            if (m >= a.M) break;
+            if (m >= M) break;
             float v = g[j];
             if constexpr (WK == 2) v *= reinterpret_cast<const float*>(a.scales)[n];
             if (a.bias) v += __half2float(a.bias[n]);
@@ -452,8 +459,8 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
               if (a.bias) uu += __half2float(a.bias[a.N + n]);
               v = v / (1.0f + expf(-v)) * uu;
             }
-            if (a.residual) v += __half2float(a.residual[(int64_t)m * a.N + n]);
-            a.y[(int64_t)m * a.N + n] = __float2half_rn(v);
+            if (resid) v += __half2float(resid[(int64_t)m * a.N + n]);
+            out[(int64_t)m * a.N + n] = __float2half_rn(v);
           }
         }
       }
@@ -466,14 +473,14 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
         float v[16];
         tc_ld16(taddr + (uint32_t)c0, v);
         const int up = SILU && c0 >= a.NB ? 1 : 0;
-        const int m0 = c0 - up * a.NB;
-        int owner = m0 / cper, mc = m0 - owner * cper;
+        const int mb = c0 - up * a.NB;
+        int owner = mb / cper, mc = mb - owner * cper;
         const uint32_t base =
             smem_u32(stages) + (uint32_t)((((int)rank * (SILU ? 2 : 1) + up) * cper * kTcBM + row) * 4);
         uint32_t remote = map_rank(base, (uint32_t)min(owner, S - 1));
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          if (m0 + j < a.M) st_dsmem_f32(remote + (uint32_t)(mc * kTcBM * 4), v[j]);
+          if (mb + j < M) st_dsmem_f32(remote + (uint32_t)(mc * kTcBM * 4), v[j]);
           if (++mc == cper) {
             mc = 0;
             ++owner;
@@ -498,8 +505,8 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       // 963 -> 896; 1.5B FP8 pass at 40 rows 1320 -> 1174).
       const float* part = reinterpret_cast<const float*>(stages);
       const int nthr = 32 * TcConv<WK>::warps;
-      const int m_lo = min((int)rank * cper, a.M);
-      const int items = (min(m_lo + cper, a.M) - m_lo) * kTcBM;
+      const int m_lo = min((int)rank * cper, M);
+      const int items = (min(m_lo + cper, M) - m_lo) * kTcBM;
       const int pstep = (SILU ? 2 : 1) * cper * kTcBM;  // floats from rank to rank
       constexpr int kIt = 4;
       for (int i0 = tid - 64; i0 < items; i0 += kIt * nthr) {
@@ -511,8 +518,8 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
           const int64_t n = tile * kTcBM + i % kTcBM;
           live[j] = i < items && n < a.N;
           g[j] = u[j] = res[j] = 0.0f;
-          if (live[j] && a.residual)
-            res[j] = __half2float(a.residual[(int64_t)(m_lo + i / kTcBM) * a.N + n]);
+          if (live[j] && resid)
+            res[j] = __half2float(resid[(int64_t)(m_lo + i / kTcBM) * a.N + n]);
         }
         for (int qq = 0; qq < S; ++qq) {
 #pragma unroll
@@ -538,8 +545,8 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
             if (a.bias) uu += __half2float(a.bias[a.N + n]);
             v = v / (1.0f + expf(-v)) * uu;
           }
-          if (a.residual) v += res[j];
-          a.y[(int64_t)(m_lo + i / kTcBM) * a.N + n] = __float2half_rn(v);
+          if (resid) v += res[j];
+          out[(int64_t)(m_lo + i / kTcBM) * a.N + n] = __float2half_rn(v);
         }
       }
     }
@@ -601,9 +608,9 @@ bool tc_supported(int M, int64_t K, int epi) {
 
 // Raises the kernel's dynamic shared-memory limit to `smem` (once per size
 // and device) and allows cluster sizes above 8.
-template <int WK, bool SILU>
+template <int WK, bool SILU, bool CB>
 static cudaError_t tc_prepare(size_t smem) {
-  auto k = tc_linear_kernel<WK, SILU>;
+  auto k = tc_linear_kernel<WK, SILU, CB>;
   static int smem_set[64] = {0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -621,7 +628,7 @@ static cudaError_t tc_prepare(size_t smem) {
 
 // Clusters of S CTAs (with `smem` bytes each) that can be resident at once,
 // from the occupancy calculator; cached per device, S and size.
-template <int WK, bool SILU>
+template <int WK, bool SILU, bool CB>
 static int tc_max_clusters(int S, size_t smem) {
   struct Entry {
     size_t smem;
@@ -632,7 +639,7 @@ static int tc_max_clusters(int S, size_t smem) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || S < 1 || S > kTcMaxSplit) return 0;
   for (Entry& en : cache[dev][S])
     if (en.smem == smem + 1) return en.n;
-  if (tc_prepare<WK, SILU>(smem) != cudaSuccess) return 0;
+  if (tc_prepare<WK, SILU, CB>(smem) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)S, 1, 1);
   cfg.blockDim = dim3(TcConv<WK>::threads);
@@ -645,7 +652,7 @@ static int tc_max_clusters(int S, size_t smem) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, tc_linear_kernel<WK, SILU>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, tc_linear_kernel<WK, SILU, CB>, &cfg) != cudaSuccess) {
     (void)cudaGetLastError();
     n = 0;
   }
@@ -666,9 +673,9 @@ static int tc_max_clusters(int S, size_t smem) {
 // 1..kTcMaxSplit that minimises (waves of resident clusters) x (k-steps per
 // CTA + 2 for the split reduction), at least 2 k-steps per CTA; ties keep
 // the smaller S.
-template <int WK, bool SILU>
+template <int WK, bool SILU, bool CB>
 static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, bool two_per_sm,
-                         bool int4_large = false, bool many_rows = false) {
+                         bool int4_large, int many_rows_steps) {
   if (WK == 1 && int4_large) {
     // two CTAs per SM: the largest power-of-two split with at most 2.2 CTAs
     // per SM in all and at least 12 k-steps per CTA (odd splits of 3 and 7
@@ -697,11 +704,13 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
       return S;
     }
     // one CTA per SM: clusters of at most the portable 8 SMs
-    if (many_rows) {
+    if (many_rows_steps > 0) {
       // many activation rows (NB > 64: every k-step also streams a large
       // activation tile and runs a long MMA): the largest S that still fits
-      // one wave
-      while (S + 1 <= max_split && S + 1 <= 8 && tiles * (S + 1) <= sms && ksteps >= 4 * (S + 1)) ++S;
+      // one wave, with many_rows_steps k-steps per CTA (six with column blocks:
+      // 1.5B o at 256 rows S = 4 8.7 us, S = 5 8.9)
+      while (S + 1 <= max_split && S + 1 <= 8 && tiles * (S + 1) <= sms && ksteps >= many_rows_steps * (S + 1))
+        ++S;
       return S;
     }
     while (2 * S <= max_split && 2 * S <= 8 && tiles * S * 2 <= sms && ksteps >= 4 * S * 2) S <<= 1;
@@ -710,7 +719,7 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
   int best_s = 1;
   int64_t best = INT64_MAX;
   for (int S = 1; S <= max_split && S <= kTcMaxSplitInt4 && ksteps >= 2 * S; ++S) {
-    const int nc = tc_max_clusters<WK, SILU>(S, smem);
+    const int nc = tc_max_clusters<WK, SILU, CB>(S, smem);
     if (nc <= 0) continue;
     const int64_t waves = (tiles + nc - 1) / nc;
     const int64_t cost = waves * ((ksteps + S - 1) / S + (S > 1 ? 2 : 0));
@@ -722,17 +731,17 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
   return best_s;
 }
 
-template <int WK, bool SILU>
+template <int WK, bool SILU, bool CB>
 static cudaError_t tc_launch_inst(const CUtensorMap& tw, const CUtensorMap& tx, TcArgs a,
                                   int64_t tiles, size_t smem, cudaStream_t st) {
-  auto k = tc_linear_kernel<WK, SILU>;
-  cudaError_t e = tc_prepare<WK, SILU>(smem);
+  auto k = tc_linear_kernel<WK, SILU, CB>;
+  cudaError_t e = tc_prepare<WK, SILU, CB>(smem);
   if (e != cudaSuccess) return e;
-  const int S = tc_pick_split<WK, SILU>(tiles, a.ksteps, smem, a.max_split, a.two_per_sm != 0,
-                                       a.int4_large != 0, a.NB > 64);
+  const int S = tc_pick_split<WK, SILU, CB>(tiles * a.colblocks, a.ksteps, smem, a.max_split, a.two_per_sm != 0,
+                                       a.int4_large != 0, a.colblocks > 1 ? 6 : a.NB > 64 ? 4 : 0);
   a.splits = S;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)S, (unsigned)tiles, 1);
+  cfg.gridDim = dim3((unsigned)S, (unsigned)tiles, (unsigned)a.colblocks);
   cfg.blockDim = dim3(TcConv<WK>::threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -758,7 +767,17 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
                       const __half* residual, __half* y, int M, int64_t N, int64_t K, int epi,
                       cudaStream_t st) {
   const bool silu = epi == SQ_EPI_SILU_GATE;
-  const int nb = (M + 15) / 16 * 16;
+  const int64_t tiles = (N + kTcBM - 1) / kTcBM;
+  const int sms = device_sm_count();
+  // Short rows (K <= 2048) under many activation rows: the tail after the last
+  // MMA costs more than the products, and the few tiles leave SMs idle, so two
+  // CTAs take half of the activation rows each where they fit beside each other.
+  // FP16 (a quantised tile would be converted twice), 1.5B, one block -> two:
+  // at 144 / 256 rows gate/up 21.4 -> 19.1 / 29.5 -> 21.3 us, q/k/v 8.4 -> 7.8 /
+  // 12.2 -> 9.3, o 7.9 -> 7.1 / 12.0 -> 8.7; at 80 rows the gate/up loses (16.8
+  // against 17.5), and so do longer rows (7B q/k/v at 256 rows 17.5 against 18.8).
+  const int colblocks = wk == SQ_W_FP16 && M > 96 && K <= 2048 && 2 * tiles <= sms ? 2 : 1;
+  const int nb = ((M + colblocks - 1) / colblocks + 15) / 16 * 16;
   const int64_t wrows = silu ? 2 * N : N;
   CUtensorMap tw, tx;
   bool ok;
@@ -782,6 +801,7 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   a.scales = scales;
   a.M = M;
   a.NB = nb;
+  a.colblocks = colblocks;
   a.N = N;
   a.K = K;
   a.epi = epi;
@@ -802,7 +822,6 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   a.c_bytes = c_bytes;
   a.stage_bytes = a.c_off + (c_bytes * S2 + 1023) / 1024 * 1024;
   // the split of K over a cluster is chosen per kernel instance (occupancy)
-  const int64_t tiles = (N + kTcBM - 1) / kTcBM;
   // INT4: room for a CTA's group scales, sized for an unsplit K range
   // (a range of n stages touches at most (n - 1) / 2 + 2 groups)
   a.sc_ng = 0;
@@ -823,7 +842,6 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   // power-of-two split: measured 20-40 % faster than one CTA per SM with the
   // occupancy cost model (14B lm_head at M = 16: 332 -> 203 us; gate/up 57
   // -> 45 us; down 45 -> 36 us).
-  const int sms = device_sm_count();
   const double wbytes = (double)wrows * (double)(K / 2) + (double)wrows * (double)(K / 128) * 2.0;
   a.int4_large = (wk == SQ_W_INT4 && nb <= 64 && wbytes >= 20e6) ? 1 : 0;
   // FP16 without the gate and from 24 tiles on: also up to 96 rows, and up to
@@ -833,8 +851,8 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   // tiles at 112 rows 12.9, 11.9 against 13.5, 12.2; 1.5B, 12 and 16 tiles, 28
   // layers at 80 rows 1153 against 1184; 14B FP8 at 80 rows 518 against 535).
   const bool more_rows =
-      wk == SQ_W_FP16 && !silu && tiles >= 24 && (nb <= 96 || (nb <= 128 && tiles >= 40));
-  a.two_per_sm = (a.int4_large || (tiles * 2 <= sms && (nb <= 64 || more_rows))) ? 1 : 0;
+      wk == SQ_W_FP16 && !silu && colblocks == 1 && tiles >= 24 && (nb <= 96 || (nb <= 128 && tiles >= 40));
+  a.two_per_sm = (a.int4_large || (tiles * 2 <= sms && ((nb <= 64 && colblocks == 1) || more_rows))) ? 1 : 0;
   const int budget = (a.two_per_sm ? 100 : 200) * 1024;
   int ns = (int)((budget - (int64_t)sc_bytes) / a.stage_bytes);
   if (ns > 8) ns = 8;
@@ -845,16 +863,19 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   a.max_split = 1;
   while (a.max_split < kTcMaxSplit) {
     const int s1 = a.max_split + 1;
-    if ((size_t)s1 * ((M + s1 - 1) / s1) * S2 * kTcBM * 4 > (size_t)ns * a.stage_bytes) break;
+    if ((size_t)s1 * (((M < nb ? M : nb) + s1 - 1) / s1) * S2 * kTcBM * 4 > (size_t)ns * a.stage_bytes) break;
     ++a.max_split;
   }
   const size_t fixed = (size_t)ns * a.stage_bytes + (3 * (size_t)ns + 2) * 8 + 16;
   a.sc_off = (int)((fixed + 15) / 16 * 16);
   const size_t smem = 1024 + (size_t)a.sc_off + sc_bytes;
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
+  if (colblocks > 1)
+    return silu ? tc_launch_inst<SQ_W_FP16, true, true>(tw, tx, a, tiles, smem, st)
+                : tc_launch_inst<SQ_W_FP16, false, true>(tw, tx, a, tiles, smem, st);
 #define SQ_TC_CASE(WK_)                                                                \
-  if (wk == WK_) return silu ? tc_launch_inst<WK_, true>(tw, tx, a, tiles, smem, st)  \
-                             : tc_launch_inst<WK_, false>(tw, tx, a, tiles, smem, st);
+  if (wk == WK_) return silu ? tc_launch_inst<WK_, true, false>(tw, tx, a, tiles, smem, st)  \
+                             : tc_launch_inst<WK_, false, false>(tw, tx, a, tiles, smem, st);
   SQ_TC_CASE(SQ_W_FP16)
   SQ_TC_CASE(SQ_W_INT4)
   SQ_TC_CASE(SQ_W_FP8)
