@@ -82,6 +82,7 @@ CASES = [
     ("fp8", 11, 3584, 18944, NONE), ("fp8", 16, 3000, 2048, SILU),
     ("fp16", 2, 8960, 1536, SILU), ("fp16", 5, 5120, 5120, RES), ("fp16", 3, 5120, 13824, RES),
     ("fp16", 7, 1543, 1568, NONE), ("fp16", 6, 70001, 1536, NONE),
+    ("fp16", 8, 24321, 8224, NONE),  # thirteen parts for twelve warps were once the cheapest split: no whole round
 ]
 
 

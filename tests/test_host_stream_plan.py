@@ -1,0 +1,93 @@
+"""The streaming engine's host arithmetic (csrc/sq_stream_plan.h), compiled for
+the CPU and checked over sizes and cluster counts: a kernel never gets a split
+with which its loops stand still, and the layout stays inside the shared memory."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+CHECK = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <initializer_list>
+#include "sq_stream_plan.h"
+using namespace sq;
+
+static void die(const char* what, int wk, bool silu, const StreamPlan& a, int clusters) {
+  std::printf("%s: kind %d silu %d M %d N %lld K %d KS %d clusters %d: S %d pass_tiles %d\n", what, wk, (int)silu,
+              a.M, (long long)a.N, a.K, a.KS, clusters, a.S, a.pass_tiles);
+  std::exit(1);
+}
+
+static long plans = 0;
+static void check(int wk, bool silu, int M, int64_t N, int K, int ks, int clusters) {
+  if (!s_fits(wk, M, K, ks) || clusters > N) return;
+  const int nw = s_warps(M == 1 ? 0 : M <= 8 ? 1 : 2);
+  StreamPlan a = {};
+  a.M = M;
+  a.K = K;
+  a.N = N;
+  a.row_bytes = wk == SQ_W_INT4 ? K / 2 : wk == SQ_W_FP8 ? K : 2 * (int64_t)K;
+  a.U = s_units(wk, K);
+  a.KS = ks;
+  double ns = -1.0;
+  const int smem = s_split(wk, silu, nw, clusters, a, &ns);
+  ++plans;
+  // what fits gets a split (no call that the rule sends here is refused)
+  if (smem <= 0 || !(ns > 0.0)) die("no split", wk, silu, a, clusters);
+  // the loops over passes advance
+  if (a.pass_tiles < 1 || a.S < 1) die("a pass without tiles", wk, silu, a, clusters);
+  const int64_t tiles = ((N + clusters - 1) / clusters + 15) / 16;
+  const bool direct = a.S == 1 && a.KS == 1;
+  const int bufs = direct ? 0 : a.pass_tiles < tiles ? 2 : 1;
+  if (!direct && (int64_t)a.pass_tiles * a.S * (silu ? 2 : 1) * 16 * M > a.red_floats)
+    die("partial sums past their buffer", wk, silu, a, clusters);
+  if (a.off_red + (int64_t)bufs * a.red_floats * 4 > a.off_ring) die("overlap", wk, silu, a, clusters);
+  if (a.ns < 3 || a.off_ring + a.ns * nw * kSlotBytes > smem || smem > kSmemMax) die("shared memory", wk, silu, a, clusters);
+}
+
+int main() {
+  // clusters of 1, 2, 4, 8 CTAs that can be resident: full GPUs and fragments of one
+  const int counts[4][4] = {{152, 148, 132, 1}, {76, 72, 66, 1}, {38, 36, 30, 1}, {19, 16, 15, 1}};
+  const int kinds[3] = {SQ_W_INT4, SQ_W_FP8, SQ_W_FP16}, ku[3] = {128, 64, 32};
+  // sizes whose rounding to whole rounds of the warps once gave passes of no tile
+  for (int c = 0; c < 4; ++c)
+    for (int j = 0; j < 4; ++j) {
+      for (int64_t N : {24321, 25699, 26752}) {
+        check(SQ_W_FP16, false, 8, N, 8224, 1 << c, counts[c][j]);
+        check(SQ_W_FP8, true, 4, N, 16448, 1 << c, counts[c][j]);
+      }
+      check(SQ_W_FP8, false, 3, 12355, 49216, 1 << c, counts[c][j]);
+    }
+  for (int k = 0; k < 3; ++k)
+    for (int M = 1; M <= 16; ++M)
+      for (int U = 1; U <= 2048; U += U < 300 ? 1 : 1 + U / 37)
+        for (int c = 0; c < 4; ++c)
+          for (int n : counts[c])
+            for (int silu = 0; silu < 2; ++silu)
+              for (int t = 1; t <= 1200; t += t < 48 ? 1 : t / 4)
+                check(kinds[k], silu, M, (int64_t)n * 16 * t - (U + t) % (16 * n), U * ku[k], 1 << c, n);
+  std::printf("%ld plans\n", plans);
+  return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def checker(tmp_path_factory):
+    d = tmp_path_factory.mktemp("stream_plan")
+    (d / "check.cpp").write_text(CHECK)
+    exe = str(d / "check")
+    r = subprocess.run(["g++", "-O2", "-std=c++17", "-Wall", "-Werror", "-I", os.path.join(ROOT, "include"),
+                        "-I", os.path.join(ROOT, "paper_2609_21704_gb300", "csrc"), str(d / "check.cpp"), "-o", exe],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return exe
+
+
+def test_every_split_makes_progress_and_fits(checker):
+    r = subprocess.run([checker], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout
+    assert int(r.stdout.split()[0]) > 1_000_000
