@@ -71,9 +71,11 @@ inline int s_split(int wkind, bool silu, int nw, int clusters, StreamPlan& a, do
   if (rows > (1 << 24)) return 0;
   // parts of K: the least busy warp's units, one and a half of overhead a job.
   // At most one part a warp, so that whole rounds of the warps (below) keep at
-  // least a tile a pass: a pass of no tile would never end.
+  // least a tile a pass: a pass of no tile would never end.  At most one part a
+  // unit of the CTA with the fewest: a warp's copies would stop for good at a
+  // part without units.
   double best = -1.0;
-  for (int S = 1; S <= nu && S <= nw; ++S) {
+  for (int S = 1; S <= a.U / a.KS && S <= nw; ++S) {
     const double cost = (double)((tiles * S + nw - 1) / nw) * ((nu + S - 1) / S + 1.5);
     if (best < 0.0 || cost < best) {
       best = cost;

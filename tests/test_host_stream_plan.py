@@ -1,6 +1,7 @@
 """The streaming engine's host arithmetic (csrc/sq_stream_plan.h), compiled for
 the CPU and checked over sizes and cluster counts: a kernel never gets a split
-with which its loops stand still, and the layout stays inside the shared memory."""
+with which its loops stand still, every part of K holds a unit in every CTA of a
+cluster, and the layout stays inside the shared memory."""
 import os
 import subprocess
 
@@ -12,6 +13,7 @@ CHECK = r"""
 #include <cstdio>
 #include <cstdlib>
 #include <initializer_list>
+#include <vector>
 #include "sq_stream_plan.h"
 using namespace sq;
 
@@ -19,6 +21,34 @@ static void die(const char* what, int wk, bool silu, const StreamPlan& a, int cl
   std::printf("%s: kind %d silu %d M %d N %lld K %d KS %d clusters %d: S %d pass_tiles %d\n", what, wk, (int)silu,
               a.M, (long long)a.N, a.K, a.KS, clusters, a.S, a.pass_tiles);
   std::exit(1);
+}
+
+// Every (tile, part) of a CTA with `rows` rows and `nu` units: taken once, by one
+// warp, and copied in the order in which it is multiplied.  The copies of a warp
+// are a sequence of jobs that goes on only while the current one has units left.
+static bool walk(const StreamPlan& a, int nw, int rows, int nu) {
+  const int ntiles = (rows + 15) / 16;
+  std::vector<char> taken((size_t)ntiles * a.S, 0);
+  for (int warp = 0; warp < nw; ++warp) {
+    int it0 = 0, ijj = warp;
+    for (int t0 = 0; t0 < ntiles; t0 += a.pass_tiles) {
+      const int nt = ntiles - t0 < a.pass_tiles ? ntiles - t0 : a.pass_tiles;
+      for (int jj = warp; jj < nt * a.S; jj += nw) {
+        const int tile = t0 + jj / a.S, part = jj % a.S;
+        while (it0 < ntiles && ijj >= (ntiles - it0 < a.pass_tiles ? ntiles - it0 : a.pass_tiles) * a.S) {
+          it0 += a.pass_tiles;
+          ijj = warp;
+        }
+        if (it0 + ijj / a.S != tile || ijj % a.S != part) return false;
+        if ((part + 1) * nu / a.S - part * nu / a.S < 1) return false;
+        ijj += nw;
+        if (taken[(size_t)tile * a.S + part]++) return false;
+      }
+    }
+  }
+  for (char c : taken)
+    if (!c) return false;
+  return true;
 }
 
 static long plans = 0;
@@ -40,6 +70,12 @@ static void check(int wk, bool silu, int M, int64_t N, int K, int ks, int cluste
   // the loops over passes advance
   if (a.pass_tiles < 1 || a.S < 1) die("a pass without tiles", wk, silu, a, clusters);
   const int64_t tiles = ((N + clusters - 1) / clusters + 15) / 16;
+  // the CTAs of a cluster hold floor or ceil(U / KS) units
+  if (a.S > a.U / a.KS) die("a part without units", wk, silu, a, clusters);
+  if (plans % 61 == 0)
+    for (int up = 0; up < 2; ++up)
+      if (!walk(a, nw, (int)((N + up * (clusters - 1)) / clusters), (a.U + up * (ks - 1)) / ks))
+        die("jobs", wk, silu, a, clusters);
   const bool direct = a.S == 1 && a.KS == 1;
   const int bufs = direct ? 0 : a.pass_tiles < tiles ? 2 : 1;
   if (!direct && (int64_t)a.pass_tiles * a.S * (silu ? 2 : 1) * 16 * M > a.red_floats)
