@@ -157,7 +157,8 @@ __device__ __forceinline__ uint2 fp8_codes8(const uint4 v, float s, float rlo, f
     lo[e >> 2] |= (uint32_t)f32x2_to_e4m3x2(f[e] * rlo, f[e + 1] * rlo) << (8 * (e & 3));
     hi[e >> 2] |= (uint32_t)f32x2_to_e4m3x2(f[e] * rhi, f[e + 1] * rhi) << (8 * (e & 3));
   }
-  if (((lo[0] ^ hi[0]) | (lo[1] ^ hi[1])) != 0u) {
+  // (a row without a scale: every code is +0, also that of a NaN, whose bounds agree)
+  if (((lo[0] ^ hi[0]) | (lo[1] ^ hi[1])) != 0u || s == 0.0f) {
     lo[0] = lo[1] = 0u;
     if (s != 0.0f)
 #pragma unroll
@@ -228,8 +229,8 @@ __global__ void __launch_bounds__(kQuantThreads) quant_fp8_kernel(const __half* 
       if (rt == 0 && in) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
     }
     const float s = __fdiv_rn(amax, 448.0f);
-    // (-1: zero and infinite scales bracket to different codes, so those rows
-    // take the division's path)
+    // (-1: under a zero or infinite scale the bounds of a number differ, so those
+    // rows take the division's path)
     const float r = s > 0.0f ? __fdiv_rn(1.0f, s) : 0.0f;
     const float rlo = bad || s == 0.0f ? -1.0f : r * (1.0f - 0x1p-21f), rhi = r * (1.0f + 0x1p-21f);
     if (in) {

@@ -1,7 +1,7 @@
 """sq_quantize, bit exact against the oracle, where its kernels change path:
 partial warps of INT4 groups, FP8 rows around what a warp's and a CTA's
-registers hold, quotients on and next to a rounding tie, and scales at the
-bottom of the fp16 range (codes by division)."""
+registers hold, quotients on and next to a rounding tie, scales at the
+bottom of the fp16 range (codes by division), and rows without a finite maximum."""
 import numpy as np
 import pytest
 import torch
@@ -55,3 +55,20 @@ def test_int4_partial_warps_ties_and_small_scales(N, K):
 @pytest.mark.parametrize("N,K", [(5, 2032), (9, 2048), (5, 2064), (2, 16384), (3, 16400), (2, 40000)])
 def test_fp8_row_lengths_ties_and_small_scales(N, K):
     _check(_rows(N, K, N + K), sq.SQ_FP8_E4M3_ROW)
+
+
+@pytest.mark.parametrize("K", [16, 2048, 4112])
+def test_fp8_rows_of_nan_and_zeros_get_code_zero(K):
+    """A row whose largest number is zero has scale 0 and codes +0, also where
+    eight neighbouring weights are all NaN (both bounds of a quotient are)."""
+    w = np.zeros((4, K), dtype=np.float16)
+    w[0] = np.nan
+    w[1, 8:16] = np.nan
+    w[2, K - 8:K - 1] = np.nan
+    w[3] = -0.0
+    codes = torch.full((4, K), 7, dtype=torch.uint8, device=dev())
+    scales = torch.full((4,), 7.0, dtype=torch.float32, device=dev())
+    sq.sq_quantize(f16_to_dev(w), sq.SQ_FP8_E4M3_ROW, codes, scales)
+    assert sq.sq_check() & sq.SQ_DEV_NONFINITE_WEIGHT
+    assert not scales.any()
+    assert not codes.any()
