@@ -19,14 +19,14 @@
 //
 // Products: A = sixteen weight rows, B = the activation rows as columns (eight
 // a tile; columns past M repeat a row and are dropped).  FP16 pieces are
-// operands as they are, E4M3 codes are converted (exactly).  An INT4 nibble
-// n = c + 8 in the low bits of an fp16 register is the subnormal n 2^-24, one
-// nibble higher 16 n 2^-24: masking gives operands, five instructions for
-// eight weights where removing the offset takes nine.  Nibbles at the two
-// positions go to two accumulators (16 De + Do), and the offset is removed
-// per group of 128: 8 times the group's activations, summed while they are
-// staged.  Infinite and NaN activations would make that difference NaN: they
-// are staged as zeros and added in the epilogue.
+// operands as they are, E4M3 codes are converted (exactly), INT4 nibbles to the
+// exact integers c, nine instructions for eight weights, four of them fp16
+// arithmetic.  Masked nibbles as fp16 subnormals, their offset removed per group
+// of 128, take five, but a product with a subnormal keeps seven bits fewer beside
+// the others of its sum (gated activations: 4 % of the fp16 results wrongly
+// rounded against 0.06 %), and the offset's sums cost more than the four: 14B at
+// 16 rows, four layers and lm_head, 451 us against 426, 1.5B at 8 rows 804
+// against 732; only one row loses (14B lm_head 4 to 6 us).
 #include <mutex>
 
 #include "sq_internal.h"
@@ -91,35 +91,9 @@ __device__ __forceinline__ uint32_t s_norm2(uint32_t xw, uint32_t gw, float r) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-constexpr int kFlagInf = 1, kFlagNan = 2;
-
-// INT4: what the non-finite activations of row m add to the dot product with
-// weight row `row` (they are zero in the staged row).
-__device__ __noinline__ float s_nonfinite(const SArgs& a, int64_t row, int m, int flag, float rinv) {
-  if (flag & kFlagNan) return __int_as_float(0x7fc00000);
-  float v = 0.0f;
-  for (int k = 0; k < a.K; ++k) {
-    __half h = a.x[(int64_t)m * a.K + k];
-    if (a.gamma) h = __ushort_as_half(lo16(s_norm2(__half_as_ushort(h), __half_as_ushort(a.gamma[k]), rinv)));
-    const float xf = __half2float(h);
-    if (isfinite(xf)) continue;
-    const uint32_t b = a.w[row * a.row_bytes + (k >> 1)];
-    const int c = (int)((k & 1) ? b >> 4 : b & 15u) - 8;
-    v += (float)c * __half2float(reinterpret_cast<const __half*>(a.scales)[row * a.U + (k >> 7)]) * xf;
-  }
-  return v;
-}
-
 // y[m, n] from the fp32 dot product v (and the up row's u).
 template <int WK, bool SILU>
-__device__ __forceinline__ void s_store(const SArgs& a, int64_t n, int m, float v, float u, const int* flags,
-                                        const float* rinv) {
-  if constexpr (WK == SQ_W_INT4) {
-    if (flags[m]) {
-      v += s_nonfinite(a, n, m, flags[m], rinv[m]);
-      if constexpr (SILU) u += s_nonfinite(a, a.N + n, m, flags[m], rinv[m]);
-    }
-  }
+__device__ __forceinline__ void s_store(const SArgs& a, int64_t n, int m, float v, float u) {
   if constexpr (WK == SQ_W_FP8) v *= reinterpret_cast<const float*>(a.scales)[n];
   if (a.bias) v += __half2float(a.bias[n]);
   if constexpr (SILU) {
@@ -147,11 +121,8 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int M = NT == 0 ? 1 : a.M;
-  float* corr = reinterpret_cast<float*>(ssm + a.off_corr);
-  int* flags = reinterpret_cast<int*>(ssm + a.off_misc);     // of this CTA's share of K
-  int* allflags = flags + kMaxRows;                          // of the whole rows
-  float* rinv = reinterpret_cast<float*>(flags + 2 * kMaxRows);
-  float* nred = rinv + kMaxRows;                             // [row][8]
+  float* rinv = reinterpret_cast<float*>(ssm + a.off_misc);
+  float* nred = rinv + kMaxRows;  // [row][8]
   float* red = reinterpret_cast<float*>(ssm + a.off_red);
 
   const int ncl = (int)gridDim.x / a.KS;
@@ -238,8 +209,6 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
     const int tl = warp / a.S, part = warp - tl * a.S;
     first_scales(tl * th, min(th, rows - tl * th), part * nu / a.S, (part + 1) * nu / a.S);
   }
-  if (tid < kMaxRows) flags[tid] = 0;
-  __syncthreads();
   griddep_wait();
   griddep_launch_dependents();
 
@@ -292,41 +261,10 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
         const int u = c / (KU / 8), ci = c % (KU / 8);
         uint4* dst = reinterpret_cast<uint4*>(ssm + m * a.xstride + u * XU);
         if constexpr (I4) {
-          uint32_t h[4] = {q.x, q.y, q.z, q.w};
-          uint32_t e = 0;  // a half with all exponent bits set?
-#pragma unroll
-          for (int j = 0; j < 4; ++j) e |= ((h[j] & 0x7c007c00u) + 0x04000400u) & 0x80008000u;
-          if (e) {
-            int f = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-              for (int p = 0; p < 2; ++p) {
-                const uint32_t hv = (h[j] >> (16 * p)) & 0x7fffu;
-                if (hv >= 0x7c00u) {
-                  f |= hv > 0x7c00u ? kFlagNan : kFlagInf;
-                  h[j] &= p ? 0x0000ffffu : 0xffff0000u;
-                }
-              }
-            atomicOr(&flags[m], f);
-          }
           // lane t reads k = 32 t + 8 i + (0,4)(2,6)(1,5)(3,7) at [i][t]
           dst[(ci & 3) * 4 + (ci >> 2)] =
-              make_uint4(__byte_perm(h[0], h[2], 0x5410), __byte_perm(h[1], h[3], 0x5410),
-                         __byte_perm(h[0], h[2], 0x7632), __byte_perm(h[1], h[3], 0x7632));
-          if constexpr (NT == 0) {
-            // the offset of the unit's nibbles: -8 2^-20 times its activations
-            float sum = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[j]));
-              sum += f.x + f.y;
-            }
-            const unsigned half = 0xffffu << (lane & 16);
-#pragma unroll
-            for (int o = 1; o < 16; o <<= 1) sum += __shfl_xor_sync(half, sum, o);
-            if (ci == 0) corr[u] = sum * -0x1p-17f;
-          }
+              make_uint4(__byte_perm(q.x, q.z, 0x5410), __byte_perm(q.y, q.w, 0x5410),
+                         __byte_perm(q.x, q.z, 0x7632), __byte_perm(q.y, q.w, 0x7632));
         } else if constexpr (WK == SQ_W_FP8) {
           dst[(ci & 1) * 4 + (ci >> 1)] = q;  // lane t: k = 16 t + 8 i .. at [i][t]
         } else {
@@ -341,53 +279,25 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
 #pragma unroll
   for (int i = 0; i < NC; ++i) xa[i] = sbase + (uint32_t)(min(8 * i + g, M - 1) * a.xstride + t * 16);
 
-  if constexpr (I4 && NT > 0) {
-    // the offsets of several rows by the tensor cores: 16 De + Do with A = -8
-    // (shuffled sums, as for one row, cost 1.2 us at five)
-    for (int u = warp; u < nu; u += NW) {
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        float de[4], dd[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint4 b = s_lds16(xa[i] + u * XU + q * 64);
-          if (q == 0) {
-            s_mma0(de, 0x80088008u, 0x80088008u, 0x80088008u, 0x80088008u, b.x, b.y);
-            s_mma0(dd, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, b.z, b.w);
-          } else {
-            s_mma(de, 0x80088008u, 0x80088008u, 0x80088008u, 0x80088008u, b.x, b.y);
-            s_mma(dd, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, b.z, b.w);
-          }
-        }
-        const int m = 8 * i + 2 * t;
-        if (g == 0 && m < M) corr[u * M + m] = fmaf(de[0], 16.0f, dd[0]);
-        if (g == 0 && m + 1 < M) corr[u * M + m + 1] = fmaf(de[1], 16.0f, dd[1]);
-      }
-    }
-    __syncthreads();
-  }
-
-  // products of one 64-byte unit of a tile: d[i][0] even nibble positions (or
-  // every other product), d[i][1] odd ones; from zero when I4
+  // products of one 64-byte unit of a tile, every other one in d[i][0] and in
+  // d[i][1]; from zero when I4
   auto unit = [&](const uint4 w0, const uint4 w1, int u, float (&d)[NC][2][4]) {
     const uint32_t r0[4] = {w0.x, w0.y, w0.z, w0.w}, r1[4] = {w1.x, w1.y, w1.z, w1.w};
     if constexpr (I4) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const uint32_t s0 = r0[q] >> 8, s1 = r1[q] >> 8;
-        const uint32_t e0 = r0[q] & 0x000f000fu, e1 = r1[q] & 0x000f000fu;
-        const uint32_t e2 = s0 & 0x000f000fu, e3 = s1 & 0x000f000fu;
-        const uint32_t o0 = r0[q] & 0x00f000f0u, o1 = r1[q] & 0x00f000f0u;
-        const uint32_t o2 = s0 & 0x00f000f0u, o3 = s1 & 0x00f000f0u;
+        uint32_t p0[4], p1[4];
+        int4x8_to_f16x2(r0[q], p0);
+        int4x8_to_f16x2(r1[q], p1);
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
           const uint4 b = s_lds16(xa[i] + u * XU + q * 64);
           if (q == 0) {
-            s_mma0(d[i][0], e0, e1, e2, e3, b.x, b.y);
-            s_mma0(d[i][1], o0, o1, o2, o3, b.z, b.w);
+            s_mma0(d[i][0], p0[0], p1[0], p0[2], p1[2], b.x, b.y);
+            s_mma0(d[i][1], p0[1], p1[1], p0[3], p1[3], b.z, b.w);
           } else {
-            s_mma(d[i][0], e0, e1, e2, e3, b.x, b.y);
-            s_mma(d[i][1], o0, o1, o2, o3, b.z, b.w);
+            s_mma(d[i][0], p0[0], p1[0], p0[2], p1[2], b.x, b.y);
+            s_mma(d[i][1], p0[1], p1[1], p0[3], p1[3], b.z, b.w);
           }
         }
       }
@@ -455,21 +365,13 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
           float e[NC][2][4];
           unit(wa, wb, uu, e);
           const float s0 = __half2float(__ushort_as_half(sc[0])), s1 = __half2float(__ushort_as_half(sc[1]));
-          if constexpr (NT == 0) {
-            const float c = corr[uu];
-            acc[h][0][0] = fmaf(s0, fmaf(e[0][0][0], 16.0f, e[0][1][0]) + c, acc[h][0][0]);
-            acc[h][0][1] = fmaf(s1, fmaf(e[0][0][2], 16.0f, e[0][1][2]) + c, acc[h][0][1]);
-          } else {
 #pragma unroll
-            for (int i = 0; i < NC; ++i) {
-              const float c0 = corr[uu * M + min(8 * i + 2 * t, M - 1)];
-              const float c1 = corr[uu * M + min(8 * i + 2 * t + 1, M - 1)];
+          for (int i = 0; i < NC; ++i)
 #pragma unroll
-              for (int q = 0; q < 4; ++q)
-                acc[h][i][q] = fmaf(q < 2 ? s0 : s1, fmaf(e[i][0][q], 16.0f, e[i][1][q]) + ((q & 1) ? c1 : c0),
-                                    acc[h][i][q]);
+            for (int x = 0; x < NE; ++x) {
+              const int q = NT == 0 ? 2 * x : x;
+              acc[h][i][x] = fmaf(q < 2 ? s0 : s1, e[i][0][q] + e[i][1][q], acc[h][i][x]);
             }
-          }
         } else {
           unit(wa, wb, uu, d[h]);
         }
@@ -495,16 +397,17 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
           part_of_step(src, 0, u, s0);
         }
       }
-      // INT4 operands carry 2^-20
+      if constexpr (!I4) {
 #pragma unroll
-      for (int h = 0; h < WR; ++h)
+        for (int h = 0; h < WR; ++h)
 #pragma unroll
-        for (int i = 0; i < NC; ++i)
+          for (int i = 0; i < NC; ++i)
 #pragma unroll
-          for (int e = 0; e < NE; ++e) {
-            const int q = NT == 0 ? 2 * e : e;
-            acc[h][i][e] = I4 ? acc[h][i][e] * 0x1p20f : d[h][i][0][q] + d[h][i][1][q];
-          }
+            for (int e = 0; e < NE; ++e) {
+              const int q = NT == 0 ? 2 * e : e;
+              acc[h][i][e] = d[h][i][0][q] + d[h][i][1][q];
+            }
+      }
 #pragma unroll
       for (int i = 0; i < NC; ++i)
 #pragma unroll
@@ -512,7 +415,7 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
           const int r = g + 8 * (NT == 0 ? e : e >> 1), m = NT == 0 ? t : 8 * i + 2 * t + (e & 1);
           if (r >= nr || m >= M) continue;
           if (direct) {
-            s_store<WK, SILU>(a, n0 + row + r, m, acc[0][i][e], acc[WR - 1][i][e], flags, rinv);
+            s_store<WK, SILU>(a, n0 + row + r, m, acc[0][i][e], acc[WR - 1][i][e]);
           } else {
 #pragma unroll
             for (int h = 0; h < WR; ++h) buf[((jj * WR + h) * M + m) * 16 + r] = acc[h][i][e];
@@ -523,15 +426,6 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
     // the parts (and the cluster's CTAs) of this pass's tiles, in order
     if (a.KS > 1) {
       s_cluster_sync();
-      if (I4 && t0 == 0) {
-        if (tid < M) {
-          int f = 0;
-          for (int q = 0; q < a.KS; ++q)
-            f |= __float_as_int(s_ld_rank(reinterpret_cast<const float*>(flags + tid), (uint32_t)q));
-          allflags[tid] = f;
-        }
-        __syncthreads();
-      }
     } else {
       __syncthreads();
     }
@@ -551,7 +445,7 @@ __global__ void __launch_bounds__(32 * s_warps(NT), NT == 1 ? 2 : 1) stream_line
           if constexpr (SILU) uv += a.KS > 1 ? s_ld_rank(p + 16 * M, (uint32_t)q) : p[16 * M];
         }
       }
-      s_store<WK, SILU>(a, n0 + t0 * th + rr, m, v, uv, a.KS > 1 ? allflags : flags, rinv);
+      s_store<WK, SILU>(a, n0 + t0 * th + rr, m, v, uv);
     }
   }
   __syncthreads();

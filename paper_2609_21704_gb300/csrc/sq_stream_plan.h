@@ -28,8 +28,7 @@ struct StreamPlan {
   int S;            // parts of a CTA's units, one job each
   int pass_tiles;   // tiles whose partial sums meet at once
   int xstride;      // shared bytes between staged rows
-  int off_corr;     // INT4: [units][M] offset products
-  int off_misc;     // flags, RMSNorm scratch
+  int off_misc;     // RMSNorm scratch
   int off_red;      // one or two buffers of partial sums
   int red_floats;   // floats of one buffer
   int off_ring;
@@ -38,13 +37,12 @@ struct StreamPlan {
 
 inline int s_units(int wkind, int64_t K) { return (int)(K / (wkind == SQ_W_INT4 ? 128 : wkind == SQ_W_FP8 ? 64 : 32)); }
 
-// Shared memory up to the partial sums: staged rows, offsets, flags.
+// Shared memory up to the partial sums: staged rows, RMSNorm scratch.
 inline int s_fixed(int wkind, int M, int nu, StreamPlan& a) {
   const int ku = wkind == SQ_W_INT4 ? 128 : wkind == SQ_W_FP8 ? 64 : 32;
   a.xstride = (nu * ku * 2 + 127) / 128 * 128 + 64;
-  a.off_corr = (M * a.xstride + 127) / 128 * 128;
-  a.off_misc = a.off_corr + (wkind == SQ_W_INT4 ? (nu * M * 4 + 15) / 16 * 16 : 0);
-  a.off_red = a.off_misc + (2 * kMaxRows + kMaxRows + 8 * kMaxRows) * 4;
+  a.off_misc = (M * a.xstride + 127) / 128 * 128;
+  a.off_red = a.off_misc + (kMaxRows + 8 * kMaxRows) * 4;
   return a.off_red;
 }
 

@@ -2,7 +2,7 @@
 dequantised weights: fewer output rows than SMs, ragged tiles, one unit of K and
 odd unit counts, the row counts at which its column tiles change (2, 8, 9, 16),
 K split over a cluster with one and with several passes of partial sums, the
-epilogues, the fused RMSNorm, and non-finite activations (INT4 stages them apart).
+epilogues, the fused RMSNorm, non-finite activations, and the precision of INT4 sums.
 Bar: relative L2 <= 1e-3, max-abs <= 2e-2."""
 import numpy as np
 import pytest
@@ -115,3 +115,23 @@ def test_nonfinite_activations_stay_in_their_row(kind, M, N, K):
         assert np.array_equal(np.isnan(got[m]), np.isnan(ref[m])), m
         ok = ~np.isnan(ref[m])
         assert np.array_equal(got[m][ok], ref[m][ok]), m
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 82000, 5120), (2, 1536, 8960), (8, 4608, 3584), (16, 4000, 1536)])
+def test_int4_sums_keep_fp32_precision(M, N, K):
+    """Activations as the gate leaves them: their products with exact codes, in fp32
+    sums, seldom move an fp16 result.  A sum of about a hundred rounded group sums of
+    up to its own size is off by some 10 * 2^-24 of the row's RMS, so about 1 in 1000
+    results (an fp16 step is 2^-10 of the largest) rounds the other way; sums that
+    drop the seven lowest bits turn 2 in 100 and more."""
+    rng = np.random.default_rng(M + K)
+    g, u = rng.normal(size=(2, M, K))
+    x = (g / (1 + np.exp(-g)) * np.abs(u)).astype(np.float16)
+    w, s, rows64 = _weights("int4", N, K, 3 * N + K)
+    y = torch.empty(M, N, dtype=torch.float16, device=dev())
+    sq.sq_linear_ex(sq.SQ_W_INT4, f16_to_dev(x), w, s, None, None, NONE, y)
+    assert sq.sq_check() == 0
+    cols = np.unique(rng.integers(0, N, 4000 // M + 200))
+    ref = x.astype(np.float64) @ rows64(torch.from_numpy(cols).to(dev())).T
+    wrong = np.mean(dev_to_f64(y)[:, cols] != ref.astype(np.float16).astype(np.float64))
+    assert wrong < 0.006, wrong
