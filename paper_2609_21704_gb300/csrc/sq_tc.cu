@@ -665,6 +665,11 @@ static int tc_max_clusters(int S, size_t smem) {
   return n;
 }
 
+// Clusters of S CTAs that run at once with two CTAs per SM, 152 SMs (measured at
+// K = 8192 by the tile count at which a second wave begins; of 13, three more
+// run but twelve are faster).
+static const int kTcClusters[kTcMaxSplit + 1] = {0, 304, 152, 101, 74, 58, 46, 38, 35, 30, 28, 23, 22, 16, 14, 14, 14};
+
 // Split-K factor.  FP16 and FP8 weights (HBM-bound): double S while the
 // split tiles still fill at most half the SMs, so that the next kernel's
 // CTAs find free SMs and start their weight loads early (programmatic
@@ -690,16 +695,15 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
     const int sms = device_sm_count();
     int S = 1;
     if (two_per_sm) {
-      // two CTAs per SM: the largest S (up to 16, a cluster on 8 SMs) that
-      // still fits one wave (1.5B down projection, M = 5: 10.4 -> 8.7 us
-      // from S = 8 to 16).  Clusters of more than five CTAs leave places of
-      // a GPC unused, so they may claim 5/6 of the places (FP16, 12 / 40 / 64
-      // rows: 14B down S = 7 of 280 CTAs 37.8 / 39.7 / 41.7 us, S = 6 26.9 /
-      // 27.8 / 29.2; 7B qkv S = 8 of 288 9.7 / 11.1 / 12.3, S = 7 8.9 / 9.6 /
-      // 10.8); up to five, all of them (14B qkv S = 5 of 280: 14.9 / 15.6 /
-      // 16.7, S = 4 15.4 / 17.0 / 17.6).
+      // two CTAs per SM: the largest S (up to 16) whose clusters all run at once
+      // (1.5B down projection, M = 5: 10.4 -> 8.7 us from S = 8 to 16).  Clusters
+      // leave places of a GPC unused, so fewer run than there are places for;
+      // kTcClusters holds how many of each size did.  One cluster more costs a
+      // second wave: FP16 gate/up, K = 8192, 8 rows, 14 / 15 tiles at S = 16
+      // 13.7 / 21.4 us, 16 / 17 at S = 13 15.0 / 16.3 (no wave, but 15.8 at S =
+      // 12), 58 / 59 at S = 5 45.2 / 57.2; plain 46 / 47 at S = 6 18.9 / 27.7.
       while (S < max_split && ksteps >= 4 * (S + 1) &&
-             tiles * (S + 1) * (S < 5 ? 1 : 6) <= (S < 5 ? 2 : 10) * (int64_t)sms)
+             tiles * kNumSMs <= kTcClusters[S + 1] * (int64_t)sms)
         ++S;
       return S;
     }

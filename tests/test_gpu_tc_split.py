@@ -87,3 +87,42 @@ def test_column_blocks_match_oracle(epi, M, N, K):
     got = dev_to_f64(y)
     assert rel_l2(got, ref) <= REL_L2
     assert np.all(np.abs(got - ref) <= MAX_ABS + 2.0 ** -11 * np.abs(ref)), f"M={M} N={N} K={K} epi={epi}"
+
+
+def _us(op, copies):
+    """Time of one launch: the same call over `copies` weight copies (more than
+    the L2 holds) in a graph, best of several replays."""
+    st = torch.cuda.Stream()
+    ops = [op(i) for i in range(copies)]
+    with torch.cuda.stream(st):
+        sq.sq_linear_chain(ops, st)
+        st.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            sq.sq_linear_chain(ops, st)
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(st)
+            g.replay()
+            b.record(st)
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+    return 1e3 * best / copies
+
+
+@pytest.mark.parametrize("tiles,more", [(14, 15), (14, 16), (58, 60)])
+def test_split_clusters_run_in_one_wave(tiles, more):
+    """A few more weight tiles cost their bytes, not a second wave of the clusters
+    (which cost 1.45 to 1.6 times the time; the bytes are at most 1.15)."""
+    M, K = 16, 8192
+    x = f16_to_dev(synth.activations_fp16(3, M, K))
+
+    def us(t):
+        w = [synth.weights_fp16_device(5 + t, 2 * 128 * t, K, dev())]
+        copies = max(3, int(3e8 // (4 * 128 * t * K)))
+        w += [w[0].clone() for _ in range(copies - 1)]
+        y = torch.empty(M, 128 * t, dtype=torch.float16, device=dev())
+        return _us(lambda i: (sq.SQ_W_FP16, x, w[i], None, None, None, sq.SQ_EPI_SILU_GATE, y), copies)
+
+    assert us(more) < 1.3 * us(tiles)
