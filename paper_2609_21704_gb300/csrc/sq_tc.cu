@@ -436,12 +436,14 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     const int row = q * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
     const int64_t n = tile * kTcBM + row;
-    // this warp's columns: the first or second half, in whole 16s
-    const int cols = S == 1 ? a.NB : a.NB * (SILU ? 2 : 1);
-    const int cmid = (cols / 16 + 1) / 2 * 16;
-    const int cb = warp < 6 ? 0 : cmid, ce = warp < 6 ? cmid : cols;
+    // The two warps of a sub-partition share the columns in blocks of 16: every
+    // other one each or, pushed without the gate from 80 columns on, the halves of
+    // the row, so that they write to different ranks (FP16: unsplit 131072 x 1024
+    // at 256 rows, halves 94 us, every other one 84; gate/up, N = 2048, K = 4096,
+    // 64 rows 15.0 and 13.7; INT4 1.5B q/k/v, 33 rows, 6.0 and 5.6; but 7B q/k/v,
+    // S = 4, at 256 rows 17.4 and 18.2).
     if (S == 1) {
-      for (int c0 = cb; c0 < ce; c0 += 16) {
+      for (int c0 = warp < 6 ? 0 : 16; c0 < a.NB; c0 += 32) {
         float g[16], u[16];
         tc_ld16(taddr + (uint32_t)c0, g);
         if (SILU) tc_ld16(taddr + (uint32_t)(a.NB + c0), u);
@@ -469,7 +471,10 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       // finishes it, m / cper, at [this rank][m % cper][row]: a warp's store
       // is 32 consecutive rows, 128 bytes of one column, and nothing waits
       // for it before the barrier.  SiLU: up columns behind the gate ones.
-      for (int c0 = cb; c0 < ce; c0 += 16) {
+      const int cols = a.NB * (SILU ? 2 : 1), half = (cols / 16 + 1) / 2 * 16;
+      const bool halves = !SILU && a.NB > 64;
+      const int cend = halves && warp < 6 ? half : cols;
+      for (int c0 = warp < 6 ? 0 : halves ? half : 16; c0 < cend; c0 += halves ? 16 : 32) {
         float v[16];
         tc_ld16(taddr + (uint32_t)c0, v);
         const int up = SILU && c0 >= a.NB ? 1 : 0;
