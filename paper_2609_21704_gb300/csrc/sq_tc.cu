@@ -27,10 +27,10 @@
 // of an MMA that accumulates over several groups).
 //
 // Split-K: the S CTAs of a cluster take consecutive K ranges of the same
-// weight tile; each writes its fp32 partial tile to its own shared memory,
-// and after a cluster barrier CTA r sums its share of the 128 rows (about
-// 128/S consecutive rows) over the S partials in rank order through
-// distributed shared memory, so the result does not depend on timing.  Every mbarrier wait is bounded (a wait
+// weight tile; each pushes its fp32 partials from TMEM to the shared memory of
+// the CTA that finishes their column, and after a cluster barrier CTA r adds the
+// S partials of its columns (about M / S consecutive ones) in rank order, so the
+// result does not depend on timing.  Every mbarrier wait is bounded (a wait
 // that gives up sets SQ_DEV_TIMEOUT and is skipped from then on), so every
 // thread always reaches the cluster barriers.  After a wait gives up, the
 // TMA producer requests nothing more and waits (bounded) for the copies it
@@ -141,6 +141,12 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
@@ -178,6 +184,7 @@ struct TcArgs {
   int sc_off;       // INT4: byte offset of the CTA's group-scale block
   int sc_ng;        // INT4: groups per row held in the block (>= any CTA's need)
   int max_split;    // largest split-K factor whose partial tile fits in the stages
+  int part_off;     // partial tile of a split: beside the stages, or 0: over them
   int two_per_sm;   // stages sized so that two CTAs share an SM
   int int4_large;   // INT4 weights of 20 MB and more at few rows: power-of-two split rule
   const __half* bias;
@@ -237,6 +244,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  if (S > 1 && a.part_off) cluster_arrive();
   griddep_launch_dependents();
 
   bool timed_out = false;
@@ -423,9 +431,11 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     tc_fence_after();
   }
   if (S > 1) {
-    // every CTA's MMAs are done: the stages of all of them are free
     __syncwarp();
-    cluster_sync();
+    // every CTA of the cluster has begun, or, where partial tiles go over the
+    // stages, has its MMAs behind it
+    if (!a.part_off) cluster_arrive();
+    cluster_wait();
   }
   const int M = CB ? min(a.NB, a.M - m0) : a.M;
   const __half* resid = CB && a.residual ? a.residual + (int64_t)m0 * a.N : a.residual;
@@ -481,7 +491,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
         const int mb = c0 - up * a.NB;
         int owner = mb / cper, mc = mb - owner * cper;
         const uint32_t base =
-            smem_u32(stages) + (uint32_t)((((int)rank * (SILU ? 2 : 1) + up) * cper * kTcBM + row) * 4);
+            smem_u32(smem) + (uint32_t)a.part_off + (uint32_t)((((int)rank * (SILU ? 2 : 1) + up) * cper * kTcBM + row) * 4);
         uint32_t remote = map_rank(base, (uint32_t)min(owner, S - 1));
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
@@ -508,7 +518,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       // in 64-byte pieces with their latency exposed (1.5B FP16 qkv, S = 6,
       // 80 / 256 rows: 9.5 -> 6.8 / 19.8 -> 12.5 us; 7B pass at 256 rows
       // 963 -> 896; 1.5B FP8 pass at 40 rows 1320 -> 1174).
-      const float* part = reinterpret_cast<const float*>(stages);
+      const float* part = reinterpret_cast<const float*>(smem + a.part_off);
       const int nthr = 32 * TcConv<WK>::warps;
       const int m_lo = min((int)rank * cper, M);
       const int items = (min(m_lo + cper, M) - m_lo) * kTcBM;
@@ -749,6 +759,22 @@ static cudaError_t tc_launch_inst(const CUtensorMap& tw, const CUtensorMap& tx, 
   const int S = tc_pick_split<WK, SILU, CB>(tiles * a.colblocks, a.ksteps, smem, a.max_split, a.two_per_sm != 0,
                                        a.int4_large != 0, a.colblocks > 1 ? 6 : a.NB > 64 ? 4 : 0);
   a.splits = S;
+  // The partial tile beside the stages where that costs no residency: the ranks
+  // then push without waiting for each other's MMAs, and one of the two cluster
+  // barriers between the last MMA and the output, about half a microsecond, is
+  // long past (FP16 896 x 4864, 9 rows: 5.3 -> 4.6 us; 1.5B q/k/v, 16 rows: 5.2 ->
+  // 4.3; INT4 1.5B down, 64 rows: 16.7 -> 13.4).
+  a.part_off = 0;
+  if (S > 1) {
+    const size_t off = (smem - 1024 + 127) / 128 * 128;
+    const size_t part = (size_t)S * (((a.M < a.NB ? a.M : a.NB) + S - 1) / S) * (SILU ? 2 : 1) * kTcBM * 4;
+    if (1024 + off + part <= (size_t)(a.two_per_sm ? 113 : 227) * 1024) {
+      a.part_off = (int)off;
+      smem = 1024 + off + part;
+      e = tc_prepare<WK, SILU, CB>(smem);
+      if (e != cudaSuccess) return e;
+    }
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)S, (unsigned)tiles, (unsigned)a.colblocks);
   cfg.blockDim = dim3(TcConv<WK>::threads);
