@@ -67,35 +67,37 @@ inline int s_split(int wkind, bool silu, int nw, int clusters, StreamPlan& a, do
   const int64_t rows = (a.N + clusters - 1) / clusters;
   const int64_t tiles = (rows + 15) / 16;
   if (rows > (1 << 24)) return 0;
-  // parts of K: the least busy warp's units, one and a half of overhead a job.
-  // At most one part a warp, so that whole rounds of the warps (below) keep at
+  // Parts of K: the busiest warp's units, one and a half of overhead a job, over
+  // the passes that the partial sums need (two buffers where one does not hold
+  // them all).  At most one part a warp, so that whole rounds of the warps keep at
   // least a tile a pass: a pass of no tile would never end.  At most one part a
   // unit of the CTA with the fewest: a warp's copies would stop for good at a
-  // part without units.
+  // part without units.  (Costed as if all tiles met at once, 16 rows of an FP8
+  // gate/up, 16384 x 4096, took seven passes of five busy warps, 53 us; now four
+  // CTAs along K, one pass, 37.)
+  const int room = kSmemMax - fixed - 128 - 3 * nw * kSlotBytes;
   double best = -1.0;
+  int64_t pt = 0;
+  int nbuf = 0;
   for (int S = 1; S <= a.U / a.KS && S <= nw; ++S) {
-    const double cost = (double)((tiles * S + nw - 1) / nw) * ((nu + S - 1) / S + 1.5);
+    const bool direct = S == 1 && a.KS == 1;
+    const int per_tile = S * wr * 16 * a.M * 4;
+    int64_t p = tiles;
+    if (!direct && p * per_tile > room) {
+      p = room / 2 / per_tile;
+      if (p * S > nw) p = p * S / nw * nw / S;  // whole rounds of the warps
+      if (p < 1) break;
+    }
+    const int64_t full = tiles / p, rest = tiles - full * p;
+    const double rounds = (double)(full * ((p * S + nw - 1) / nw) + (rest * S + nw - 1) / nw);
+    const double cost = rounds * ((nu + S - 1) / S + 1.5);
     if (best < 0.0 || cost < best) {
       best = cost;
       a.S = S;
+      pt = p;
+      nbuf = direct ? 0 : p < tiles ? 2 : 1;
     }
     if (tiles >= 4 * nw) break;  // enough whole rows for every warp: no partial sums
-  }
-  const bool direct = a.S == 1 && a.KS == 1;
-  // partial sums of as many tiles as fit (two buffers when that is not all)
-  const int per_tile = a.S * wr * 16 * a.M * 4;
-  int64_t pt = tiles;
-  int nbuf = direct ? 0 : 1;
-  const int room = kSmemMax - fixed - 128 - 3 * nw * kSlotBytes;
-  if (!direct && pt * per_tile > room) {
-    pt = room / 2 / per_tile;
-    if (pt < 1) {
-      a.S = 1;  // (a deep split of wide rows: whole jobs instead)
-      pt = room / 2 / (wr * 16 * a.M * 4);
-      if (pt < 1) return 0;
-    }
-    if (pt * a.S > nw) pt = pt * a.S / nw * nw / a.S;  // whole rounds of the warps
-    nbuf = 2;
   }
   if (pt < 1) return 0;
   a.pass_tiles = (int)pt;

@@ -1,7 +1,8 @@
 """The streaming engine's host arithmetic (csrc/sq_stream_plan.h), compiled for
 the CPU and checked over sizes and cluster counts: a kernel never gets a split
 with which its loops stand still, every part of K holds a unit in every CTA of a
-cluster, and the layout stays inside the shared memory."""
+cluster, the layout stays inside the shared memory, and the estimate by which a
+split is chosen covers all of its passes."""
 import os
 import subprocess
 
@@ -76,6 +77,12 @@ static void check(int wk, bool silu, int M, int64_t N, int K, int ks, int cluste
     for (int up = 0; up < 2; ++up)
       if (!walk(a, nw, (int)((N + up * (clusters - 1)) / clusters), (a.U + up * (ks - 1)) / ks))
         die("jobs", wk, silu, a, clusters);
+  // the estimate counts every round of the warps, those of all passes
+  long rounds = 0;
+  for (int64_t t = 0; t < tiles; t += a.pass_tiles)
+    rounds += ((tiles - t < a.pass_tiles ? tiles - t : a.pass_tiles) * a.S + nw - 1) / nw;
+  const int nu = (a.U + ks - 1) / ks;
+  if (ns < 330.0 * (silu ? 2 : 1) * rounds * ((nu + a.S - 1) / a.S)) die("rounds not counted", wk, silu, a, clusters);
   const bool direct = a.S == 1 && a.KS == 1;
   const int bufs = direct ? 0 : a.pass_tiles < tiles ? 2 : 1;
   if (!direct && (int64_t)a.pass_tiles * a.S * (silu ? 2 : 1) * 16 * M > a.red_floats)
