@@ -680,10 +680,14 @@ static int tc_max_clusters(int S, size_t smem) {
   return n;
 }
 
-// Clusters of S CTAs that run at once with two CTAs per SM, 152 SMs (measured at
-// K = 8192 by the tile count at which a second wave begins; of 13, three more
-// run but twelve are faster).
-static const int kTcClusters[kTcMaxSplit + 1] = {0, 304, 152, 101, 74, 58, 46, 38, 35, 30, 28, 23, 22, 16, 14, 14, 14};
+// Clusters of S CTAs that a split may take with two CTAs per SM, 152 SMs: as many
+// as run at once, measured at K = 8192 by the tile count at which a second wave
+// begins (74, 58 of four, five CTAs; 14 of 14 to 16; of 13 three more run, but
+// twelve CTAs are faster), and above five CTAs at most 5/6 of the places.  Up to
+// 46 of six, 38 of seven, 30 of nine, 28 of ten run alone, but behind another
+// kernel, whose last CTAs still hold places, some wait: 7B FP16 at three rows, 28
+// tiles, S = 9 / 10, four layers without lm_head 332 / 367 us.
+static const int kTcClusters[kTcMaxSplit + 1] = {0, 304, 152, 101, 74, 58, 42, 36, 31, 28, 25, 22, 21, 16, 14, 14, 14};
 
 // Split-K factor.  FP16 and FP8 weights (HBM-bound): double S while the
 // split tiles still fill at most half the SMs, so that the next kernel's
@@ -712,11 +716,10 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
     if (two_per_sm) {
       // two CTAs per SM: the largest S (up to 16) whose clusters all run at once
       // (1.5B down projection, M = 5: 10.4 -> 8.7 us from S = 8 to 16).  Clusters
-      // leave places of a GPC unused, so fewer run than there are places for;
-      // kTcClusters holds how many of each size did.  One cluster more costs a
-      // second wave: FP16 gate/up, K = 8192, 8 rows, 14 / 15 tiles at S = 16
+      // leave places of a GPC unused, so fewer run than there are places for
+      // (kTcClusters).  One too many costs a second wave: FP16 gate/up, K = 8192, 8 rows, 14 / 15 tiles at S = 16
       // 13.7 / 21.4 us, 16 / 17 at S = 13 15.0 / 16.3 (no wave, but 15.8 at S =
-      // 12), 58 / 59 at S = 5 45.2 / 57.2; plain 46 / 47 at S = 6 18.9 / 27.7.
+      // 12), 58 / 59 at S = 5 45.2 / 57.2.
       while (S < max_split && ksteps >= 4 * (S + 1) &&
              tiles * kNumSMs <= kTcClusters[S + 1] * (int64_t)sms)
         ++S;
