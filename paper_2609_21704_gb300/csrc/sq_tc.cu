@@ -183,6 +183,7 @@ struct TcArgs {
   int c_bytes;      // bytes of one code tile
   int sc_off;       // INT4: byte offset of the CTA's group-scale block
   int sc_ng;        // INT4: groups per row held in the block (>= any CTA's need)
+  int sc_bytes;     // INT4: bytes of the block
   int max_split;    // largest split-K factor whose partial tile fits in the stages
   int part_off;     // partial tile of a split: beside the stages, or 0: over them
   int two_per_sm;   // stages sized so that two CTAs share an SM
@@ -753,6 +754,12 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
   return best_s;
 }
 
+// Shared memory of ns stages: the stages, the barriers, the INT4 scale block.
+static int tc_sc_off(const TcArgs& a, int ns) { return (ns * a.stage_bytes + (3 * ns + 2) * 8 + 16 + 15) / 16 * 16; }
+static size_t tc_smem(const TcArgs& a, int ns) { return 1024 + (size_t)tc_sc_off(a, ns) + (size_t)a.sc_bytes; }
+// ... and a partial tile of `part` bytes behind them.
+static size_t tc_part_end(const TcArgs& a, int ns, size_t part) { return (tc_smem(a, ns) + 127) / 128 * 128 + part; }
+
 template <int WK, bool SILU, bool CB>
 static cudaError_t tc_launch_inst(const CUtensorMap& tw, const CUtensorMap& tx, TcArgs a,
                                   int64_t tiles, size_t smem, cudaStream_t st) {
@@ -762,18 +769,27 @@ static cudaError_t tc_launch_inst(const CUtensorMap& tw, const CUtensorMap& tx, 
   const int S = tc_pick_split<WK, SILU, CB>(tiles * a.colblocks, a.ksteps, smem, a.max_split, a.two_per_sm != 0,
                                        a.int4_large != 0, a.colblocks > 1 ? 6 : a.NB > 64 ? 4 : 0);
   a.splits = S;
-  // The partial tile beside the stages where that costs no residency: the ranks
-  // then push without waiting for each other's MMAs, and one of the two cluster
-  // barriers between the last MMA and the output, about half a microsecond, is
-  // long past (FP16 896 x 4864, 9 rows: 5.3 -> 4.6 us; 1.5B q/k/v, 16 rows: 5.2 ->
-  // 4.3; INT4 1.5B down, 64 rows: 16.7 -> 13.4).
+  // The partial tile beside the stages where that costs no residency, and then no
+  // more stages than a CTA has k-steps: the ranks push without waiting for each
+  // other's MMAs, and one of the two cluster barriers between the last MMA and the
+  // output, about half a microsecond, is long past (FP16 896 x 4864, 9 rows: 5.3 ->
+  // 4.6 us; 1.5B q/k/v, 16 rows: 5.2 -> 4.3).  Up to 16 rows four stages rather than
+  // five keep two CTAs within 2 x 97 KB: above that the SM's shared-memory
+  // configuration differs from that of the kernels around, which start later (28
+  // layers of 1.5B at 9 rows 807 us without that, 774 with; a 1.5B decoder pass of
+  // five tokens 1474 and 1456; at 24 rows 97 KB as a bound for all 882, so 852).
   a.part_off = 0;
   if (S > 1) {
-    const size_t off = (smem - 1024 + 127) / 128 * 128;
+    const int nk = (a.ksteps + S - 1) / S;
+    int ns = a.nstages < nk ? a.nstages : nk < 2 ? 2 : nk;
     const size_t part = (size_t)S * (((a.M < a.NB ? a.M : a.NB) + S - 1) / S) * (SILU ? 2 : 1) * kTcBM * 4;
-    if (1024 + off + part <= (size_t)(a.two_per_sm ? 113 : 227) * 1024) {
-      a.part_off = (int)off;
-      smem = 1024 + off + part;
+    const size_t limit = (size_t)(!a.two_per_sm ? 227 : a.NB > 16 ? 113 : 97) * 1024;
+    while (a.two_per_sm && a.NB == 16 && ns > 4 && tc_part_end(a, ns, part) > limit) --ns;
+    if (tc_part_end(a, ns, part) <= limit) {
+      a.nstages = ns;
+      a.sc_off = tc_sc_off(a, ns);
+      smem = tc_part_end(a, ns, part);
+      a.part_off = (int)(smem - part - 1024);
       e = tc_prepare<WK, SILU, CB>(smem);
       if (e != cudaSuccess) return e;
     }
@@ -904,9 +920,9 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
     if ((size_t)s1 * (((M < nb ? M : nb) + s1 - 1) / s1) * S2 * kTcBM * 4 > (size_t)ns * a.stage_bytes) break;
     ++a.max_split;
   }
-  const size_t fixed = (size_t)ns * a.stage_bytes + (3 * (size_t)ns + 2) * 8 + 16;
-  a.sc_off = (int)((fixed + 15) / 16 * 16);
-  const size_t smem = 1024 + (size_t)a.sc_off + sc_bytes;
+  a.sc_bytes = (int)sc_bytes;
+  a.sc_off = tc_sc_off(a, ns);
+  const size_t smem = tc_smem(a, ns);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   if (colblocks > 1)
     return silu ? tc_launch_inst<SQ_W_FP16, true, true>(tw, tx, a, tiles, smem, st)
