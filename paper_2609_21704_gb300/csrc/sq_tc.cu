@@ -51,20 +51,17 @@ static __device__ unsigned int g_tc_status;
 
 constexpr int kTcBM = 128;      // weight rows per tile (MMA M)
 constexpr int kTcBK = 64;       // k per stage: 64 fp16 = one 128-byte swizzle row
-// Warp roles: warp 0 TMA, warp 1 MMA + TMEM, warps 2..9 the epilogue (two per
-// TMEM sub-partition, half of the columns each) and, for quantised weights,
-// the conversion of every stage before it (two per SM sub-partition, so that
-// one's dependent chain hides behind the other's).  What follows the last MMA
-// is latency bound (TMEM loads, the gate's exponential and quotient, cluster
-// loads of the partials), so warps hide it: FP16 weights, four such warps ->
-// eight, four layers (28 at 1.5B) per pass: 14B at 256 rows 817 -> 682 us, at
-// 80 rows (and lm_head) 794 -> 759; 7B at 256 1182 -> 963; 1.5B at 256
-// 3576 -> 2529; 14B at 16 rows 734 -> 730.
-template <int WK>
-struct TcConv {
-  static constexpr int warps = 8;
-  static constexpr int threads = 64 + 32 * warps;
-};
+// Warp roles: warp 0 TMA, warp 1 MMA + TMEM, the EW others the epilogue (one or
+// two per TMEM sub-partition) and, for quantised weights, the conversion of every
+// stage before it (two per SM sub-partition, so that one's dependent chain hides
+// behind the other's).  What follows the last MMA is latency bound (TMEM loads, the
+// gate's exponential and quotient, the partials), so warps hide it: FP16 weights,
+// four such warps -> eight, four layers (28 at 1.5B) per pass: 14B at 256 rows 817
+// -> 682 us, at 80 rows (and lm_head) 794 -> 759; 7B at 256 1182 -> 963; 1.5B at
+// 256 3576 -> 2529.  Up to 16 rows (FP16) a sub-partition has one block of
+// columns, and four warps leave registers to the next launch's CTA: 28 layers of
+// 1.5B at 9 rows 794 -> 784, a 1.5B decoder pass of three tokens 1342 -> 1330.
+constexpr int tc_threads(int ew) { return 64 + 32 * ew; }
 constexpr int kTcStageA = kTcBM * kTcBK * 2;  // 16 KB
 // CTAs per cluster along K: up to 16 (non-portable cluster size, allowed at
 // launch); the INT4 search keeps to the portable 8 it was measured at.
@@ -195,9 +192,9 @@ struct TcArgs {
 
 // WK: 0 fp16 weights, 1 INT4 codes, 2 FP8 codes (the GEMV family's numbering).
 // CB: column blocks (instances of their own: the offsets cost the others up to
-// 1.8 %).
-template <int WK, bool SILU, bool CB>
-__global__ void __launch_bounds__(TcConv<WK>::threads, 1)
+// 1.8 %).  EW: epilogue warps.
+template <int WK, bool SILU, bool CB, int EW>
+__global__ void __launch_bounds__(tc_threads(EW), 1)
     tc_linear_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tx,
                      const TcArgs a) {
   constexpr bool QUANT = WK != 0;
@@ -229,7 +226,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     for (int s = 0; s < a.nstages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&conv[s], TcConv<WK>::warps);
+      mbar_init(&conv[s], EW);
     }
     mbar_init(accf, 1);
     fence_mbar_init();
@@ -342,14 +339,14 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
         const int g_lo = (k_begin * kTcBK) >> 7;
         const int ng = nk > 0 ? (((k_end * kTcBK) - 1) >> 7) + 1 - g_lo : 0;
         __half* sblk = reinterpret_cast<__half*>(smem + a.sc_off);
-        for (int r = ct; r < (SILU ? 2 : 1) * kTcBM; r += 32 * TcConv<WK>::warps) {
+        for (int r = ct; r < (SILU ? 2 : 1) * kTcBM; r += 32 * EW) {
           const int h = r / kTcBM, rr = r - h * kTcBM;
           const int64_t wrow = (h ? a.N : 0) + tile * kTcBM + rr;
           const __half* src = reinterpret_cast<const __half*>(a.scales) + wrow * G + g_lo;
           __half* dst = sblk + (size_t)r * a.sc_ng;
           for (int gi = 0; gi < ng; ++gi) dst[gi] = wrow < wrows ? __ldg(src + gi) : __ushort_as_half(0);
         }
-        named_bar_sync(1, 32 * TcConv<WK>::warps);  // the converter warps
+        named_bar_sync(1, 32 * EW);  // the converter warps
       }
     }
     griddep_wait();
@@ -378,7 +375,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
           constexpr int kJobsPerRow = WK == 1 ? 2 : 4;
           constexpr int kChunksPerJob = 8 / kJobsPerRow;
 #pragma unroll
-          for (int job = ct; job < kTcBM * kJobsPerRow; job += 32 * TcConv<WK>::warps) {
+          for (int job = ct; job < kTcBM * kJobsPerRow; job += 32 * EW) {
             const int row = job / kJobsPerRow, jp = job % kJobsPerRow;
             const uint4 cw = *reinterpret_cast<const uint4*>(codes + row * (kTcBK * (WK == 1 ? 1 : 2) / 2) +
                                                              jp * 16);
@@ -454,7 +451,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
     // 64 rows 15.0 and 13.7; INT4 1.5B q/k/v, 33 rows, 6.0 and 5.6; but 7B q/k/v,
     // S = 4, at 256 rows 17.4 and 18.2).
     if (S == 1) {
-      for (int c0 = warp < 6 ? 0 : 16; c0 < a.NB; c0 += 32) {
+      for (int c0 = warp < 6 ? 0 : 16; c0 < a.NB; c0 += 4 * EW) {
         float g[16], u[16];
         tc_ld16(taddr + (uint32_t)c0, g);
         if (SILU) tc_ld16(taddr + (uint32_t)(a.NB + c0), u);
@@ -483,9 +480,9 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       // is 32 consecutive rows, 128 bytes of one column, and nothing waits
       // for it before the barrier.  SiLU: up columns behind the gate ones.
       const int cols = a.NB * (SILU ? 2 : 1), half = (cols / 16 + 1) / 2 * 16;
-      const bool halves = !SILU && a.NB > 64;
+      const bool halves = EW == 8 && !SILU && a.NB > 64;
       const int cend = halves && warp < 6 ? half : cols;
-      for (int c0 = warp < 6 ? 0 : halves ? half : 16; c0 < cend; c0 += halves ? 16 : 32) {
+      for (int c0 = warp < 6 ? 0 : halves ? half : 16; c0 < cend; c0 += halves ? 16 : 4 * EW) {
         float v[16];
         tc_ld16(taddr + (uint32_t)c0, v);
         const int up = SILU && c0 >= a.NB ? 1 : 0;
@@ -520,7 +517,7 @@ __global__ void __launch_bounds__(TcConv<WK>::threads, 1)
       // 80 / 256 rows: 9.5 -> 6.8 / 19.8 -> 12.5 us; 7B pass at 256 rows
       // 963 -> 896; 1.5B FP8 pass at 40 rows 1320 -> 1174).
       const float* part = reinterpret_cast<const float*>(smem + a.part_off);
-      const int nthr = 32 * TcConv<WK>::warps;
+      const int nthr = 32 * EW;
       const int m_lo = min((int)rank * cper, M);
       const int items = (min(m_lo + cper, M) - m_lo) * kTcBM;
       const int pstep = (SILU ? 2 : 1) * cper * kTcBM;  // floats from rank to rank
@@ -624,9 +621,9 @@ bool tc_supported(int M, int64_t K, int epi) {
 
 // Raises the kernel's dynamic shared-memory limit to `smem` (once per size
 // and device) and allows cluster sizes above 8.
-template <int WK, bool SILU, bool CB>
+template <int WK, bool SILU, bool CB, int EW>
 static cudaError_t tc_prepare(size_t smem) {
-  auto k = tc_linear_kernel<WK, SILU, CB>;
+  auto k = tc_linear_kernel<WK, SILU, CB, EW>;
   static int smem_set[64] = {0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -644,7 +641,7 @@ static cudaError_t tc_prepare(size_t smem) {
 
 // Clusters of S CTAs (with `smem` bytes each) that can be resident at once,
 // from the occupancy calculator; cached per device, S and size.
-template <int WK, bool SILU, bool CB>
+template <int WK, bool SILU, bool CB, int EW>
 static int tc_max_clusters(int S, size_t smem) {
   struct Entry {
     size_t smem;
@@ -655,10 +652,10 @@ static int tc_max_clusters(int S, size_t smem) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || S < 1 || S > kTcMaxSplit) return 0;
   for (Entry& en : cache[dev][S])
     if (en.smem == smem + 1) return en.n;
-  if (tc_prepare<WK, SILU, CB>(smem) != cudaSuccess) return 0;
+  if (tc_prepare<WK, SILU, CB, EW>(smem) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)S, 1, 1);
-  cfg.blockDim = dim3(TcConv<WK>::threads);
+  cfg.blockDim = dim3(tc_threads(EW));
   cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -668,7 +665,7 @@ static int tc_max_clusters(int S, size_t smem) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, tc_linear_kernel<WK, SILU, CB>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, tc_linear_kernel<WK, SILU, CB, EW>, &cfg) != cudaSuccess) {
     (void)cudaGetLastError();
     n = 0;
   }
@@ -698,7 +695,7 @@ static const int kTcClusters[kTcMaxSplit + 1] = {0, 304, 152, 101, 74, 58, 42, 3
 // 1..kTcMaxSplit that minimises (waves of resident clusters) x (k-steps per
 // CTA + 2 for the split reduction), at least 2 k-steps per CTA; ties keep
 // the smaller S.
-template <int WK, bool SILU, bool CB>
+template <int WK, bool SILU, bool CB, int EW>
 static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, bool two_per_sm,
                          bool int4_large, int many_rows_steps) {
   if (WK == 1 && int4_large) {
@@ -742,7 +739,7 @@ static int tc_pick_split(int64_t tiles, int ksteps, size_t smem, int max_split, 
   int best_s = 1;
   int64_t best = INT64_MAX;
   for (int S = 1; S <= max_split && S <= kTcMaxSplitInt4 && ksteps >= 2 * S; ++S) {
-    const int nc = tc_max_clusters<WK, SILU, CB>(S, smem);
+    const int nc = tc_max_clusters<WK, SILU, CB, EW>(S, smem);
     if (nc <= 0) continue;
     const int64_t waves = (tiles + nc - 1) / nc;
     const int64_t cost = waves * ((ksteps + S - 1) / S + (S > 1 ? 2 : 0));
@@ -760,13 +757,13 @@ static size_t tc_smem(const TcArgs& a, int ns) { return 1024 + (size_t)tc_sc_off
 // ... and a partial tile of `part` bytes behind them.
 static size_t tc_part_end(const TcArgs& a, int ns, size_t part) { return (tc_smem(a, ns) + 127) / 128 * 128 + part; }
 
-template <int WK, bool SILU, bool CB>
+template <int WK, bool SILU, bool CB, int EW>
 static cudaError_t tc_launch_inst(const CUtensorMap& tw, const CUtensorMap& tx, TcArgs a,
                                   int64_t tiles, size_t smem, cudaStream_t st) {
-  auto k = tc_linear_kernel<WK, SILU, CB>;
-  cudaError_t e = tc_prepare<WK, SILU, CB>(smem);
+  auto k = tc_linear_kernel<WK, SILU, CB, EW>;
+  cudaError_t e = tc_prepare<WK, SILU, CB, EW>(smem);
   if (e != cudaSuccess) return e;
-  const int S = tc_pick_split<WK, SILU, CB>(tiles * a.colblocks, a.ksteps, smem, a.max_split, a.two_per_sm != 0,
+  const int S = tc_pick_split<WK, SILU, CB, EW>(tiles * a.colblocks, a.ksteps, smem, a.max_split, a.two_per_sm != 0,
                                        a.int4_large != 0, a.colblocks > 1 ? 6 : a.NB > 64 ? 4 : 0);
   a.splits = S;
   // The partial tile beside the stages where that costs no residency, and then no
@@ -790,13 +787,13 @@ static cudaError_t tc_launch_inst(const CUtensorMap& tw, const CUtensorMap& tx, 
       a.sc_off = tc_sc_off(a, ns);
       smem = tc_part_end(a, ns, part);
       a.part_off = (int)(smem - part - 1024);
-      e = tc_prepare<WK, SILU, CB>(smem);
+      e = tc_prepare<WK, SILU, CB, EW>(smem);
       if (e != cudaSuccess) return e;
     }
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)S, (unsigned)tiles, (unsigned)a.colblocks);
-  cfg.blockDim = dim3(TcConv<WK>::threads);
+  cfg.blockDim = dim3(tc_threads(EW));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -925,11 +922,14 @@ cudaError_t launch_tc(int wk, const __half* x, const void* w, const void* scales
   const size_t smem = tc_smem(a, ns);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   if (colblocks > 1)
-    return silu ? tc_launch_inst<SQ_W_FP16, true, true>(tw, tx, a, tiles, smem, st)
-                : tc_launch_inst<SQ_W_FP16, false, true>(tw, tx, a, tiles, smem, st);
+    return silu ? tc_launch_inst<SQ_W_FP16, true, true, 8>(tw, tx, a, tiles, smem, st)
+                : tc_launch_inst<SQ_W_FP16, false, true, 8>(tw, tx, a, tiles, smem, st);
+  if (wk == SQ_W_FP16 && nb == 16)
+    return silu ? tc_launch_inst<SQ_W_FP16, true, false, 4>(tw, tx, a, tiles, smem, st)
+                : tc_launch_inst<SQ_W_FP16, false, false, 4>(tw, tx, a, tiles, smem, st);
 #define SQ_TC_CASE(WK_)                                                                \
-  if (wk == WK_) return silu ? tc_launch_inst<WK_, true, false>(tw, tx, a, tiles, smem, st)  \
-                             : tc_launch_inst<WK_, false, false>(tw, tx, a, tiles, smem, st);
+  if (wk == WK_) return silu ? tc_launch_inst<WK_, true, false, 8>(tw, tx, a, tiles, smem, st)  \
+                             : tc_launch_inst<WK_, false, false, 8>(tw, tx, a, tiles, smem, st);
   SQ_TC_CASE(SQ_W_FP16)
   SQ_TC_CASE(SQ_W_INT4)
   SQ_TC_CASE(SQ_W_FP8)
