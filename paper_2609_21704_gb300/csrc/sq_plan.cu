@@ -187,49 +187,65 @@ bool use_ring(int wkind, int M, int64_t N, int64_t K, int epi) {
   return false;
 }
 
-// The streaming engine (sq_stream.cu) where it measured faster than whatever
-// ran before (us a launch, weights cold, PDL graph of the same call; 1.5B, 7B
-// and 14B projections at 1 .. 5, 8, 9, 12 and 16 rows):
-//   INT4, one row: the lm_head of >= 400 Mi weights (14B 80.5 -> 72.0); smaller
+// The streaming engine (sq_stream.cu) where it measured faster than the engines
+// below: us a launch, weights cold, graphs of the same call with each engine forced
+// in turn (139 shapes, 512 .. 152064 outputs, K 1024 .. 18944, plain and gated), and
+// whole passes of the 1.5B, 7B and 14B stacks with one projection's engine changed,
+// which decide where the two disagree (kernels of different shared-memory needs
+// overlap less).
+//   INT4, one row: the lm_head of >= 400 Mi weights (14B 80.5 -> 74.2); smaller
 //     matrices stay on the GEMV family, whose lanes need no partial sums (1.5B
 //     q/k/v 2.4 against 3.3), and the fused gate/up on the ring (alone it gains,
-//     22.4 -> 17.6, but between launches of the GEMV family the four 14B layers
-//     take 253 us instead of 196);
+//     but between launches of the GEMV family the four 14B layers take 253 us
+//     instead of 196).
 //   INT4 and FP8, 2 .. 8 rows: everything (14B q/k/v INT4 at 2 rows 10.6 -> 8.5,
 //     down FP8 at 8 rows 36.8 -> 17.2) but the FP8 lm_head of >= 200 Mi, which
-//     the ring streams as fast as memory gives (14B 131 against 137, 1.5B 49
-//     against 51);
-//   INT4 and FP8, 9 .. 16 rows: everything (14B lm_head INT4 at 16 rows 192 ->
-//     138, down FP8 at 16 38.4 -> 21.1) but long rows of small matrices (0.5B
-//     down FP8 5.7 against 7.2) and, from 13 rows on, long rows of FP8 (7B down
-//     21.6 against 25.0), narrow mid-sized FP8 (7B q/k/v 9.1 against 10.0) and
-//     the smallest INT4 matrices (1.5B o 4.6 against 6.1);
-//   FP16, 2 .. 8 rows: at two rows the fused gate/up and the lm_head (14B lm_head
-//     384 -> 253); from three rows on matrices of 8 Mi weights and more with K <
-//     8192 (14B o at five rows 16.3 -> 12.0; from 32 Mi up to five rows: 14B
-//     q/k/v at eight 15.2 against 16.2), the 14B down shape (36.9 -> 27.4),
-//     and, where the tile path's 128-row tiles are few, fused gate/up below 64 Mi
-//     (1.5B at five 12.5 -> 11.2) and lm_heads below 400 Mi (1.5B 96.6 -> 80.4);
-//     small matrices from six rows on (1.5B q/k/v at eight 5.5 -> 3.8).
+//     the ring streams as fast as memory gives (14B at 2 rows 127 against 133).
+//   INT4, 9 .. 16 rows: everything, as the other engines spend their time on the
+//     conversion (14B lm_head at 16 rows 196 -> 137, 512 x 8192 at 12 rows 22.8 ->
+//     7.0); at 16 rows, where the tile path takes small matrices too, from 3 Mi
+//     weights on (1536 x 1536 4.4 against 5.2).
+//   FP8, 9 .. 16 rows: everything (14B lm_head at 16 rows 272 -> 167) but plain
+//     outputs of K >= 2048 in up to 8 weight tiles, whose K the tile path splits over
+//     many CTAs (512 x 8192 at 16 rows 6.7 against 9.0), and, from 14 rows on, where
+//     the staged rows take most of the shared memory, of 25 to 39 tiles (4096 x 8192
+//     13.4 against 15.4; 7B passes at 16 rows with the down projection here 711 us
+//     against 686, with q/k/v 699, but 14B's down, 40 tiles, 464 against 476).
+//   FP16, plain.  The tile path runs two CTAs an SM up to 76 weight tiles: there
+//     it is the faster one for long rows (K >= 8192: 14B down at 5 rows 25.9
+//     against 27.6) and at eight rows from K = 2048 on (7B q/k/v 8.4 against 8.9);
+//     else the streaming engine is (14B q/k/v at 5 rows 18.9 -> 15.4, 24576 x 1536 at
+//     8 rows 21.8 -> 14.7): from 8 Mi weights on, or, at six and seven rows, where the
+//     alternative is the GEMV, any (896 x 4864 10.3 -> 6.4).  Its lm_head of >= 400
+//     Mi takes two rows only (14B 383 -> 254; at five 251 against 257).
+//   FP16, gated: from 64 Mi weights on at two rows (7B pass 1031 -> 917; 1.5B, 26 Mi,
+//     832 against 881); small ones at six and seven rows (GEMV: 1024 x 4096 15.0 ->
+//     7.5); short rows below 32 Mi at three to six (1.5B pass at five rows 864 -> 828,
+//     but at eight 851 against 882) and few long rows (512 x 16384 at three 14.1 ->
+//     10.7); the tile path has the rest (16384 x 1024 at three 13.0 against 14.7).
 bool use_stream(int wkind, int M, int64_t N, int64_t K, int epi) {
   if (!stream_supported(wkind, M, N, K, epi)) return false;
   const bool silu = epi == SQ_EPI_SILU_GATE;
   const int64_t Mi = (int64_t)1 << 20;
   const int64_t weights = (silu ? 2 * N : N) * K;
   const bool head = !silu && N >= 65536;
+  const int64_t tiles = (N + 127) / 128;  // of the tile path
   if (M == 1) return wkind == SQ_W_INT4 && head && weights >= 400 * Mi;
   if (wkind == SQ_W_FP16) {
     if (M > 8) return false;
-    if (silu) return weights < 64 * Mi ? weights >= 16 * Mi || M >= 6 : M == 2;
     if (head) return weights < 400 * Mi ? M >= 3 : M == 2;
-    if (K >= 8192) return M >= 3 && N >= 4096 && K < 16384;
-    if (K >= 4096 && weights < 8 * Mi) return false;
-    return M >= (weights >= 8 * Mi ? 3 : 6) && !(M >= 6 && weights >= 32 * Mi);
+    if (silu) {
+      if (M == 2) return weights >= 64 * Mi;
+      if (weights < 16 * Mi) return M == 6 || M == 7 || (M == 8 && K <= 2048);
+      return (M <= 6 && K <= 2048 && weights < 32 * Mi) || tiles <= 8;
+    }
+    if (M == 2) return false;
+    if (M == 8) return K < 2048 || tiles > 76;
+    return K >= 8192 ? tiles > 76 : M >= 6 || weights >= 8 * Mi;
   }
   if (M <= 8) return !(wkind == SQ_W_FP8 && head && weights >= 200 * Mi);
-  if (K >= 4096 && weights < 8 * Mi) return false;
-  if (M >= 13) return wkind == SQ_W_FP8 ? K < 16384 && (K < 3072 || N > 6144 || weights < 14 * Mi) : weights >= 3 * Mi;
-  return true;
+  if (wkind == SQ_W_INT4) return M < 16 || weights >= 3 * Mi;
+  return silu || K < 2048 || (tiles > 8 && (M < 14 || tiles <= 24 || tiles >= 40));
 }
 
 }  // namespace sq
