@@ -213,7 +213,8 @@ def kernel_digest(kernel_tag: str) -> str:
     files = {"gemv": ("sq_gemv.cuh", f"sq_gemv_{fmt}.cu"),
              "mma": ("sq_gemv.cuh", "sq_gemv_mma.cuh", f"sq_gemv_{fmt}.cu"),
              "tc": ("sq_tc.cu",),
-             "ring": ("sq_ring.cu",)}[engine] + _COMMON
+             "ring": ("sq_ring.cu",),
+             "stream": ("sq_stream.cu", "sq_stream_plan.h")}[engine] + _COMMON
     return source_digest([os.path.join(_CSRC, f) for f in files])
 
 
@@ -910,7 +911,7 @@ def main():
 
     # ---- dominant kernel: the fused gate/up + SiLU linear (largest per-launch
     # weight matrix in the layers); all layers' launches of it in one graph
-    engine = {1: "tc", 2: "mma", 3: "ring"}.get(sq.sq_linear_path(stk.WKIND[args.draft], B, shape.intermediate,
+    engine = {1: "tc", 2: "mma", 3: "ring", 4: "stream"}.get(sq.sq_linear_path(stk.WKIND[args.draft], B, shape.intermediate,
                                                       shape.hidden, sq.SQ_EPI_SILU_GATE), "gemv")
     kernel_tag = f"{engine}_{args.draft}_gateup_silu_m{B}"
     gu_projs = [layer[2] for layer in stack.layers]

@@ -125,7 +125,7 @@ SQ_API sq_status sq_quantize(const void* w16, int64_t N, int64_t K, sq_qkind kin
  * nearest fp16 once.  1 <= M <= 256; N >= 1; K as for sq_quantize (INT4:
  * K % 128 == 0, FP8: K % 16 == 0, FP16: K % 8 == 0).  x, codes, w16 and y
  * must be 16-byte aligned.  Each call runs on one of these engines, chosen
- * from (format, M, N, K, epilogue) alone (sq_linear_path reports the class):
+ * from (format, M, N, K, epilogue) alone (sq_linear_path reports which):
  * the CUDA-core GEMV family for few rows (for one INT4 row over many output
  * rows, with its products on the tensor cores' register-operand path), the
  * shared-memory ring engine for one row of large weights, the streaming
@@ -176,16 +176,16 @@ SQ_API sq_status sq_linear_norm(sq_wkind wkind, const void* x, const void* gamma
                                 const void* w, const void* scales, const void* bias, const void* residual,
                                 sq_epilogue epi, void* y, int M, int64_t N, int64_t K, sq_stream_t stream);
 
-/* Class of engine for these sizes: 1 = tensor-core tiles (tcgen05), 0 = few
- * rows of a small matrix (CUDA-core GEMV), 2 = one INT4 activation row over at
- * least 192 16-row output tiles with the products on the tensor cores'
- * register-operand path (mma.sync), 3 = one to eight activation rows streamed
- * through a shared-memory ring of asynchronous copies, products on the same
- * register-operand path.  Inside a class a call may run on the streaming
- * engine instead (a ring of asynchronous copies and the register-operand path
- * too): most calls of two to sixteen rows, and the largest INT4 lm_heads at
- * one row.  -1 = sizes or kinds sq_linear_ex rejects (pointers are not examined;
- * nothing runs on the device).  The paper has no counterpart: this is
+/* Engine sq_linear_ex uses for these sizes: 1 = tensor-core tiles (tcgen05),
+ * 0 = few rows of a small matrix (CUDA-core GEMV), 2 = one INT4 activation row
+ * over at least 192 16-row output tiles with the products on the tensor cores'
+ * register-operand path (mma.sync), 3 = the shared-memory ring of asynchronous
+ * copies, products on the same register-operand path (one row of large
+ * matrices, two to eight of the largest FP8 lm_heads), 4 = the streaming engine
+ * (equal row shares through per-lane rings, the same products: most calls of two
+ * to sixteen rows, and the largest INT4 lm_heads at one row).  -1 = sizes or
+ * kinds sq_linear_ex rejects (pointers are not examined; nothing runs on the
+ * device).  The paper has no counterpart: this is
  * introspection for tests and tuning. */
 SQ_API int sq_linear_path(sq_wkind wkind, int M, int64_t N, int64_t K, sq_epilogue epi);
 

@@ -147,9 +147,10 @@ def sq_version() -> int:
 
 
 def sq_linear_path(wkind: int, M: int, N: int, K: int, epi: int = SQ_EPI_NONE) -> int:
-    """1: tcgen05 tensor-core tiles, 0: CUDA-core GEMV, 2: one INT4 row with
-    its products on the tensor cores' register-operand path, 3: one row
-    through the shared-memory ring engine, -1: sizes sq_linear_ex rejects."""
+    """Engine of a call: 1: tcgen05 tensor-core tiles, 0: CUDA-core GEMV, 2: one
+    INT4 row with its products on the tensor cores' register-operand path, 3: the
+    shared-memory ring (one row; two to eight of large FP8 lm_heads), 4: the
+    streaming engine, -1: sizes sq_linear_ex rejects."""
     return load().sq_linear_path(wkind, M, N, K, epi)
 
 

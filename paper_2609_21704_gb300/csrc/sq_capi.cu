@@ -308,6 +308,7 @@ sq_status sq_selftest_wait(int which, uint64_t limit, sq_stream_t stream) {
 
 int sq_linear_path(sq_wkind wkind, int M, int64_t N, int64_t K, sq_epilogue epi) {
   if (check_linear_sizes(wkind, M, N, K, epi) != SQ_OK) return -1;
+  if (use_stream(wkind, M, N, K, epi)) return 4;
   if (use_ring(wkind, M, N, K, epi)) return 3;
   if (use_tensor_cores(wkind, M, N, K, epi) && tc_supported(M, K, epi)) return 1;
   return gemv_uses_mma(wkind, M, N) ? 2 : 0;

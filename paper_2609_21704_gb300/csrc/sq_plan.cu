@@ -79,8 +79,7 @@ int gemv_cap_mr(int wk, int64_t K) {
 }
 
 // Tensor cores or CUDA cores, for the calls that neither the streaming engine
-// nor the ring takes (the class of the others, for sq_linear_path).  From 16 rows
-// on a CUDA-core GEMV is issue bound (16 fused multiply-adds per weight); below
+// nor the ring takes.  From 16 rows on a CUDA-core GEMV is issue bound (16 fused multiply-adds per weight); below
 // that the choice follows timings of both paths on the 1.5B/7B/14B projection
 // shapes:
 //   * 8..15 rows: tensor cores for FP16 and FP8 weights (1.5-3x faster on
@@ -160,25 +159,23 @@ cudaError_t launch_gemv(int wk, const GemvArgs& a0, cudaStream_t st) {
   return cudaSuccess;
 }
 
-// The shared-memory ring engine (sq_ring.cu), one activation row, where it
+// The shared-memory ring engine (sq_ring.cu), mostly one activation row, where it
 // measured faster than the GEMV family (GB300, graphs of whole-stack launch
 // sequences; us per launch, ring vs previous engine):
 //   INT4 fused gate/up of >= 64 Mi weights (7B, 14B): 14B 19.5 vs 25.8;
 //     the 1.5B one (27.5 Mi) stays on the register-operand path (6.9 vs 5.0);
 //   FP16 fused gate/up of >= 16 Mi weights: 14B 49.5 vs 54.0, 1.5B 10.0 vs
 //     11.3; FP16 lm_head (N >= 65536): 14B 228 vs 375, 1.5B 74.6 vs 79.5;
-//   FP8 lm_head of >= 400 Mi weights: 14B 124 vs 164 (1.5B: 46.0 vs 41.1).
+//   FP8 lm_head of >= 400 Mi weights: 14B 124 vs 164 (1.5B: 46.0 vs 41.1), and at
+//     two to eight rows, against the streaming engine, of >= 200 Mi (use_stream).
 // q/k/v, o and down (96..448 tiles of 16 rows) stay on the GEMV family: at
 // 2-3 tiles per SM the ring's whole-tile work split leaves SMs idle.
 bool use_ring(int wkind, int M, int64_t N, int64_t K, int epi) {
   if (!ring_supported(wkind, M, K)) return false;
-  // two to eight INT4 / FP8 rows cost the products of one and form one class
-  // with this engine; of these calls only the FP8 lm_head of >= 200 Mi weights
-  // reaches it, the streaming engine is asked first (use_stream)
-  if (M > 1) return wkind != SQ_W_FP16;
   const bool silu = epi == SQ_EPI_SILU_GATE;
   const int64_t weights = (silu ? 2 * N : N) * K;
   const int64_t Mi = (int64_t)1 << 20;
+  if (M > 1) return wkind == SQ_W_FP8 && !silu && N >= 65536 && weights >= 200 * Mi;
   switch (wkind) {
     case SQ_W_INT4: return silu && weights >= 64 * Mi;
     case SQ_W_FP16: return (silu && weights >= 16 * Mi) || (!silu && N >= 65536);

@@ -127,10 +127,12 @@ def test_single_row_engine_choice(lib):
     """sq_linear_path is host logic: one activation row takes the shared-
     memory ring (3) for the large matrices where it measured faster (INT4
     fused gate/up of >= 64 Mi weights, FP16 fused gate/up of >= 16 Mi and
-    lm_head rows, FP8 lm_head of >= 400 Mi weights), two to eight INT4 or
-    FP8 rows take it whenever their activations fit; otherwise one INT4 row
-    over at least 192 16-row output tiles takes the register-operand tensor
-    path (2) and other few-row calls the streaming CUDA-core GEMV (0).  (The
+    lm_head rows, FP8 lm_head of >= 400 Mi weights, and of >= 200 Mi at two to
+    eight rows); two to sixteen INT4 or FP8 rows, the FP16 shapes where it
+    measured faster and the largest INT4 lm_heads take the streaming engine (4);
+    otherwise one INT4 row over at least 192 16-row output tiles takes the
+    register-operand tensor path (2) and other few-row calls the streaming
+    CUDA-core GEMV (0).  (The
     tcgen05 path (1) needs a device to encode its tensor maps: checked in
     tests/test_gpu_tc.py.)"""
     W4, W8, W16 = sq.SQ_W_INT4, sq.SQ_W_FP8, sq.SQ_W_FP16
@@ -139,7 +141,7 @@ def test_single_row_engine_choice(lib):
     assert sq.sq_linear_path(W4, 1, 151936, 1536, NONE) == 2    # 1.5B lm_head
     assert sq.sq_linear_path(W4, 1, 18944, 3584, SILU) == 3     # 7B fused gate/up (136 Mi)
     assert sq.sq_linear_path(W4, 1, 13824, 5120, SILU) == 3     # 14B fused gate/up
-    assert sq.sq_linear_path(W4, 1, 152064, 5120, NONE) == 2    # 14B lm_head
+    assert sq.sq_linear_path(W4, 1, 152064, 5120, NONE) == 4    # 14B lm_head (742 Mi)
     assert sq.sq_linear_path(W4, 1, 2048, 1536, NONE) == 0      # 1.5B q/k/v
     assert sq.sq_linear_path(W4, 1, 1536, 1536, RES) == 0       # 1.5B o
     assert sq.sq_linear_path(W4, 1, 1536, 8960, RES) == 0       # 1.5B down
@@ -149,10 +151,16 @@ def test_single_row_engine_choice(lib):
     assert sq.sq_linear_path(W4, 1, 4608, 3584, NONE) == 2      # 7B q/k/v (288 tiles)
     assert sq.sq_linear_path(W4, 1, 3584, 18944, RES) == 2      # 7B down (224 tiles)
     assert sq.sq_linear_path(W4, 1, 32768, 2176, SILU) == 2     # 17 groups: odd, not the ring
-    assert sq.sq_linear_path(W4, 2, 151936, 1536, NONE) == 3    # two rows: the ring too
-    assert sq.sq_linear_path(W8, 8, 7168, 5120, NONE) == 3      # FP8 draft at batch 8
+    assert sq.sq_linear_path(W4, 2, 151936, 1536, NONE) == 4    # two rows: streamed
+    assert sq.sq_linear_path(W8, 8, 7168, 5120, NONE) == 4      # FP8 draft at batch 8
+    assert sq.sq_linear_path(W8, 8, 152064, 5120, NONE) == 3    # its lm_head: the ring
+    assert sq.sq_linear_path(W8, 8, 120000, 1728, NONE) == 4    # (below 200 Mi)
     assert sq.sq_linear_path(W16, 2, 2048, 1536, NONE) == 0     # FP16 rows: not the ring
-    assert sq.sq_linear_path(W4, 9, 2048, 1536, NONE) == 0      # nine rows: not the ring
+    assert sq.sq_linear_path(W4, 9, 2048, 1536, NONE) == 4      # nine rows
+    assert sq.sq_linear_path(W16, 5, 5120, 5120, RES) == 4      # 14B o
+    assert sq.sq_linear_path(W16, 6, 896, 4864, NONE) == 4      # six rows: any size below K = 8192
+    assert sq.sq_linear_path(W16, 2, 13824, 5120, SILU) == 4    # 14B fused gate/up at two rows
+    assert sq.sq_linear_path(W16, 2, 8960, 1536, SILU) == 0     # the 1.5B one (27.5 Mi)
     assert sq.sq_linear_path(W8, 1, 151936, 1536, NONE) == 0    # 1.5B FP8 lm_head (233 Mi)
     assert sq.sq_linear_path(W8, 1, 152064, 5120, NONE) == 3    # 14B FP8 lm_head (779 Mi)
     assert sq.sq_linear_path(W8, 1, 13824, 5120, SILU) == 0
@@ -160,4 +168,4 @@ def test_single_row_engine_choice(lib):
     assert sq.sq_linear_path(W16, 1, 8960, 1536, SILU) == 3     # FP16 fused gate/up (27.5 Mi)
     assert sq.sq_linear_path(W16, 1, 4864, 896, SILU) == 0      # 0.5B-shaped (8.7 Mi)
     assert sq.sq_linear_path(W16, 1, 2048, 1536, NONE) == 0
-    assert sq.sq_linear_path(W16, 5, 151936, 1536, NONE) == 0   # five rows: not the ring
+    assert sq.sq_linear_path(W16, 5, 151936, 1536, NONE) == 4   # five rows

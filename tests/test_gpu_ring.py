@@ -3,7 +3,7 @@ III-D.2 draft pass at batch 1, and direct decoding with the parent) against
 the fp64 oracle over the same dequantised weights.
 
 The cases are shapes sq_linear_path sends to the ring (engine 3), at one
-activation row and at two to eight (INT4 and FP8): ragged
+activation row and at two to eight (large FP8 lm_heads): ragged
 last tiles, row splits over several warps (few tiles) and whole-row jobs
 (many tiles), partial last stages, the epilogues (bias, SiLU gate,
 residual), calls chained on one stream that read the previous call's output
@@ -101,21 +101,18 @@ CASES = [
     ("fp16", 9400 + 5, 896, SILU), ("fp16", 2048, 4096 + 128, SILU),
     # INT4 fused gate/up of >= 64 Mi weights (even group count)
     ("int4", 13824 + 9, 2560, SILU), ("int4", 2048 + 16, 16384, SILU),
+    # rows so long that the staged one leaves room for 12 and for 8 warps
+    ("int4", 800 + 3, 49152, SILU), ("int4", 600, 65536, SILU),
     # FP8 lm_head-like (>= 400 Mi weights)
     ("fp8", 110003, 4096, NONE), ("fp8", 51203, 8192 + 128, RES),
 ]
 
 
-# two to eight activation rows (INT4 and FP8 drafts at batch > 1): every
-# row count's column layout, ragged tiles, the K split, the epilogues
+# two to eight activation rows of large FP8 lm_heads: every row count's column
+# layout, ragged tiles, long rows
 CASES_M = [
-    ("int4", 2, 7168 + 5, 5120, NONE), ("int4", 3, 1000, 2048, RES), ("int4", 4, 13824, 5120, SILU),
-    ("int4", 5, 5120, 5120, NONE), ("int4", 8, 4133, 1536, SILU), ("int4", 8, 152064, 5120, NONE),
-    ("int4", 4, 5120, 13824, RES), ("fp8", 8, 7168, 5120, NONE), ("fp8", 5, 300, 1024, SILU),
-    ("fp8", 4, 37, 13824, RES),
-    # INT4 warp counts when the staged rows leave less room: 12 warps at two
-    # rows of K = 27648, 8 warps at eight rows of K = 8192
-    ("int4", 2, 3000, 27648, SILU), ("int4", 8, 1000 + 3, 8192, RES),
+    ("fp8", 2, 65536 + 5, 3328, NONE), ("fp8", 3, 110003, 2048, RES), ("fp8", 4, 65551, 8192, NONE),
+    ("fp8", 5, 70001, 3200, NONE), ("fp8", 7, 136573, 1536, RES), ("fp8", 8, 65536, 3328, NONE),
 ]
 
 
@@ -134,7 +131,9 @@ def test_ring_rows_match_oracle(kind, M, N, K, epi):
 
 @pytest.mark.parametrize("kind,N,K,epi", CASES)
 def test_ring_matches_oracle(kind, N, K, epi):
-    x = f16_to_dev(synth.activations_fp16(N % 1000 + K, 1, K))
+    # (a quarter of the longest rows' activations: gated results stay below 32, where
+    # the fp16 rounding of the exact one is within the bar)
+    x = f16_to_dev(synth.activations_fp16(N % 1000 + K, 1, K) * np.float16(0.25 if K > 40000 else 1.0))
     res = f16_to_dev(synth.activations_fp16(N % 777, 1, N)) if epi == RES else None
     op = _Op(kind, N * 7 + K, N, K, x, epi=epi, bias=(N % 2 == 1), residual=res)
     op.run()

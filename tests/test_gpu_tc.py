@@ -128,21 +128,21 @@ def test_tc_fp8_full_size_qkv_7b_sampled():
     assert_close(dev_to_f64(y)[:, cols], oracle.linear(x64, oracle.dequant_fp8(c, s)), "fp8 7B qkv M=48")
 
 
-# Below 16 rows the tensor-core path takes the formats and shapes where it
-# is faster than the CUDA-core GEMV; rows past M are zero-filled tile rows.
+# Below 16 rows the tensor-core path takes the formats and shapes where it is
+# faster than the streaming engine (or that one cannot take: K) and the CUDA-core
+# GEMV; rows past M are zero-filled tile rows.
 SMALL_M_TC = [
     ("fp16", 3, 384, 8960, sq.SQ_EPI_NONE),      # long rows
     ("fp16", 5, 200, 8192, sq.SQ_EPI_NONE),
-    ("fp16", 7, 65600, 2048, sq.SQ_EPI_NONE),    # wide output
+    ("fp16", 7, 65600, 2056, sq.SQ_EPI_NONE),    # wide output (K not in whole units of the streaming engine)
     ("fp16", 5, 2816, 3072, sq.SQ_EPI_SILU_GATE),
     ("fp16", 8, 200, 1000, sq.SQ_EPI_NONE),
     ("fp16", 9, 1536, 1536, sq.SQ_EPI_NONE),
     ("fp16", 15, 300, 640, sq.SQ_EPI_NONE),
-    ("fp8", 9, 200, 1024, sq.SQ_EPI_NONE),
+    ("fp8", 9, 200, 1040, sq.SQ_EPI_NONE),
     ("fp8", 9, 384, 8960, sq.SQ_EPI_NONE),
-    ("fp8", 12, 256, 1536, sq.SQ_EPI_SILU_GATE),
-    ("int4", 9, 1024, 8192, sq.SQ_EPI_NONE),
-    ("int4", 13, 2048, 4096, sq.SQ_EPI_NONE),
+    ("fp8", 12, 256, 1552, sq.SQ_EPI_SILU_GATE),
+    ("fp8", 14, 3200, 2048, sq.SQ_EPI_NONE),
 ]
 
 
@@ -174,13 +174,17 @@ def test_engine_choice_small_rows():
     assert sq.sq_linear_path(sq.SQ_W_INT4, 1, 2048, 1536, sq.SQ_EPI_NONE) == 0
     assert sq.sq_linear_path(sq.SQ_W_FP8, 1, 151936, 1536, sq.SQ_EPI_NONE) == 0
     assert sq.sq_linear_path(sq.SQ_W_FP16, 5, 2048, 1536, sq.SQ_EPI_NONE) == 0
-    assert sq.sq_linear_path(sq.SQ_W_FP16, 5, 151936, 1536, sq.SQ_EPI_NONE) == 0
-    # two to eight INT4 / FP8 rows: the shared-memory ring engine
-    assert sq.sq_linear_path(sq.SQ_W_FP8, 5, 17920, 1536, sq.SQ_EPI_NONE) == 3
-    assert sq.sq_linear_path(sq.SQ_W_INT4, 8, 2048, 1536, sq.SQ_EPI_NONE) == 3
-    assert sq.sq_linear_path(sq.SQ_W_INT4, 8, 5120, 13824, sq.SQ_EPI_NONE) == 1  # 8 rows x 13824: no room
-    # from 16 rows on: tensor cores
-    assert sq.sq_linear_path(sq.SQ_W_INT4, 16, 2048, 1536, sq.SQ_EPI_NONE) == 1
+    # two to sixteen rows: the streaming engine, where it is faster
+    assert sq.sq_linear_path(sq.SQ_W_FP16, 5, 151936, 1536, sq.SQ_EPI_NONE) == 4
+    assert sq.sq_linear_path(sq.SQ_W_FP8, 5, 17920, 1536, sq.SQ_EPI_NONE) == 4
+    assert sq.sq_linear_path(sq.SQ_W_INT4, 8, 2048, 1536, sq.SQ_EPI_NONE) == 4
+    assert sq.sq_linear_path(sq.SQ_W_INT4, 8, 5120, 13824, sq.SQ_EPI_NONE) == 4
+    assert sq.sq_linear_path(sq.SQ_W_INT4, 16, 2048, 1536, sq.SQ_EPI_NONE) == 4
+    assert sq.sq_linear_path(sq.SQ_W_FP16, 5, 5120, 13824, sq.SQ_EPI_NONE) == 1  # long rows in 40 weight tiles
+    assert sq.sq_linear_path(sq.SQ_W_FP16, 8, 4608, 3584, sq.SQ_EPI_NONE) == 1
+    # then tensor-core tiles
+    assert sq.sq_linear_path(sq.SQ_W_INT4, 16, 1536, 1536, sq.SQ_EPI_NONE) == 1
+    assert sq.sq_linear_path(sq.SQ_W_INT4, 17, 2048, 1536, sq.SQ_EPI_NONE) == 1
     assert sq.sq_linear_path(sq.SQ_W_FP16, 16, 128, 64, sq.SQ_EPI_NONE) == 1
     # sizes sq_linear_ex rejects
     assert sq.sq_linear_path(sq.SQ_W_INT4, 1, 256, 100, sq.SQ_EPI_NONE) == -1
@@ -208,12 +212,12 @@ def test_tc_silu_largest_m(kind):
 
 
 @pytest.mark.parametrize("M,N,K,epi", [
-    (16, 8192, 5120, sq.SQ_EPI_NONE),         # 21.5 MB of INT4: two CTAs per SM, split 4
-    (8, 5120, 13824, sq.SQ_EPI_NONE),         # the 14B down shape: split 8
-    (16, 2 * 6912, 5120, sq.SQ_EPI_SILU_GATE),  # a fused gate/up of 36 MB: split 2
+    (17, 8192, 5120, sq.SQ_EPI_NONE),         # 21.5 MB of INT4: two CTAs per SM, split 4
+    (33, 5120, 13824, sq.SQ_EPI_NONE),        # the 14B down shape: split 8
+    (64, 2 * 6912, 5120, sq.SQ_EPI_SILU_GATE),  # a fused gate/up of 36 MB: split 2
 ])
 def test_tc_int4_large_matrices_sampled(M, N, K, epi):
-    # INT4 matrices of 20 MB and more at few rows take their own split rule;
+    # INT4 matrices of 20 MB and more at up to 64 rows take their own split rule;
     # checked on sampled output columns (the oracle dequantises those rows)
     w = synth.weights_fp16(N + K + M, N, K)
     x = synth.activations_fp16(M + 3, M, K)
