@@ -543,28 +543,34 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   unsigned long long m0 = r0, m1 = r1;
   if (use_p) {
     if constexpr (Src::kUnit) {
-      // no mass in the residual (rare): the row's own, chunk by chunk
+      // no mass in the residual (rare): the row's own, a warp per chunk, into the
+      // second slot of the partials
       const auto pn = src.prow(b, n);
-      m0 = m1 = 0;
-      for (int c = 0; c < a.C; ++c) {
-        const int64_t v0 = (int64_t)c * a.chunk;
-        const int64_t v1 = v0 + a.chunk < V ? v0 + a.chunk : V;
-        const int64_t vb = v0 + 8 * (int64_t)tid;
-        unsigned long long sum = 0;
-        if (vb < v1) {
-          float pv[8];
-          pn.load8(vb, v1, pv);
+      for (int c = warp; c < a.C; c += kAcceptThreads / 32) {
+        uint32_t hi = 0, lo = 0, cnt = 0;
+#pragma unroll 1
+        for (int64_t v0 = (int64_t)c * kAcceptChunk + 8 * lane; v0 < (int64_t)(c + 1) * kAcceptChunk; v0 += 1024) {
+          uint4 pr[4];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) sum += fix44(pv[j]);
+          for (int i = 0; i < 4; ++i)
+            if (v0 + 256 * i < V) pr[i] = pn.raw8(v0 + 256 * i, V);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (v0 + 256 * i < V) {
+              float pv[8];
+              pn.sum8(pr[i], v0 + 256 * i, V, pv);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) add_fix44(pv[j], hi, lo);
+              cnt += 8;
+            }
         }
-        sum = block_sum_u64<kAcceptThreads>(sum, blk);
-        if (c == c0) m0 = sum;
-        if (c == c1) m1 = sum;
+        const unsigned long long sum = warp_sum_u64(fix44_total(hi, lo, cnt));
+        if (lane == 0) a.part[((int64_t)b * a.C + c) * a.slots + 1] = sum;
       }
-    } else {
-      m0 = partial(c0, 1);
-      m1 = partial(c1, 1);
+      __syncthreads();
     }
+    m0 = partial(c0, 1);
+    m1 = partial(c1, 1);
     S = block_sum_u64<kAcceptThreads>(m0 + m1, blk);
   }
   const int ok = s_valid && S != 0;

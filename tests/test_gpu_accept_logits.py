@@ -113,6 +113,27 @@ def test_accept_logits_outcome_spread():
     assert len(set(on.tolist())) >= 3
 
 
+@pytest.mark.parametrize("V", [5, 2041, 2048, 8201, 152064])  # chunks of 2048, pieces of eight
+def test_residual_without_mass_samples_the_row(V):
+    B, K = 3, 4
+    rng = np.random.default_rng(V)
+    zp = rng.normal(0, 2.0, (B, K + 1, V)).astype(np.float16)
+    draft = rng.integers(0, V, (B, K)).astype(np.int32)
+    for b in range(B):  # the drafted tokens have no probability, all others the draft's: residual zero
+        zp[b, np.arange(K), draft[b]] = np.float16(-60000.0)
+    zq = np.ascontiguousarray(np.transpose(zp[:, :K], (1, 0, 2)))
+    u = np.concatenate([rng.random((B - 1, K + 1)), np.full((1, K + 1), 0.99999994)]).astype(np.float32)
+    ws = torch.zeros(sq.sq_accept_logits_workspace_bytes(B, K, V), dtype=torch.uint8, device=dev())
+    n = torch.empty(B, dtype=torch.int32, device=dev())
+    tok = torch.empty(B, K + 1, dtype=torch.int32, device=dev())
+    _, on, otok = oracle.accept_logits(zp, zq, draft, u, 1.0)
+    assert not on.any()
+    for _ in range(2):
+        sq.sq_accept_logits(_t(zp), _t(zq), _t(draft), _t(u), 1.0, sq.SQ_ACCEPT_SAMPLE, n, tok, ws)
+        assert sq.sq_check() == 0
+        assert np.array_equal(n.cpu().numpy(), on) and np.array_equal(tok.cpu().numpy(), otok)
+
+
 @pytest.mark.parametrize("B,V,T", [(1, 151936, 1.0), (7, 12345, 0.6)])
 def test_sample_logits_matches_oracle(B, V, T):
     rng = np.random.default_rng(B + V)
