@@ -74,6 +74,7 @@ CASES = [
     (2, 8, 32000, 1.0, 0.5, sq.SQ_ACCEPT_GREEDY),
     (5, 3, 4097, 2.0, None, sq.SQ_ACCEPT_GREEDY),
     (6, 0, 20000, 1.0, None, sq.SQ_ACCEPT_SAMPLE),
+    (40, 8, 18001, 1.0, 0.5, sq.SQ_ACCEPT_GREEDY),  # more than two chunks for every CTA place
 ]
 
 
