@@ -858,10 +858,13 @@ __global__ void __launch_bounds__(kAcceptThreads) softmax_stats_kernel(SoftmaxAr
 
 static cudaError_t launch_stats(const SoftmaxArgs& sa, cudaStream_t st) {
   // CTAs per row: one per 2048 entries, up to 8 (16 for few rows, where a row
-  // per 8 CTAs would leave most of the GPU idle)
+  // per 8 CTAs would leave most of the GPU idle), but half as many, and half
+  // again, while that fills the GPU and a row still fits its threads' registers
   const int64_t want = (sa.V + 8 * kAcceptThreads - 1) / (8 * kAcceptThreads);
   const int most = sa.rows * kStatsMaxCluster <= 4 * device_sm_count() ? kStatsMaxCluster : 8;
-  const int CL = (int)(want < most ? want : most);
+  int CL = (int)(want < most ? want : most);
+  while (CL > 1 && sa.rows * ((CL + 1) / 2) >= 4 * device_sm_count() && want <= kStatsKeep * (int64_t)((CL + 1) / 2))
+    CL = (CL + 1) / 2;
   static std::mutex mu;
   static bool ready[64] = {false};
   int dev = 0;

@@ -37,7 +37,8 @@ def _t(a):
     return torch.from_numpy(np.ascontiguousarray(a)).to(dev())
 
 
-@pytest.mark.parametrize("R,V,T", [(5, 151936, 1.0), (3, 152064, 0.7), (33, 9001, 2.3), (1, 1, 1.0)])
+@pytest.mark.parametrize("R,V,T", [(5, 151936, 1.0), (3, 152064, 0.7), (33, 9001, 2.3), (1, 1, 1.0), (303, 6001, 1.0), (305, 6001, 1.0),
+                                   (410, 4097, 0.9), (700, 8000, 1.0)])  # CTAs a row: as the rows fill the SMs
 def test_softmax_bit_exact(R, V, T):
     z = np.random.default_rng(R * V).normal(0, 3.0, (R, V)).astype(np.float16)
     ws = torch.zeros(sq.sq_softmax_workspace_bytes(R, V), dtype=torch.uint8, device=dev())
