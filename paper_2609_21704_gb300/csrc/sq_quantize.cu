@@ -55,7 +55,7 @@ __device__ __forceinline__ uint32_t int4_code(float w, float s) {
   return (uint32_t)((int)fminf(fmaxf(rintf(__fdiv_rn(w, s)), -8.0f), 7.0f) + 8);
 }
 
-// A warp takes 1024 consecutive weights, eight groups, as four coalesced
+// A warp takes 1024 consecutive weights (PER = 4), eight groups, as four coalesced
 // 16-byte loads a lane (lane l holds chunk 32 i + l: sixteen lanes a group and
 // load).  The maxima of a lane's four groups are reduced together, packed in
 // pairs; lane j mod 4 then divides for group j only, so a group's two divides
@@ -63,66 +63,76 @@ __device__ __forceinline__ uint32_t int4_code(float w, float s) {
 // 5120) takes 73 us, 4.9 TB/s of the measured 6.8; one lane per four weights
 // with a divide per weight took 214.  Bound: about half issue slots (7 a
 // weight), half memory.
+// PER = 1: 256 weights a warp, for matrices that leave SMs without one otherwise
+// (100 x 1024: 2.9 us with four, 2.1 with one).
+template <int PER>
 __global__ void __launch_bounds__(kQuantThreads) quant_int4_kernel(const __half* __restrict__ w, int64_t N,
                                                                    int64_t K, uint8_t* __restrict__ codes,
                                                                    __half* __restrict__ scales) {
   griddep_wait();  // no early trigger: a linear call may read these outputs at once
   const int lane = threadIdx.x & 31;
   const int64_t total = N * (K / 8);  // chunks; a row is whole groups of 16, so groups are contiguous
-  const int64_t step = (int64_t)gridDim.x * (kQuantThreads / 32) * 128;
-  for (int64_t c0 = ((int64_t)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5)) * 128; c0 < total; c0 += step) {
-    uint4 v[4];
-    uint32_t m[4];
+  const int64_t step = (int64_t)gridDim.x * (kQuantThreads / 32) * 32 * PER;
+  for (int64_t c0 = ((int64_t)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5)) * 32 * PER; c0 < total; c0 += step) {
+    uint4 v[PER];
+    uint32_t m[PER];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < PER; ++i) {
       const int64_t c = c0 + 32 * i + lane;  // the lanes of a group are in or out together
       v[i] = c < total ? ld_stream16(w + 8 * c) : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < PER; ++i) {
       m[i] = absmax8(v[i], 0u);
       m[i] = max(m[i] & 0xffffu, m[i] >> 16);
     }
-    uint32_t pk[2] = {m[0] | (m[1] << 16), m[2] | (m[3] << 16)};
+    // this lane's group: load lane mod PER, half-warp lane >> 4
+    uint32_t mine;
+    if constexpr (PER == 4) {
+      uint32_t pk[2] = {m[0] | (m[1] << 16), m[2] | (m[3] << 16)};
 #pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-      pk[0] = __vmaxu2(pk[0], __shfl_xor_sync(0xffffffffu, pk[0], o));
-      pk[1] = __vmaxu2(pk[1], __shfl_xor_sync(0xffffffffu, pk[1], o));
+      for (int o = 1; o < 16; o <<= 1) {
+        pk[0] = __vmaxu2(pk[0], __shfl_xor_sync(0xffffffffu, pk[0], o));
+        pk[1] = __vmaxu2(pk[1], __shfl_xor_sync(0xffffffffu, pk[1], o));
+      }
+      mine = ((lane & 2 ? pk[1] : pk[0]) >> (16 * (lane & 1))) & 0xffffu;
+    } else {
+      mine = m[0];
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) mine = max(mine, __shfl_xor_sync(0xffffffffu, mine, o));
     }
-    // this lane's group: load lane & 3, half-warp lane >> 4
-    const uint32_t mine = ((lane & 2 ? pk[1] : pk[0]) >> (16 * (lane & 1))) & 0xffffu;
     const bool bad = mine >= 0x7c00u;
     float amax = __half2float(__ushort_as_half((uint16_t)mine));
     if (__any_sync(0xffffffffu, bad)) {
       // the largest magnitude that is not NaN, as fmaxf takes it
       float keep = amax;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < PER; ++i) {
         float f[8], a = 0.0f;
         halves8(v[i], f);
 #pragma unroll
         for (int e = 0; e < 8; ++e) a = fmaxf(a, fabsf(f[e]));
 #pragma unroll
         for (int o = 1; o < 16; o <<= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-        if ((lane & 3) == i) keep = a;
+        if (lane % PER == i) keep = a;
       }
       amax = keep;
-      if (bad && (lane & 12) == 0) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
+      if (bad && (lane & 15) < PER) atomicOr(&g_quant_status, SQ_DEV_NONFINITE_WEIGHT);
     }
     __half sh = __float2half_rn(__fdiv_rn(amax, 7.0f));
     if (amax > 0.0f && __half_as_ushort(sh) == 0) sh = __ushort_as_half(1);
     const float s = __half2float(sh);
     // -1: the codes by division (below the normal scales a code can pass 7)
     const float r = bad || s < 0x1p-14f ? -1.0f : __fdiv_rn(1.0f, s);
-    if ((lane & 12) == 0) {
-      const int64_t g = (c0 >> 4) + 2 * (lane & 3) + (lane >> 4);
+    if ((lane & 15) < PER) {
+      const int64_t g = (c0 >> 4) + 2 * (lane % PER) + (lane >> 4);
       if (g < (total >> 4)) scales[g] = sh;
     }
     // codes by bracketing: fma(w, r, magic) rounds the quotient into the low
     // bits of the sum, the integer sums of those bits (shifted) place the nibbles
     const float magic = 12582912.0f + 8.0f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < PER; ++i) {
       const int src = (lane & 16) | i;
       const float gs = __shfl_sync(0xffffffffu, s, src), gr = __shfl_sync(0xffffffffu, r, src);
       const float rlo = gr * (1.0f - 0x1p-21f), rhi = gr * (1.0f + 0x1p-21f);
@@ -250,9 +260,12 @@ cudaError_t launch_quant_int4(const void* w, int64_t N, int64_t K, void* codes, 
                               cudaStream_t st) {
   const int64_t total = N * (K / 8);
   if (total == 0) return cudaSuccess;
-  const int64_t want = (total + 4 * kQuantThreads - 1) / (4 * kQuantThreads);
   const int64_t cap = (int64_t)device_sm_count() * 16;
-  return launch_pdl(quant_int4_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kQuantThreads), 0, st,
+  const bool few = total <= (int64_t)device_sm_count() * 4 * kQuantThreads;
+  const int64_t per = (few ? 1 : 4) * kQuantThreads;
+  const int64_t want = (total + per - 1) / per;
+  return launch_pdl(few ? quant_int4_kernel<1> : quant_int4_kernel<4>, dim3((unsigned)(want < cap ? want : cap)),
+                    dim3(kQuantThreads), 0, st,
                     reinterpret_cast<const __half*>(w), N, K, reinterpret_cast<uint8_t*>(codes),
                     reinterpret_cast<__half*>(scales));
 }

@@ -47,7 +47,8 @@ def _rows(N, K, seed):
     return w
 
 
-@pytest.mark.parametrize("N,K", [(1, 128), (3, 384), (9, 128), (37, 1152), (130, 256)])
+@pytest.mark.parametrize("N,K", [(1, 128), (3, 384), (9, 128), (37, 1152), (130, 256),
+                                 (1216, 1024), (1217, 1024)])  # the most with 256 weights a warp, the least with 1024
 def test_int4_partial_warps_ties_and_small_scales(N, K):
     _check(_rows(N, K, N + K), sq.SQ_INT4_G128)
 
