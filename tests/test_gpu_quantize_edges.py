@@ -53,22 +53,24 @@ def test_int4_partial_warps_ties_and_small_scales(N, K):
     _check(_rows(N, K, N + K), sq.SQ_INT4_G128)
 
 
-@pytest.mark.parametrize("N,K", [(5, 2032), (9, 2048), (5, 2064), (2, 16384), (3, 16400), (2, 40000)])
+@pytest.mark.parametrize("N,K", [(5, 2032), (9, 2048), (5, 2064), (2, 16384), (3, 16400), (2, 40000),
+                                 (455, 272), (456, 272), (459, 2032), (461, 2048), (460, 2064)])  # a warp per row
 def test_fp8_row_lengths_ties_and_small_scales(N, K):
     _check(_rows(N, K, N + K), sq.SQ_FP8_E4M3_ROW)
 
 
+@pytest.mark.parametrize("N", [4, 460])  # a CTA per row, a warp per row
 @pytest.mark.parametrize("K", [16, 2048, 4112])
-def test_fp8_rows_of_nan_and_zeros_get_code_zero(K):
+def test_fp8_rows_of_nan_and_zeros_get_code_zero(N, K):
     """A row whose largest number is zero has scale 0 and codes +0, also where
     eight neighbouring weights are all NaN (both bounds of a quotient are)."""
-    w = np.zeros((4, K), dtype=np.float16)
+    w = np.zeros((N, K), dtype=np.float16)
     w[0] = np.nan
     w[1, 8:16] = np.nan
     w[2, K - 8:K - 1] = np.nan
     w[3] = -0.0
-    codes = torch.full((4, K), 7, dtype=torch.uint8, device=dev())
-    scales = torch.full((4,), 7.0, dtype=torch.float32, device=dev())
+    codes = torch.full((N, K), 7, dtype=torch.uint8, device=dev())
+    scales = torch.full((N,), 7.0, dtype=torch.float32, device=dev())
     sq.sq_quantize(f16_to_dev(w), sq.SQ_FP8_E4M3_ROW, codes, scales)
     assert sq.sq_check() & sq.SQ_DEV_NONFINITE_WEIGHT
     assert not scales.any()
