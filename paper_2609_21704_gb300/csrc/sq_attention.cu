@@ -223,7 +223,6 @@ struct AttnCfg {
   static constexpr int kKeysWarp = kBlockKeys / kWK;   // keys of a block a warp takes
   static constexpr int kKeysStep = kKeysWarp < 32 ? kKeysWarp : 32;
   static constexpr int kStages = WM > 1 ? 2 : 3;
-  static constexpr int kMaxTokens = kQT < kMaxT && WM < 4 ? kQT : kMaxT;  // new tokens a launch may have
   static constexpr int kQBytes = WM * NT * 4096;       // packed query tiles
   static constexpr int kOffFac = kQBytes;              // per query: factor of its scores
   static constexpr int kOffStage = kOffFac + (kQT * 4 + 127) / 128 * 128;
@@ -840,33 +839,38 @@ size_t attention_workspace_bytes(int B, int T, int Hq, int Hkv, int64_t max_ctx)
 int attention_max_tokens() { return kMaxT; }
 
 constexpr int kAttnMaxCluster = 16;
+constexpr int kTwoPerSmTokens = 24;  // new tokens up to which two CTAs of every instance share an SM
+constexpr int kShortBlocks = 8;
 
 // Prepares an instance and returns how many clusters of S of its CTAs can be
-// resident (cached per device and S; S = 0: only prepares).
+// resident (cached per device, S and shared memory of up to kTwoPerSmTokens or
+// kMaxT new tokens; S = 0: only prepares).
 template <int WM, int NT>
-static cudaError_t attn_resident(int S, int* n) {
+static cudaError_t attn_resident(int S, int T, int* n) {
   auto k = attention_kernel<WM, NT>;
-  constexpr int kMaxSmem = attn_smem(AttnCfg<WM, NT>::kOffCs, AttnCfg<WM, NT>::kMaxTokens);
+  constexpr int kSmem[2] = {attn_smem(AttnCfg<WM, NT>::kOffCs, kTwoPerSmTokens),
+                            attn_smem(AttnCfg<WM, NT>::kOffCs, kMaxT)};
   static std::mutex mu;
   static bool ready[64] = {false};
-  static int cache[64][kAttnMaxCluster + 1] = {};
+  static int cache[64][2][kAttnMaxCluster + 1] = {};
+  const int wide = T > kTwoPerSmTokens;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
   if (!ready[dev]) {
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem[1]);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     ready[dev] = true;
   }
   if (S == 0) return cudaSuccess;
-  if (cache[dev][S] == 0) {
+  if (cache[dev][wide][S] == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)S);
     cfg.blockDim = dim3(kAttnThreads);
-    cfg.dynamicSmemBytes = (size_t)kMaxSmem;
+    cfg.dynamicSmemBytes = (size_t)kSmem[wide];
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)S;
@@ -878,9 +882,9 @@ static cudaError_t attn_resident(int S, int* n) {
       (void)cudaGetLastError();
       c = 0;
     }
-    cache[dev][S] = c + 1;
+    cache[dev][wide][S] = c + 1;
   }
-  *n = cache[dev][S] - 1;
+  *n = cache[dev][wide][S] - 1;
   return cudaSuccess;
 }
 
@@ -903,12 +907,12 @@ static cudaError_t launch_attn_inst(AttnArgs a, cudaStream_t st) {
   if (S < 1) S = 1;
   a.cluster = S > 1 && (S <= kAttnMaxCluster || blocks <= kAttnMaxCluster * 16);
   int n = 0;
-  cudaError_t e = attn_resident<WM, NT>(0, &n);
+  cudaError_t e = attn_resident<WM, NT>(0, a.T, &n);
   if (e != cudaSuccess) return e;
   if (a.cluster) {
     if (S > kAttnMaxCluster) S = kAttnMaxCluster;
     for (; S > 1; --S) {
-      e = attn_resident<WM, NT>((int)S, &n);
+      e = attn_resident<WM, NT>((int)S, a.T, &n);
       if (e != cudaSuccess) return e;
       if (n >= base) break;
     }
@@ -966,7 +970,19 @@ cudaError_t launch_attention(const __half* qkv, int B, int T, int Hq, int Hkv, c
   a.max_ctx = max_ctx;
   a.rf = rope_freq(theta);
   a.scale = 1.0f / sqrtf((float)kHeadDim);
-  if (a.Q <= 8) return launch_attn_inst<1, 1>(a, st);
+  // Instances by the group's queries, so that the keys are read once a group.
+  // A cache of at most kShortBlocks blocks has no keys to share out, and a CTA's
+  // time is its chain of queries: there eight queries a CTA while those CTAs are
+  // resident at once (one block, above 32 queries: two rounds of them still are
+  // faster; above kTwoPerSmTokens one such CTA fills an SM).  Cache of 64, 28 / 4
+  // heads, 7 tokens: 1 sequence 21.5 -> 7.2 us, 16 sequences 21.8 -> 14.4; cache
+  // of 512, 40 / 8 heads, 4 tokens: 10.8 -> 7.8.  20 tokens of 16 sequences, 8 / 8
+  // heads (384 CTAs of 32 queries at most): 13.9, with eight 16.0.
+  const int64_t blocks = (max_ctx + kBlockKeys - 1) / kBlockKeys;
+  const int64_t sms = device_sm_count(), groups = (int64_t)B * Hkv * ((a.Q + 7) / 8);
+  const bool few = blocks <= kShortBlocks && (T <= kTwoPerSmTokens ? groups <= (blocks == 1 && a.Q > 32 ? 4 : 2) * sms
+                                                                   : groups * blocks <= sms);
+  if (a.Q <= 8 || few) return launch_attn_inst<1, 1>(a, st);
   if (a.Q <= 16) return launch_attn_inst<1, 2>(a, st);
   if (a.Q <= 32) return launch_attn_inst<2, 2>(a, st);
   return launch_attn_inst<4, 2>(a, st);

@@ -57,8 +57,21 @@ def _case(B, T, Hq, Hkv, pos0, max_ctx, qstd=1.0, fused=False, seed=0):
 @pytest.mark.parametrize("T,Hq,Hkv", [(8, 1, 1), (9, 1, 1), (4, 8, 2), (17, 2, 2), (32, 2, 1), (13, 5, 1),
                                       (25, 8, 1), (1, 40, 8), (2, 5, 1)])
 @pytest.mark.parametrize("ctx", [0, 63, 200])
-def test_query_counts(T, Hq, Hkv, ctx):
-    _case(1, T, Hq, Hkv, [ctx], 256, fused=T <= 9, seed=ctx)
+@pytest.mark.parametrize("max_ctx", [256, 577])  # eight queries a CTA up to 512; an instance per query count
+def test_query_counts(T, Hq, Hkv, ctx, max_ctx):
+    _case(1, T, Hq, Hkv, [ctx], max_ctx, fused=T <= 9, seed=ctx)
+
+
+@pytest.mark.parametrize("B,T,Hq,Hkv,max_ctx", [
+    (2, 24, 16, 2, 512), (2, 25, 16, 2, 512),  # two CTAs of eight queries on an SM; one
+    (1, 32, 6, 1, 64), (1, 32, 6, 1, 512),     # the most tokens: every group resident, and not
+    (3, 7, 28, 4, 513), (3, 7, 28, 4, 512),    # the longest short cache, and one entry more
+    (16, 7, 28, 4, 64), (24, 7, 28, 4, 64),    # two rounds of CTAs over one block; too many
+])
+@pytest.mark.parametrize("fused", [False, True])
+def test_short_caches(B, T, Hq, Hkv, max_ctx, fused):
+    _case(B, T, Hq, Hkv, [(37 * b) % (max_ctx - T + 1) for b in range(B - 1)] + [max_ctx - T], max_ctx, fused=fused,
+          seed=T)
 
 
 @pytest.mark.parametrize("ctx", [62, 63, 64, 127, 128])
