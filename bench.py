@@ -905,9 +905,9 @@ def main():
     draft_bytes = stack.weight_bytes(args.draft) + stack.activation_bytes(B)
     ver_bytes = stack.weight_bytes("fp16") + stack.activation_bytes(Mv)
     acc_bytes = B * (2 * V * 4 + 2 * K * 4)
-    # accept from logits: two statistics passes over the 2K+1 rows of fp16
+    # accept from logits: one statistics pass over the 2K+1 rows of fp16
     # logits, then the correction rows (p and q) once more
-    accl_bytes = B * ((2 * K + 1) * V * 2 * 2 + 2 * V * 2)
+    accl_bytes = B * ((2 * K + 1) * V * 2 + 2 * V * 2)
 
     # ---- dominant kernel: the fused gate/up + SiLU linear (largest per-launch
     # weight matrix in the layers); all layers' launches of it in one graph

@@ -167,8 +167,8 @@ SQ_API sq_status sq_linear_ex(sq_wkind wkind, const void* x, const void* w, cons
  * pre-norm projections (q/k/v, gate/up, lm_head) in one call.  rmsnorm is
  * sq_rmsnorm's (fp32 arithmetic, the normalised rows rounded to fp16) and
  * the result is bit-identical to sq_rmsnorm followed by sq_linear_ex.  The
- * CUDA-core GEMV normalises the activation rows as it stages them (no extra
- * launch); the tensor-core path and the shared-memory ring engine write them
+ * CUDA-core GEMV and the streaming engine normalise the activation rows as they
+ * stage them (no extra launch); the tensor-core path and the shared-memory ring engine write them
  * to xn (fp16 [M, K], 16-byte aligned, not aliasing x, y or the residual)
  * first.  gamma fp16 [K], 16-byte
  * aligned; eps >= 0. */
@@ -342,7 +342,8 @@ SQ_API sq_status sq_softmax(const void* z, int64_t R, int64_t V, float temperatu
  * q heads, then k heads, then v heads); D = 128; Hq a multiple of Hkv; token
  * t of sequence b is at position pos0[b] + t (pos0 int32 [B], device).
  * Caches k_cache, v_cache fp16 [B, Hkv, max_ctx, D], 16-byte aligned.  RoPE rotates pairs
- * (d, d + D/2) by pos * theta^(-2d/D) (angle computed in fp64).
+ * (d, d + D/2) by pos * theta^(-2d/D) (inverse frequencies rounded to 2^-64 of a
+ * turn on the host; the angle's reduction to one turn is exact).
  *
  * sq_kv_append: rotates the new keys and writes keys and values into the
  *   caches at their positions.  A position outside [0, max_ctx) writes

@@ -7,7 +7,7 @@
 // cache keeps only the accepted prefix.  Definitions (no model internals
 // are given in the paper; these are the Qwen2.5 decoder's):
 //   RMSNorm   y = x / sqrt(mean(x^2) + eps) * gamma       (fp32, fp16 out)
-//   RoPE      pairs (d, d + D/2), angle pos * theta^(-2d/D) (fp64 angle)
+//   RoPE      pairs (d, d + D/2), angle pos * theta^(-2d/D) in 2^-64 turns
 //   attention softmax(q . k / sqrt(D)) v over cache positions <= the
 //             query's position; query head h reads key/value head
 //             h / (Hq / Hkv).

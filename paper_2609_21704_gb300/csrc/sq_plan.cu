@@ -79,9 +79,9 @@ int gemv_cap_mr(int wk, int64_t K) {
 }
 
 // Tensor cores or CUDA cores, for the calls that neither the streaming engine
-// nor the ring takes.  From 16 rows on a CUDA-core GEMV is issue bound (16 fused multiply-adds per weight); below
-// that the choice follows timings of both paths on the 1.5B/7B/14B projection
-// shapes:
+// nor the ring takes.  From 16 rows on a CUDA-core GEMV is issue bound (16 fused
+// multiply-adds per weight); below that the choice follows timings of both paths
+// on the 1.5B/7B/14B projection shapes:
 //   * 8..15 rows: tensor cores for FP16 and FP8 weights (1.5-3x faster on
 //     every shape), and for INT4 weights from 8 Mi weights on (the INT4
 //     GEMV keeps small matrices, where its 8 x dequant reuse still pays);

@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(kQuantThreads) quant_int4_kernel(const __half*
   const int lane = threadIdx.x & 31;
   const int64_t total = N * (K / 8);  // chunks; a row is whole groups of 16, so groups are contiguous
   const int64_t step = (int64_t)gridDim.x * (kQuantThreads / 32) * 32 * PER;
-  for (int64_t c0 = ((int64_t)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5)) * 32 * PER; c0 < total; c0 += step) {
+  const int64_t wid = (int64_t)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5);
+  for (int64_t c0 = wid * 32 * PER; c0 < total; c0 += step) {
     uint4 v[PER];
     uint32_t m[PER];
 #pragma unroll

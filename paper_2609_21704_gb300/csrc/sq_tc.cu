@@ -2,18 +2,19 @@
 // padded to a multiple of 16 on the MMA's N side).
 //
 // Sec. III-D.3: the verify pass scores B * (K+1) rows at once (the draft
-// pass B rows).  sq_linear_ex sends a call here from 16 rows on, and from 3
-// to 15 rows for the formats and shapes where this path measured faster
-// than the CUDA-core GEMV (rows past M are zero-filled by the TMA load).  Swap-AB: the weight tile is the MMA's A
-// operand (M_mma = 128 weight rows), the activations are B (N_mma = NB, the
+// pass B rows).  sq_linear_ex sends every call of more than 16 rows here, and from
+// 3 to 16 rows the formats and shapes where this path measured faster than the
+// streaming engine and the CUDA-core GEMV (rows past M are zero-filled by the TMA
+// load).  Swap-AB: the weight tile is the MMA's A operand (M_mma = 128 weight rows), the activations are B (N_mma = NB, the
 // activation rows padded to a multiple of 16), D = 128 x NB fp32 in TMEM:
 //     D[n, m] = sum_k W[n, k] * x[m, k]   ->   y[m, n]
 // Both operands are K-major fp16 tiles of 64 k (128 bytes per row) loaded by
 // 2-D TMA with 128-byte swizzle into a ring of shared-memory stages; warp 0
 // lane 0 issues the TMA copies, warp 1 lane 0 issues tcgen05.mma (4 x K16
-// per stage) and commits each stage back to the producer; warps 2..9 read
-// the accumulator with tcgen05.ld (each warp half the columns of its 32-lane
-// TMEM sub-partition) and run the epilogue.  With the fused SiLU gate the CTA also loads the up
+// per stage) and commits each stage back to the producer; the epilogue warps,
+// from warp 2 on, read the accumulator with tcgen05.ld (two warps share a 32-lane
+// TMEM sub-partition and alternate blocks of its columns; up to 16 FP16 rows one
+// has them all) and run the epilogue.  With the fused SiLU gate the CTA also loads the up
 // rows' tile and accumulates a second NB-column block of TMEM.
 //
 // FP8 and INT4 weights: TMA brings the code tiles instead, and the eight
@@ -60,7 +61,7 @@ constexpr int kTcBK = 64;       // k per stage: 64 fp16 = one 128-byte swizzle r
 // -> 682 us, at 80 rows (and lm_head) 794 -> 759; 7B at 256 1182 -> 963; 1.5B at
 // 256 3576 -> 2529.  Up to 16 rows (FP16) a sub-partition has one block of
 // columns, and four warps leave registers to the next launch's CTA: 28 layers of
-// 1.5B at 9 rows 794 -> 784, a 1.5B decoder pass of three tokens 1342 -> 1330.
+// 1.5B at 16 rows 802 -> 795, a 1.5B decoder pass of three tokens 1318 -> 1314.
 constexpr int tc_threads(int ew) { return 64 + 32 * ew; }
 constexpr int kTcStageA = kTcBM * kTcBK * 2;  // 16 KB
 // CTAs per cluster along K: up to 16 (non-portable cluster size, allowed at
@@ -488,8 +489,8 @@ __global__ void __launch_bounds__(tc_threads(EW), 1)
         const int up = SILU && c0 >= a.NB ? 1 : 0;
         const int mb = c0 - up * a.NB;
         int owner = mb / cper, mc = mb - owner * cper;
-        const uint32_t base =
-            smem_u32(smem) + (uint32_t)a.part_off + (uint32_t)((((int)rank * (SILU ? 2 : 1) + up) * cper * kTcBM + row) * 4);
+        const int off = (((int)rank * (SILU ? 2 : 1) + up) * cper * kTcBM + row) * 4;
+        const uint32_t base = smem_u32(smem) + (uint32_t)a.part_off + (uint32_t)off;
         uint32_t remote = map_rank(base, (uint32_t)min(owner, S - 1));
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
