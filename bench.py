@@ -722,7 +722,7 @@ def main():
         sq.sq_accept_logits(zp, zq, td, tu, temperature, sq.SQ_ACCEPT_SAMPLE, n_out, tok_out, ws_l,
                             stream)
 
-    launches_per_step = (K + 1) * stack.launches_per_pass() + 3 * K + 3
+    launches_per_step = (K + 1) * stack.launches_per_pass() + 2 * K + 2
 
     def capture(fn):
         with torch.cuda.stream(stream):
