@@ -383,12 +383,14 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   if constexpr (Src::kUnit) {
     if (a.mode == SQ_ACCEPT_SAMPLE) {
       // all of the CTA's chunks at once: their loads, their sums, one barrier.
-      // (The row's own mass, for a residual without any, is summed only if it
-      // turns out to be wanted.)
+      // The row's own mass is wanted only if the whole residual is zero: a warp
+      // sums its share where its residual is (slot 1 is complete then), in a loop
+      // of its own, since code that is rarely run costs the others their fetches.
       const auto pn = src.prow(b, n);
       const bool use_q = n < K;
       const auto qn = src.qrow(b, use_q ? n : 0);
       uint4 pr[kAcceptMaxCpc], qr[kAcceptMaxCpc];
+      uint32_t zero = 0;  // chunks without residual in this warp
 #pragma unroll
       for (int i = 0; i < kAcceptMaxCpc; ++i) {
         const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
@@ -411,13 +413,38 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
           sr = fix44_total(hi, lo, 8);
         }
         sr = warp_sum_u64(sr);
-        if (lane == 0) red[warp][i] = sr;
+        if (sr == 0 && use_q) zero |= 1u << i;
+        if (lane == 0) {
+          red[warp][i] = sr;
+          red[warp][kAcceptMaxCpc + i] = 0;
+        }
+      }
+#pragma unroll 1
+      for (; zero != 0; zero &= zero - 1) {
+        const int i = __ffs(zero) - 1;
+        const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
+        unsigned long long sp = 0;
+        if (cb + i < ce && v < V) {
+          uint32_t hi = 0, lo = 0;
+          float pv[8];
+          pn.sum8(pn.raw8(v, V), v, V, pv);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) add_fix44(pv[j], hi, lo);
+          sp = fix44_total(hi, lo, 8);
+        }
+        sp = warp_sum_u64(sp);
+        if (lane == 0) red[warp][kAcceptMaxCpc + i] = sp;
       }
       __syncthreads();
       if (tid < ce - cb) {
-        unsigned long long tr = 0;
-        for (int w = 0; w < kAcceptThreads / 32; ++w) tr += red[w][tid];
-        a.part[((int64_t)b * a.C + cb + tid) * a.slots] = tr;
+        unsigned long long tr = 0, tp = 0;
+        for (int w = 0; w < kAcceptThreads / 32; ++w) {
+          tr += red[w][tid];
+          tp += red[w][kAcceptMaxCpc + tid];
+        }
+        unsigned long long* part = a.part + ((int64_t)b * a.C + cb + tid) * a.slots;
+        part[0] = tr;
+        part[1] = tp;
       }
     }
   }
@@ -542,33 +569,6 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   const int use_p = (S == 0 && n < K) ? 1 : 0;  // block-uniform
   unsigned long long m0 = r0, m1 = r1;
   if (use_p) {
-    if constexpr (Src::kUnit) {
-      // no mass in the residual (rare): the row's own, a warp per chunk, into the
-      // second slot of the partials
-      const auto pn = src.prow(b, n);
-      for (int c = warp; c < a.C; c += kAcceptThreads / 32) {
-        uint32_t hi = 0, lo = 0, cnt = 0;
-#pragma unroll 1
-        for (int64_t v0 = (int64_t)c * kAcceptChunk + 8 * lane; v0 < (int64_t)(c + 1) * kAcceptChunk; v0 += 1024) {
-          uint4 pr[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (v0 + 256 * i < V) pr[i] = pn.raw8(v0 + 256 * i, V);
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (v0 + 256 * i < V) {
-              float pv[8];
-              pn.sum8(pr[i], v0 + 256 * i, V, pv);
-#pragma unroll
-              for (int j = 0; j < 8; ++j) add_fix44(pv[j], hi, lo);
-              cnt += 8;
-            }
-        }
-        const unsigned long long sum = warp_sum_u64(fix44_total(hi, lo, cnt));
-        if (lane == 0) a.part[((int64_t)b * a.C + c) * a.slots + 1] = sum;
-      }
-      __syncthreads();
-    }
     m0 = partial(c0, 1);
     m1 = partial(c1, 1);
     S = block_sum_u64<kAcceptThreads>(m0 + m1, blk);
