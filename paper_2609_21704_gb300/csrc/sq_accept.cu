@@ -330,7 +330,7 @@ constexpr int kAcceptMaxCpc = 4;  // chunks of one CTA at most
 static_assert(kAcceptChunk == 8 * kAcceptThreads, "a thread owns 8 consecutive entries of a chunk");
 static_assert(kSoftmaxChunk == 8 * kAcceptThreads, "a thread owns 8 consecutive entries of a chunk");
 
-template <class Src>
+template <class Src, bool SAMPLE>
 __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Src src) {
   griddep_wait();
   griddep_launch_dependents();
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
     if (lane < K) {
       const int32_t x = xb[lane];
       bad = (x < 0 || (int64_t)x >= V);
-      if (!bad && !rows_mask && a.mode == SQ_ACCEPT_SAMPLE)
+      if (SAMPLE && !bad && !rows_mask)
         acc = (double)ub[lane] * (double)src.qrow(b, lane)(x) < (double)src.prow(b, lane)(x);
     }
     const float uk = ub[K];
@@ -380,80 +380,78 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
   const int n = s_n;
 
   // ---- chunk partials
-  if constexpr (Src::kUnit) {
-    if (a.mode == SQ_ACCEPT_SAMPLE) {
-      // all of the CTA's chunks at once: their loads, their sums, one barrier.
-      // The row's own mass is wanted only if the whole residual is zero: a warp
-      // sums its share where its residual is (slot 1 is complete then), in a loop
-      // of its own, since code that is rarely run costs the others their fetches.
-      const auto pn = src.prow(b, n);
-      const bool use_q = n < K;
-      const auto qn = src.qrow(b, use_q ? n : 0);
-      uint4 pr[kAcceptMaxCpc], qr[kAcceptMaxCpc];
-      uint32_t zero = 0;  // chunks without residual in this warp
+  if constexpr (Src::kUnit && SAMPLE) {
+    // all of the CTA's chunks at once: their loads, their sums, one barrier.
+    // The row's own mass is wanted only if the whole residual is zero: a warp
+    // sums its share where its residual is (slot 1 is complete then), in a loop
+    // of its own, since code that is rarely run costs the others their fetches.
+    const auto pn = src.prow(b, n);
+    const bool use_q = n < K;
+    const auto qn = src.qrow(b, use_q ? n : 0);
+    uint4 pr[kAcceptMaxCpc], qr[kAcceptMaxCpc];
+    uint32_t zero = 0;  // chunks without residual in this warp
 #pragma unroll
-      for (int i = 0; i < kAcceptMaxCpc; ++i) {
-        const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
-        if (cb + i < ce && v < V) {
-          pr[i] = pn.raw8(v, V);
-          if (use_q) qr[i] = qn.raw8(v, V);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < kAcceptMaxCpc; ++i) {
-        const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
-        unsigned long long sr = 0;
-        if (cb + i < ce && v < V) {
-          uint32_t hi = 0, lo = 0;
-          float pv[8], qv[8];
-          pn.sum8(pr[i], v, V, pv);
-          if (use_q) qn.sum8(qr[i], v, V, qv);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) add_fix44(use_q ? fmaxf(pv[j] - qv[j], 0.0f) : pv[j], hi, lo);
-          sr = fix44_total(hi, lo, 8);
-        }
-        sr = warp_sum_u64(sr);
-        if (sr == 0 && use_q) zero |= 1u << i;
-        if (lane == 0) {
-          red[warp][i] = sr;
-          red[warp][kAcceptMaxCpc + i] = 0;
-        }
-      }
-#pragma unroll 1
-      for (; zero != 0; zero &= zero - 1) {
-        const int i = __ffs(zero) - 1;
-        const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
-        unsigned long long sp = 0;
-        if (cb + i < ce && v < V) {
-          uint32_t hi = 0, lo = 0;
-          float pv[8];
-          pn.sum8(pn.raw8(v, V), v, V, pv);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) add_fix44(pv[j], hi, lo);
-          sp = fix44_total(hi, lo, 8);
-        }
-        sp = warp_sum_u64(sp);
-        if (lane == 0) red[warp][kAcceptMaxCpc + i] = sp;
-      }
-      __syncthreads();
-      if (tid < ce - cb) {
-        unsigned long long tr = 0, tp = 0;
-        for (int w = 0; w < kAcceptThreads / 32; ++w) {
-          tr += red[w][tid];
-          tp += red[w][kAcceptMaxCpc + tid];
-        }
-        unsigned long long* part = a.part + ((int64_t)b * a.C + cb + tid) * a.slots;
-        part[0] = tr;
-        part[1] = tp;
+    for (int i = 0; i < kAcceptMaxCpc; ++i) {
+      const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
+      if (cb + i < ce && v < V) {
+        pr[i] = pn.raw8(v, V);
+        if (use_q) qr[i] = qn.raw8(v, V);
       }
     }
+#pragma unroll
+    for (int i = 0; i < kAcceptMaxCpc; ++i) {
+      const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
+      unsigned long long sr = 0;
+      if (cb + i < ce && v < V) {
+        uint32_t hi = 0, lo = 0;
+        float pv[8], qv[8];
+        pn.sum8(pr[i], v, V, pv);
+        if (use_q) qn.sum8(qr[i], v, V, qv);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) add_fix44(use_q ? fmaxf(pv[j] - qv[j], 0.0f) : pv[j], hi, lo);
+        sr = fix44_total(hi, lo, 8);
+      }
+      sr = warp_sum_u64(sr);
+      if (sr == 0 && use_q) zero |= 1u << i;
+      if (lane == 0) {
+        red[warp][i] = sr;
+        red[warp][kAcceptMaxCpc + i] = 0;
+      }
+    }
+#pragma unroll 1
+    for (; zero != 0; zero &= zero - 1) {
+      const int i = __ffs(zero) - 1;
+      const int64_t v = ((int64_t)(cb + i) * kAcceptThreads + tid) * 8;
+      unsigned long long sp = 0;
+      if (cb + i < ce && v < V) {
+        uint32_t hi = 0, lo = 0;
+        float pv[8];
+        pn.sum8(pn.raw8(v, V), v, V, pv);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) add_fix44(pv[j], hi, lo);
+        sp = fix44_total(hi, lo, 8);
+      }
+      sp = warp_sum_u64(sp);
+      if (lane == 0) red[warp][kAcceptMaxCpc + i] = sp;
+    }
+    __syncthreads();
+    if (tid < ce - cb) {
+      unsigned long long tr = 0, tp = 0;
+      for (int w = 0; w < kAcceptThreads / 32; ++w) {
+        tr += red[w][tid];
+        tp += red[w][kAcceptMaxCpc + tid];
+      }
+      unsigned long long* part = a.part + ((int64_t)b * a.C + cb + tid) * a.slots;
+      part[0] = tr;
+      part[1] = tp;
+    }
   }
-  for (int c = cb; c < ce && !(Src::kUnit && a.mode == SQ_ACCEPT_SAMPLE); ++c) {
+  for (int c = cb; c < ce && !(Src::kUnit && SAMPLE); ++c) {
     const int64_t v0 = (int64_t)c * a.chunk;
     const int64_t v1 = v0 + a.chunk < V ? v0 + a.chunk : V;
     const int64_t vb = v0 + 8 * (int64_t)tid;  // thread t: the 8 entries [v0 + 8t, v0 + 8t + 8)
     unsigned long long* part = a.part + ((int64_t)b * a.C + c) * a.slots;
-    if (a.mode == SQ_ACCEPT_SAMPLE) {
+    if constexpr (SAMPLE) {
       const auto pn = src.prow(b, n);
       const bool use_q = n < K;
       const auto qn = src.qrow(b, use_q ? n : 0);
@@ -536,7 +534,7 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, Sr
     return cc < a.C ? __ldcg(pall + (int64_t)cc * a.slots + slot) : 0ull;
   };
 
-  if (a.mode == SQ_ACCEPT_GREEDY) {
+  if constexpr (!SAMPLE) {
     for (int i = 0; i <= K; ++i) {
       const unsigned long long k0 = partial(c0, i), k1 = partial(c1, i);
       const unsigned long long best = block_max_u64<kAcceptThreads>(k0 > k1 ? k0 : k1, blk);
@@ -681,7 +679,8 @@ cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t st) {
   AcceptArgs b = a;
   b.cpc = accept_chunks_per_cta(a, false);
   ProbSrc src{a.p, a.q, a.K, a.V};
-  return launch_pdl(accept_kernel<ProbSrc>, dim3((unsigned)(a.B * ((a.C + b.cpc - 1) / b.cpc))),
+  return launch_pdl(a.mode == SQ_ACCEPT_SAMPLE ? accept_kernel<ProbSrc, true> : accept_kernel<ProbSrc, false>,
+                    dim3((unsigned)(a.B * ((a.C + b.cpc - 1) / b.cpc))),
                     dim3(kAcceptThreads), 0, st, b, src);
 }
 
@@ -910,7 +909,8 @@ cudaError_t launch_accept_logits(const AcceptArgs& a, const SoftmaxArgs& sa, cud
   LogitSrc src{sa.zp, sa.zq, sa.m, sa.s, sa.invT, a.B, a.K, a.V};
   AcceptArgs b = a;
   b.cpc = accept_chunks_per_cta(a, a.mode == SQ_ACCEPT_SAMPLE);
-  return launch_pdl(accept_kernel<LogitSrc>, dim3((unsigned)(a.B * ((a.C + b.cpc - 1) / b.cpc))),
+  return launch_pdl(a.mode == SQ_ACCEPT_SAMPLE ? accept_kernel<LogitSrc, true> : accept_kernel<LogitSrc, false>,
+                    dim3((unsigned)(a.B * ((a.C + b.cpc - 1) / b.cpc))),
                     dim3(kAcceptThreads), 0, st, b, src);
 }
 
