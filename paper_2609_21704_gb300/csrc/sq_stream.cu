@@ -15,7 +15,8 @@
 // the first ones before the wait on the kernel that produces x.  Up to eight
 // rows a CTA keeps to 80 registers a thread and, where it has little to
 // stream, to half the shared memory: the next launch's CTA fits beside it and
-// its first copies run while this one computes.
+// its first copies run while this one computes.  A call with much to stream
+// takes more than half, so that none does.
 //
 // Products: A = sixteen weight rows, B = the activation rows as columns (eight
 // a tile; columns past M repeat a row and are dropped).  FP16 pieces are

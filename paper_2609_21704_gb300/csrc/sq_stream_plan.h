@@ -115,9 +115,14 @@ inline int s_split(int wkind, bool silu, int nw, int clusters, StreamPlan& a, do
   // of activations a nanosecond (every CTA reads the same lines), a cluster's
   // launch and its two barriers, one more for every further pass.
   static const double kCluster[9] = {0, 0, 1500, 0, 2500, 0, 0, 0, 6000};
-  *ns = best * wr * 330.0 * (a.KS > 1 ? 1.1 : a.ns == 3 && !little ? 1.15 : 1.0) + 2.0 * a.M * a.K / a.KS / 25.0 + kCluster[a.KS] +
+  *ns = best * wr * 330.0 * (a.KS > 1 ? 1.1 : a.ns == 3 && !little ? 1.15 : 1.0) +
+        2.0 * a.M * a.K / a.KS / 25.0 + kCluster[a.KS] +
         (a.KS > 1 ? 2000.0 * (double)((tiles + pt - 1) / pt - 1) : 0.0);
-  return a.off_ring + a.ns * nw * kSlotBytes;
+  // A call with much to stream takes more than half: another CTA on its SM would
+  // slow the one that the call ends with (1.5B FP16 at three rows, whose gate/up
+  // just fits in half: a pass of 28 layers and lm_head 830 us, so 797).
+  const int smem = a.off_ring + a.ns * nw * kSlotBytes;
+  return !little && smem <= kSmemHalf ? kSmemHalf + 1024 : smem;
 }
 
 }  // namespace sq

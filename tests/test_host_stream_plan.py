@@ -1,7 +1,8 @@
 """The streaming engine's host arithmetic (csrc/sq_stream_plan.h), compiled for
 the CPU and checked over sizes and cluster counts: a kernel never gets a split
 with which its loops stand still, every part of K holds a unit in every CTA of a
-cluster, the layout stays inside the shared memory, and the estimate by which a
+cluster, the layout stays inside the shared memory (above half of it where a call
+streams much), and the estimate by which a
 split is chosen covers all of its passes."""
 import os
 import subprocess
@@ -89,6 +90,9 @@ static void check(int wk, bool silu, int M, int64_t N, int K, int ks, int cluste
     die("partial sums past their buffer", wk, silu, a, clusters);
   if (a.off_red + (int64_t)bufs * a.red_floats * 4 > a.off_ring) die("overlap", wk, silu, a, clusters);
   if (a.ns < 3 || a.off_ring + a.ns * nw * kSlotBytes > smem || smem > kSmemMax) die("shared memory", wk, silu, a, clusters);
+  // with much to stream no second CTA shares the SM
+  if ((N + clusters - 1) / clusters * (silu ? 2 : 1) * a.row_bytes / ks > 96 * 1024 && smem <= kSmemHalf)
+    die("two CTAs an SM", wk, silu, a, clusters);
 }
 
 int main() {
