@@ -215,11 +215,12 @@ bool use_ring(int wkind, int M, int64_t N, int64_t K, int epi) {
 //     8 rows 21.8 -> 14.7): from 8 Mi weights on, or, at six and seven rows, where the
 //     alternative is the GEMV, any (896 x 4864 10.3 -> 6.4).  Its lm_head of >= 400
 //     Mi takes two rows only (14B 383 -> 254; at five 251 against 257).
-//   FP16, gated: from 64 Mi weights on at two rows (7B pass 1031 -> 917; 1.5B, 26 Mi,
-//     832 against 881); small ones at six and seven rows (GEMV: 1024 x 4096 15.0 ->
-//     7.5); short rows below 32 Mi at three to six (1.5B pass at five rows 864 -> 828,
-//     but at eight 851 against 882) and few long rows (512 x 16384 at three 14.1 ->
-//     10.7); the tile path has the rest (16384 x 1024 at three 13.0 against 14.7).
+//   FP16, gated: from 16 Mi weights on at two rows (7B pass 829 -> 716; 1.5B, 26 Mi,
+//     757 -> 690); small ones at six and seven rows (GEMV: 1024 x 4096 15.0 -> 7.5);
+//     short rows below 32 Mi at three to six (1.5B pass at three rows 727 -> 711, at
+//     five 753 -> 732; at six 754 against 771 between linear calls alone, but 1610 ->
+//     1579 in a decoder pass) and few long rows (512 x 16384 at three 14.1 -> 10.7);
+//     the tile path has the rest (7B pass at three rows 636 against 654).
 bool use_stream(int wkind, int M, int64_t N, int64_t K, int epi) {
   if (!stream_supported(wkind, M, N, K, epi)) return false;
   const bool silu = epi == SQ_EPI_SILU_GATE;
@@ -232,7 +233,7 @@ bool use_stream(int wkind, int M, int64_t N, int64_t K, int epi) {
     if (M > 8) return false;
     if (head) return weights < 400 * Mi ? M >= 3 : M == 2;
     if (silu) {
-      if (M == 2) return weights >= 64 * Mi;
+      if (M == 2) return weights >= 16 * Mi;
       if (weights < 16 * Mi) return M == 6 || M == 7 || (M == 8 && K <= 2048);
       return (M <= 6 && K <= 2048 && weights < 32 * Mi) || tiles <= 8;
     }

@@ -160,7 +160,8 @@ def test_single_row_engine_choice(lib):
     assert sq.sq_linear_path(W16, 5, 5120, 5120, RES) == 4      # 14B o
     assert sq.sq_linear_path(W16, 6, 896, 4864, NONE) == 4      # six rows: any size below K = 8192
     assert sq.sq_linear_path(W16, 2, 13824, 5120, SILU) == 4    # 14B fused gate/up at two rows
-    assert sq.sq_linear_path(W16, 2, 8960, 1536, SILU) == 0     # the 1.5B one (27.5 Mi)
+    assert sq.sq_linear_path(W16, 2, 8960, 1536, SILU) == 4     # the 1.5B one (26 Mi)
+    assert sq.sq_linear_path(W16, 2, 2048, 3072, SILU) == 0     # below 16 Mi
     assert sq.sq_linear_path(W8, 1, 151936, 1536, NONE) == 0    # 1.5B FP8 lm_head (233 Mi)
     assert sq.sq_linear_path(W8, 1, 152064, 5120, NONE) == 3    # 14B FP8 lm_head (779 Mi)
     assert sq.sq_linear_path(W8, 1, 13824, 5120, SILU) == 0
